@@ -362,6 +362,16 @@ LBM_API int lbm_exact_moments_host(const double* d, int64_t n, double* out);
 LBM_API int lbm_fx_pairs_host(const double* d, const double* terms, int64_t n, double qm, double qp, int flags,
                               double* out, int* ok);
 
+/* Host image of the whole LBM_F64 collision in fixed point (moments, class
+ * terms and pair update), run on the host.  d: host double [n][19], the PDFs of
+ * n nodes as params' storage holds them (deviations when params.shifted); s:
+ * host float [n], Brinkman solid fractions, or NULL.  out: host double [n][19],
+ * the post-collision PDFs in the same storage; ok: host int [n], 0 where the
+ * node is outside the fixed-point range (out is then 0; the kernels take the
+ * FP64 update there).  LBM_ERR_ARG for bad params, NULL pointers or n < 0. */
+LBM_API int lbm_fx_collide_host(const double* d, const float* s, int64_t n, const lbm_params* params, double* out,
+                                int* ok);
+
 /* Check the host tables: entries in range, adjacency reciprocity
  * (adj[i][n] = m >= 0  <=>  adj[inv i][m] = n), run table decoding back to the
  * adjacency list exactly, runs sorted and covering [0, N).  Returns

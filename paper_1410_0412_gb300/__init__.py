@@ -597,6 +597,29 @@ def lbm_fx_pairs_host(d, terms, qm, qp, lp1, general=False):
     return out, ok.astype(bool)
 
 
+def lbm_fx_collide_host(d, params, s=None):
+    """Host image of the whole FP64 collision in fixed point (``lbm_fx_collide_host``).
+
+    d: [n, 19] PDFs in the storage of ``params`` (deviations when shifted); s:
+    [n] Brinkman solid fractions or None.  Returns (out [n, 19], ok [n]).
+    """
+    import numpy as np
+    a = np.ascontiguousarray(np.asarray(d, dtype=np.float64))
+    if a.ndim != 2 or a.shape[1] != 19:
+        raise ValueError("d must have shape [n, 19]")
+    sf = None
+    if s is not None:
+        sf = np.ascontiguousarray(np.asarray(s, dtype=np.float32))
+        if sf.shape != (a.shape[0],):
+            raise ValueError("s must have shape [n]")
+    out = np.empty((a.shape[0], 19), dtype=np.float64)
+    ok = np.empty(a.shape[0], dtype=np.int32)
+    check(_lib.load().lbm_fx_collide_host(a.ctypes.data, None if sf is None else sf.ctypes.data, a.shape[0],
+                                          ctypes.byref(params.c()), out.ctypes.data, ok.ctypes.data),
+          "lbm_fx_collide_host")
+    return out, ok.astype(bool)
+
+
 def lbm_bandwidth_kernel(kind, dst, src=None, arrays=1, stream=None):
     """One launch of the CNT-kA (kind 0, copy src -> dst with streaming stores) or
     U-kA (kind 1, update dst in place) bandwidth kernel over ``arrays`` equal
@@ -852,7 +875,7 @@ __all__ = [
     "PartitionedSolver", "lbm_halo_exchange", "lbm_partition_run_aa", "lbm_partition_run_osnt",
     "lbm_objective_flux", "lbm_adjoint_step", "lbm_ckpt_workspace_bytes", "lbm_flux_forward", "lbm_flux_backward",
     "flux_objective", "new_adjoint", "lbm_macroscopic_noalloc", "lbm_check_finite", "lbm_bandwidth_kernel", "lbm_fp64_peak_kernel",
-    "lbm_exact_moments_host", "lbm_fx_pairs_host",
+    "lbm_exact_moments_host", "lbm_fx_pairs_host", "lbm_fx_collide_host",
     "State", "FluxObjective",
 ]
 

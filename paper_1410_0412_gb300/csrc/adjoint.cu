@@ -299,8 +299,8 @@ __global__ void __launch_bounds__(kBlock) k_adjoint(DevTables t, KParams kp, Col
                          : k == 6 ? Bxf + Bzf : k == 7 ? Bxf - Bzf : k == 8 ? Byf + Bzf : Byf - Bzf;
         const int64_t Df = static_cast<int64_t>(static_cast<uint64_t>(Di[k]) << kxa);
         int64_t e = Af;
-        if (!LP1) e += mulhi_q64(cc.qp_fx, static_cast<int64_t>(static_cast<uint64_t>(Pi[k]) << kxa));
-        const int64_t o = mulhi_q64(cc.qm_fx, Df) + Bc;
+        if (!LP1) e += mulhi_q64(cc.fx.qp, static_cast<int64_t>(static_cast<uint64_t>(Pi[k]) << kxa));
+        const int64_t o = mulhi_q64(cc.fx.qm, Df) + Bc;
         L::st(lam + at(a, t.npad, n), fx_to_double(e + o, es));
         L::st(lam + at(a + 1, t.npad, n), fx_to_double(e - o, es));
       }

@@ -385,13 +385,57 @@ int lbm_fx_pairs_host(const double* d, const double* terms, int64_t n, double qm
     const int kx = lp1 ? 4 : 2;
     const dev::FxClass q = dev::fx_class(emax - kx, t[0], t[1], t[2], t[3], t[4], t[5], t[6], t[7], t[8], t[9]);
     if (lp1)
-      general ? dev::fx_pairs<true, 4, true>(q, D, Sk, qm_fx, qp_fx, emax - kx, p)
-              : dev::fx_pairs<true, 4>(q, D, Sk, qm_fx, qp_fx, emax - kx, p);
+      general ? dev::fx_pairs<true, true>(q, D, Sk, qm_fx, qp_fx, emax - kx, kx, p)
+              : dev::fx_pairs<true>(q, D, Sk, qm_fx, qp_fx, emax - kx, kx, p);
     else
-      general ? dev::fx_pairs<false, 2, true>(q, D, Sk, qm_fx, qp_fx, emax - kx, p)
-              : dev::fx_pairs<false, 2>(q, D, Sk, qm_fx, qp_fx, emax - kx, p);
+      general ? dev::fx_pairs<false, true>(q, D, Sk, qm_fx, qp_fx, emax - kx, kx, p)
+              : dev::fx_pairs<false>(q, D, Sk, qm_fx, qp_fx, emax - kx, kx, p);
     o[0] = static_cast<double>(emax - kx);  // the pair scale es: units of 2^(es - 1080)
     for (int i = 1; i < 19; ++i) o[i] = p[i];
+  }
+  return LBM_OK;
+}
+
+}  // extern "C"
+
+namespace {
+
+template <bool FORCE, bool DRAG, bool LP1>
+int fx_collide_node(const dev::FxColl& c, double (&f)[19], double s) {
+  int64_t Sk[10], D[10], S, Jx, Jy, Jz, f0;
+  int emax_fast;
+  const bool near = dev::fx_pos_near(f, emax_fast);
+  const int emax = near ? dev::fx_moments<true, true>(f, Sk, D, S, Jx, Jy, Jz, emax_fast, &f0)
+                        : dev::fx_moments<true>(f, Sk, D, S, Jx, Jy, Jz, 0, &f0, c.emin);
+  const int kx = dev::fx_kx<LP1>(c, near);
+  dev::FxClass q;
+  if (!dev::fx_class_int<FORCE, DRAG, LP1>(c, emax, kx, S, Jx, Jy, Jz, s, q)) return 0;
+  dev::fx_update<LP1>(c, q, emax, kx, D, Sk, f0, f);
+  return 1;
+}
+
+}  // namespace
+
+extern "C" {
+
+int lbm_fx_collide_host(const double* d, const float* s, int64_t n, const lbm_params* params, double* out, int* ok) {
+  KParams kp;
+  if (int rc = make_kparams(params, LBM_F64, &kp)) return rc;
+  if (n < 0 || (n > 0 && (!d || !out || !ok))) return set_error(LBM_ERR_ARG, "d, out or ok is NULL, or n < 0");
+  const dev::FxColl c = dev::make_fx_coll(kp.lp, kp.lm, kp.g, kp.rho_s);
+  const bool force = kp.g[0] != 0.0 || kp.g[1] != 0.0 || kp.g[2] != 0.0, lp1 = kp.lp == 1.0;
+  for (int64_t k = 0; k < n; ++k) {
+    double f[19];
+    std::memcpy(f, d + 19 * k, sizeof f);
+    const double sn = s ? double(s[k]) : 0.0;
+    if (s)
+      ok[k] = lp1 ? fx_collide_node<true, true, true>(c, f, sn) : fx_collide_node<true, true, false>(c, f, sn);
+    else if (force)
+      ok[k] = lp1 ? fx_collide_node<true, false, true>(c, f, sn) : fx_collide_node<true, false, false>(c, f, sn);
+    else
+      ok[k] = lp1 ? fx_collide_node<false, false, true>(c, f, sn) : fx_collide_node<false, false, false>(c, f, sn);
+    if (!ok[k]) std::memset(f, 0, sizeof f);
+    std::memcpy(out + 19 * k, f, sizeof f);
   }
   return LBM_OK;
 }

@@ -1,21 +1,28 @@
 // Integer-pipe arithmetic for the FP64 collision.
 //
 // GB300 executes FP64 arithmetic on two lanes per SM per clock, against 64
-// integer and 128 FP32 lanes, so the native FP64 step is bound by its FP64
-// instruction count while the other pipes idle.  Two pieces of the collision
-// are exact in integer arithmetic and move there:
+// integer and 128 FMA lanes, so an FP64 step written in FP64 instructions is
+// bound by them while the other pipes idle.  The collision runs in 64-bit fixed
+// point instead:
 //
 //  * the moments that the TRT collision (Sect. 2) starts from, the density
 //    and momentum sums and the pair sums and differences: the 19 PDFs of a
 //    node are converted to 64-bit fixed point with a per-node scale (the largest
-//    exponent among them, with 5 bits of headroom), summed exactly, and each
-//    sum is rounded once to the nearest double.  A PDF at most 5 binades below
-//    the node's largest converts exactly; smaller ones lose bits below 2^-57
-//    of the largest.  A moment's error is at most 19 * 2^-57 * max|f_i| plus
+//    exponent among them, with 5 bits of headroom) and summed exactly.  A PDF
+//    at most 5 binades below the node's largest converts exactly; smaller ones
+//    lose bits below 2^-57 of the largest.  Rounded once to the nearest double
+//    (exact_moments), a moment's error is at most 19 * 2^-57 * max|f_i| plus
 //    half an ulp of the result, below the error bound (n - 1) * 2^-53 * sum|f_i|
 //    of the IEEE double sum of n terms that it replaces;
-//  * halving: an exponent decrement, identical to 0.5 * x for every x whose
-//    half is a normal number, Inf or NaN.
+//  * the class terms and the pair update (FxClass, fx_class_int, fx_pairs),
+//    rounded once per output;
+//  * halving, where the FP64 update remains: an exponent decrement, identical
+//    to 0.5 * x for every x whose half is a normal number, Inf or NaN.
+//
+// On the 256^3 bed (10.9 M nodes) the FP64 AA-R step pair went from 1.61 ms,
+// with the class terms in FP64 (31 FP64 instructions a node), to 1.23 ms; the
+// even step moves its bytes at 0.96 of the measured copy rate (ncu: DRAM 78 %,
+// integer pipe 66 %, FP64 pipe 71 %).
 //
 // All functions are __host__ __device__ so that a host test can check the
 // moments bit for bit against exact rational arithmetic.
@@ -144,43 +151,31 @@ __host__ __device__ __forceinline__ int64_t fx_of_pos_near(uint64_t b, unsigned 
   return static_cast<int64_t>((static_cast<uint64_t>(shf_l(lo, mh, k)) << 32) | (lo << k));
 }
 
-// fx_to_double for the common case, in 32-bit halves: 2^32 <= v < 2^63 (the
-// high word is a positive int32).  Same bits as fx_to_double.
-__host__ __device__ __forceinline__ double fx_to_double_pos(int64_t v, int emax) {
-  const uint32_t hi = static_cast<uint32_t>(static_cast<uint64_t>(v) >> 32), lo = static_cast<uint32_t>(v);
-  const int lz = clz32(hi);                                // 1..31
-  const uint32_t ah = shf_l(lo, hi, lz), al = lo << lz;    // leading one at bit 63
-  const uint32_t mh = ah >> 11, ml = shf_r(al, ah, 11);    // 53 significant bits
-  // round to nearest, ties to even: the 11 bits below plus 0x3ff plus the
-  // last kept bit reach 2^11 exactly when rounding up
-  const uint32_t up = ((al & 0x7ffu) + 0x3ffu + (ml & 1u)) >> 11;
-  const uint64_t m = ((static_cast<uint64_t>(mh) << 32) | ml) + up;  // may carry to 2^53: exponent + 1
-  return dfrom((static_cast<uint64_t>(emax + 5 - lz) << 52) + m);
-}
-
-// True when fx_to_double_pos applies to v.
-__host__ __device__ __forceinline__ bool fx_pos_wide(int64_t v) { return (v >> 32) >= 1; }
-
 // fx_to_double through the hardware's int64 -> double conversion (round to
 // nearest, ties to even: the same rounding, so the same bits), then an exact
-// scaling by 2^(emax - 1080) as an exponent-field add.  The conversion runs
-// on the FP64 pipe, the rest on the integer pipe; the kernels use it for part
-// of the outputs to balance the two.  For kFxMinExp - 4 <= emax < kFxMaxExp
-// every non-zero result is a normal number.
+// scaling by 2^(emax - 1080) as an exponent-field add.  The conversion is one
+// instruction of the FP64 pipe, which has nothing else to do in the fixed-point
+// collision (19 conversions a node keep it 60-70 % busy), and takes about 12
+// instructions off the integer pipe, the busier one: with 9 / 7 / 5 of the
+// pairs converted this way the FP64 AA-R pair on the 256^3 bed took 1.36 /
+// 1.38 / 1.48 ms.  For kFxMinExp - 4 <= emax < kFxMaxExp every non-zero result
+// is a normal number.
 __host__ __device__ __forceinline__ double fx_to_double_cvt(int64_t v, int emax) {
 #ifdef __CUDA_ARCH__
   const double x = __ll2double_rn(static_cast<long long>(v));
 #else
   const double x = static_cast<double>(v);
 #endif
-  const uint64_t scaled = dbits(x) + (static_cast<uint64_t>(static_cast<int64_t>(emax - 1080)) << 52);
-  return v == 0 ? 0.0 : dfrom(scaled);
+  const uint64_t b = dbits(x);
+  const uint32_t hi = static_cast<uint32_t>(b >> 32);
+  const uint32_t scaled = hi ? hi + (static_cast<uint32_t>(emax - 1080) << 20) : 0u;
+  return dfrom((static_cast<uint64_t>(scaled) << 32) | static_cast<uint32_t>(b));
 }
 
-// Node scale of the 19 PDFs: the largest biased exponent, at least kFxMinExp.
+// Node scale of the 19 PDFs: the largest biased exponent, at least emin (>= kFxMinExp).
 template <int Q>
-__host__ __device__ __forceinline__ int fx_scale(const uint64_t (&b)[Q]) {
-  int emax = kFxMinExp;
+__host__ __device__ __forceinline__ int fx_scale(const uint64_t (&b)[Q], int emin = kFxMinExp) {
+  int emax = emin;
 #pragma unroll
   for (int i = 0; i < Q; ++i) {
     const int e = static_cast<int>(b[i] >> 52) & 0x7ff;
@@ -201,7 +196,8 @@ __host__ __device__ __forceinline__ int fx_scale(const uint64_t (&b)[Q]) {
 template <bool NEED_SA, bool FAST = false>
 __host__ __device__ __forceinline__ int fx_moments(const double (&d)[19], int64_t (&Sk)[10], int64_t (&D)[10],
                                                    int64_t& S, int64_t& Jx, int64_t& Jy, int64_t& Jz,
-                                                   int emax_fast = 0) {
+                                                   int emax_fast = 0, int64_t* f0 = nullptr,
+                                                   int emin = kFxMinExp) {
   uint64_t b[19];
 #pragma unroll
   for (int i = 0; i < 19; ++i) b[i] = dbits(d[i]);
@@ -213,11 +209,12 @@ __host__ __device__ __forceinline__ int fx_moments(const double (&d)[19], int64_
 #pragma unroll
     for (int i = 0; i < 19; ++i) f[i] = fx_of_pos_near(b[i], static_cast<unsigned>(static_cast<int>(b[i] >> 52) + 5 - emax));
   } else {
-    emax = fx_scale(b);
+    emax = fx_scale(b, emin);
 #pragma unroll
     for (int i = 0; i < 19; ++i) f[i] = fx_of(b[i], emax);
   }
   S = f[0];
+  if (f0) *f0 = f[0];
 #pragma unroll
   for (int k = 1; k <= 9; ++k) {
     const int64_t s = f[2 * k - 1] + f[2 * k];
@@ -236,18 +233,17 @@ __host__ __device__ __forceinline__ int fx_moments(const double (&d)[19], int64_
 // largest (so fx_of_pos_near's shift stays in [0, 5]; PDFs near w_i rho span
 // 4).  emax: the node scale (the largest exponent field; meaningful when true).
 __host__ __device__ __forceinline__ bool fx_pos_near(const double (&d)[19], int& emax) {
-  uint32_t sgn = 0;
-  int emin = 2047;
-  emax = 0;
+  // positive doubles order like their high words, and one negative high word
+  // makes the minimum negative: a min and a max per PDF decide
+  int32_t mn = 0x7fffffff, mx = 0;
 #pragma unroll
   for (int i = 0; i < 19; ++i) {
-    const uint32_t hi = static_cast<uint32_t>(dbits(d[i]) >> 32);
-    sgn |= hi;
-    const int e = static_cast<int>(hi >> 20);
-    emax = e > emax ? e : emax;
-    emin = e < emin ? e : emin;
+    const int32_t hi = static_cast<int32_t>(dbits(d[i]) >> 32);
+    mn = hi < mn ? hi : mn;
+    mx = hi > mx ? hi : mx;
   }
-  return !(sgn & 0x80000000u) && emin >= kFxMinExp && emax < kFxMaxExp && emax - emin <= 5;
+  emax = mx >> 20;
+  return (mn >> 20) >= kFxMinExp && emax < kFxMaxExp && emax - (mn >> 20) <= 5;
 }
 
 // The moments as doubles: pair sums sa_k (only when NEED_SA) and differences
@@ -270,15 +266,29 @@ __host__ __device__ __forceinline__ void exact_moments(const double (&d)[19], do
   jz = fx_to_double(Jz, emax);
 }
 
-// floor(a * b / 2^64) for signed 64-bit a, b: the product of a Q64 fraction
-// (|a| < 2^63, the value a / 2^64) with a fixed-point value, at the latter's scale.
-__host__ __device__ __forceinline__ int64_t mulhi_q64(int64_t a, int64_t b) {
-#ifdef __CUDA_ARCH__
-  return __mul64hi(a, b);
-#else
-  return static_cast<int64_t>((static_cast<__int128>(a) * b) >> 64);
-#endif
+// a * b / 2^64 for signed 64-bit a, b, within 3/4 of a unit (unbiased): the
+// product of a Q64 fraction (|a| < 2^63, the value a / 2^64) with a fixed-point
+// value, at the latter's scale.  Both factors are split in balanced halves
+// (a = ah 2^32 + al with al a signed 32-bit word), so every partial product is
+// one signed 32 x 32 -> 64 multiply-add on the FMA pipe, and the product of
+// the low words, at most a quarter of a unit, is left out: three multiply-adds
+// and about four ALU instructions, where the exact high word of a signed
+// 64 x 64 product takes about 14.  Both factors must stay below 2^63 - 2^31
+// in magnitude (the high halves round up) and one of them below 2^62 (the
+// middle sum).
+struct Bal {
+  int32_t h, l;
+};
+__host__ __device__ __forceinline__ Bal bal(int64_t v) {
+  const int32_t l = static_cast<int32_t>(v);
+  return Bal{static_cast<int32_t>(v >> 32) + static_cast<int32_t>(static_cast<uint32_t>(l) >> 31), l};
 }
+__host__ __device__ __forceinline__ int64_t mulhi_q64(Bal a, Bal b) {
+  int64_t m = static_cast<int64_t>(a.h) * b.l + 0x80000000ll;
+  m += static_cast<int64_t>(b.h) * a.l;
+  return static_cast<int64_t>(a.h) * b.h + (m >> 32);
+}
+__host__ __device__ __forceinline__ int64_t mulhi_q64(int64_t a, int64_t b) { return mulhi_q64(bal(a), bal(b)); }
 
 // Biased exponent field of a double.
 __host__ __device__ __forceinline__ int dexp(double x) { return static_cast<int>(dbits(x) >> 52) & 0x7ff; }
@@ -289,24 +299,42 @@ __host__ __device__ __forceinline__ int dexp(double x) { return static_cast<int>
 // of the axis class (the diagonal class uses them halved) -- and the exact
 // pair sums Sk and differences Dk, the post-collision pair is
 //   e = K0 + (c.u)(c.T) [+ qp Sk],  o = qm Dk + c.O,  p_a = e + o,  p_b = e - o,
-// with qm = (1 - l-)/2 and qp = (1 - l+)/2 as Q64 fractions.  The pair stage
+// with qm = (1 - l-)/2 and qp = (1 - l+)/2 as Q64 fractions.  The nine even
+// products share six: (c.u)(c.T) is A_a = u_a T_a for an axis pair and
+// A_a + A_b +- C_ab, C_ab = u_a T_b + u_b T_a, for a diagonal one.  The class
+// values are held halved, as the six diagonal pairs use them.  The pair stage
 // works at a scale kx bits finer than the moments, 2^(es - 1080) with
-// es = emax - kx (kx = 4 when qp = 0, else 2): Dk and Sk enter shifted left by
-// kx, exactly.  Every sum is exact; the products (c.u)(c.T), qm Dk and qp Sk
-// are truncated to the scale (floor), and so are u, K0, T and O when they
-// enter.  The error of p before its one rounding to double is below 8 units
-// of 2^(es - 1080), i.e. below 2^-(54 + kx) of B = 2^(emax - 1023), the
-// binade of the node's largest PDF (for PDFs near w_i rho, below a quarter of
-// an ulp of the smallest, the diagonal ones, when kx = 4).
+// es = emax - kx: Dk and Sk enter multiplied by 2^kx, exactly.  Every sum is
+// exact; products are within 3/4 of a unit.  From class values given as
+// doubles (fx_class, each truncated to the scale) the error of p before its
+// one rounding to double is below 8 units of 2^(es - 1080), i.e. below
+// 2^-(54 + kx) of B = 2^(emax - 1023), the binade of the node's largest PDF
+// (for PDFs near w_i rho, below a quarter of an ulp of the smallest, the
+// diagonal ones, when kx = 4).
 //
-// Valid when |u_a| < 1/4 (biased exponent <= 1020), |K0| < B/2 (exponent
-// <= emax - 2) and |T_a|, |O_a| < B/4 (exponent <= emax - 3); with every
-// |d_i| < 2B this keeps |c.u| < 1/2 and every intermediate below 2^63 at
-// either kx.  fx_class_ok checks it.
+// For class values given as doubles the host image takes kx = 4 when l+ = 1,
+// else 2; valid when |u_a| < 1/4 (biased exponent <= 1020), |K0| < B/2
+// (exponent <= emax - 2) and |T_a|, |O_a| < B/4 (exponent <= emax - 3), which
+// with every |d_i| < 2B keeps every intermediate below 2^63.  fx_class_ok
+// checks it.
 struct FxClass {
-  int64_t ux, uy, uz;  // Q64
-  int64_t K0, Tx, Ty, Tz, Ox, Oy, Oz;
+  int64_t K0;                 // even constant of the axis class
+  int64_t Ax, Ay, Az;         // u_a T_a / 2
+  int64_t Cxy, Cxz, Cyz;      // (u_a T_b + u_b T_a) / 2
+  int64_t Ox, Oy, Oz;         // O_a / 2
 };
+
+// The even products from u (Q64) and T / 2.
+__host__ __device__ __forceinline__ void fx_even(FxClass& q, int64_t ux, int64_t uy, int64_t uz, int64_t Tx, int64_t Ty,
+                                                 int64_t Tz) {
+  const Bal bx = bal(ux), by = bal(uy), bz = bal(uz), tx = bal(Tx), ty = bal(Ty), tz = bal(Tz);
+  q.Ax = mulhi_q64(bx, tx);
+  q.Ay = mulhi_q64(by, ty);
+  q.Az = mulhi_q64(bz, tz);
+  q.Cxy = mulhi_q64(bx, ty) + mulhi_q64(by, tx);
+  q.Cxz = mulhi_q64(bx, tz) + mulhi_q64(bz, tx);
+  q.Cyz = mulhi_q64(by, tz) + mulhi_q64(bz, ty);
+}
 
 __host__ __device__ __forceinline__ bool fx_class_ok(int emax, double ux, double uy, double uz, double K0, double Tx,
                                                      double Ty, double Tz, double Ox, double Oy, double Oz) {
@@ -320,102 +348,289 @@ __host__ __device__ __forceinline__ bool fx_class_ok(int emax, double ux, double
   return emax < kFxMaxExp && eu <= 1020 && dexp(K0) <= emax - 2 && eto <= emax - 3;
 }
 
-// The class values at the pair scale es (see above).
+// The class values at the pair scale es from doubles (see above).
 __host__ __device__ __forceinline__ FxClass fx_class(int es, double ux, double uy, double uz, double K0, double Tx,
                                                      double Ty, double Tz, double Ox, double Oy, double Oz) {
   FxClass q;
-  q.ux = fx_of(dbits(ux), 1016);  // u * 2^64
-  q.uy = fx_of(dbits(uy), 1016);
-  q.uz = fx_of(dbits(uz), 1016);
   q.K0 = fx_of(dbits(K0), es);
-  q.Tx = fx_of(dbits(Tx), es);
-  q.Ty = fx_of(dbits(Ty), es);
-  q.Tz = fx_of(dbits(Tz), es);
-  q.Ox = fx_of(dbits(Ox), es);
-  q.Oy = fx_of(dbits(Oy), es);
-  q.Oz = fx_of(dbits(Oz), es);
+  fx_even(q, fx_of(dbits(ux), 1016), fx_of(dbits(uy), 1016), fx_of(dbits(uz), 1016),  // u * 2^64
+          fx_of(dbits(Tx), es + 1), fx_of(dbits(Ty), es + 1), fx_of(dbits(Tz), es + 1));
+  q.Ox = fx_of(dbits(Ox), es + 1);
+  q.Oy = fx_of(dbits(Oy), es + 1);
+  q.Oz = fx_of(dbits(Oz), es + 1);
   return q;
 }
 
-// c . v for a direction with components X, Y, Z in {-1, 0, 1} (exact integer sums).
-template <int X, int Y, int Z>
-__host__ __device__ __forceinline__ int64_t fx_cdot(int64_t vx, int64_t vy, int64_t vz) {
-  int64_t acc = 0;
-  if (X) acc = X > 0 ? vx : -vx;
-  if (Y) acc = X ? (Y > 0 ? acc + vy : acc - vy) : (Y > 0 ? vy : -vy);
-  if (Z) acc = (X || Y) ? (Z > 0 ? acc + vz : acc - vz) : (Z > 0 ? vz : -vz);
-  return acc;
+// One pair from its even part e (without qp Sk) and c.O.  The two values are
+// converted on the FP64 pipe (fx_to_double_cvt); GENERAL: with the integer
+// routine, the same bits.
+template <bool LP1, bool GENERAL>
+__host__ __device__ __forceinline__ void fx_pair(int64_t e, int64_t co, int64_t Dk, int64_t Sk, Bal qm, Bal qp,
+                                                 uint32_t px, int es, double& pa, double& pb) {
+  // 2^kx D as a product: the FMA pipe has room, the integer pipe has not
+  const int64_t o = mulhi_q64(qm, bal(static_cast<int64_t>(static_cast<uint64_t>(Dk) * px))) + co;
+  if (!LP1) e += mulhi_q64(qp, bal(static_cast<int64_t>(static_cast<uint64_t>(Sk) * px)));
+  pa = GENERAL ? fx_to_double(e + o, es) : fx_to_double_cvt(e + o, es);
+  pb = GENERAL ? fx_to_double(e - o, es) : fx_to_double_cvt(e - o, es);
 }
-
-// Pair with first direction (X, Y, Z): DIAG for the face diagonals (weight
-// 1/36: K0, T and O halved), LP1 when qp = 0.  The two values are converted
-// with fx_to_double_pos when both qualify in every thread of the warp (on the
-// host: in this node), otherwise with fx_to_double; the bits are the same.
-// CVT: convert with fx_to_double_cvt (the FP64 pipe's int64 -> double).
-template <int X, int Y, int Z, bool DIAG, bool LP1, bool GENERAL = false, bool CVT = false>
-__host__ __device__ __forceinline__ void fx_pair(const FxClass& q, int64_t Dk, int64_t Sk, int64_t qm, int64_t qp,
-                                                 int es, double& pa, double& pb) {
-  const int64_t cu = fx_cdot<X, Y, Z>(q.ux, q.uy, q.uz);
-  const int64_t ct = fx_cdot<X, Y, Z>(q.Tx, q.Ty, q.Tz);
-  const int64_t co = fx_cdot<X, Y, Z>(q.Ox, q.Oy, q.Oz);
-  int64_t e = q.K0 + mulhi_q64(cu, ct);
-  int64_t o = mulhi_q64(qm, Dk);
-  if (DIAG) {
-    e >>= 1;
-    o += co >> 1;
-  } else {
-    o += co;
-  }
-  if (!LP1) e += mulhi_q64(qp, Sk);
-  const int64_t va = e + o, vb = e - o;
-  if (CVT && !GENERAL) {
-    pa = fx_to_double_cvt(va, es);
-    pb = fx_to_double_cvt(vb, es);
-    return;
-  }
-  bool fast = !GENERAL && fx_pos_wide(va) && fx_pos_wide(vb);
-#ifdef __CUDA_ARCH__
-  fast = __all_sync(__activemask(), fast);
-#endif
-  if (fast) {
-    pa = fx_to_double_pos(va, es);
-    pb = fx_to_double_pos(vb, es);
-  } else {
-    pa = fx_to_double(va, es);
-    pb = fx_to_double(vb, es);
-  }
-}
-
-#ifndef LBM_FX_CVT_PAIRS
-#define LBM_FX_CVT_PAIRS 2
-#endif
-constexpr int kFxCvtPairs = LBM_FX_CVT_PAIRS;
 
 // The nine pairs in the direction order of the lattice (see fx_moments), from
-// the moment-scale D and Sk of fx_moments; es = emax - KX.
-template <bool LP1, int KX, bool GENERAL = false>
+// the moment-scale D and Sk of fx_moments; es = emax - kx.
+template <bool LP1, bool GENERAL = false>
 __host__ __device__ __forceinline__ void fx_pairs(const FxClass& q, const int64_t (&D)[10], const int64_t (&Sk)[10],
-                                                  int64_t qm, int64_t qp, int es, double (&p)[19]) {
-  int64_t Df[10], Sf[10];
-#pragma unroll
-  for (int k = 1; k <= 9; ++k) {
-    Df[k] = static_cast<int64_t>(static_cast<uint64_t>(D[k]) << KX);
-    Sf[k] = LP1 ? 0 : static_cast<int64_t>(static_cast<uint64_t>(Sk[k]) << KX);
-  }
-  // the first kFxCvtPairs pairs convert on the FP64 pipe (fx_to_double_cvt)
-  fx_pair<1, 0, 0, false, LP1, GENERAL, (kFxCvtPairs > 0)>(q, Df[1], Sf[1], qm, qp, es, p[1], p[2]);
-  fx_pair<0, 1, 0, false, LP1, GENERAL, (kFxCvtPairs > 1)>(q, Df[2], Sf[2], qm, qp, es, p[3], p[4]);
-  fx_pair<0, 0, 1, false, LP1, GENERAL, (kFxCvtPairs > 2)>(q, Df[3], Sf[3], qm, qp, es, p[5], p[6]);
-  fx_pair<1, 1, 0, true, LP1, GENERAL, (kFxCvtPairs > 3)>(q, Df[4], Sf[4], qm, qp, es, p[7], p[8]);
-  fx_pair<1, -1, 0, true, LP1, GENERAL, (kFxCvtPairs > 4)>(q, Df[5], Sf[5], qm, qp, es, p[9], p[10]);
-  fx_pair<1, 0, 1, true, LP1, GENERAL, (kFxCvtPairs > 5)>(q, Df[6], Sf[6], qm, qp, es, p[11], p[12]);
-  fx_pair<1, 0, -1, true, LP1, GENERAL, (kFxCvtPairs > 6)>(q, Df[7], Sf[7], qm, qp, es, p[13], p[14]);
-  fx_pair<0, 1, 1, true, LP1, GENERAL, (kFxCvtPairs > 7)>(q, Df[8], Sf[8], qm, qp, es, p[15], p[16]);
-  fx_pair<0, 1, -1, true, LP1, GENERAL, (kFxCvtPairs > 8)>(q, Df[9], Sf[9], qm, qp, es, p[17], p[18]);
+                                                  int64_t qm64, int64_t qp64, int es, int kx, double (&p)[19]) {
+  const Bal qm = bal(qm64), qp = bal(qp64);
+  const uint32_t px = 1u << kx;
+  fx_pair<LP1, GENERAL>(q.K0 + 2 * q.Ax, 2 * q.Ox, D[1], Sk[1], qm, qp, px, es, p[1], p[2]);
+  fx_pair<LP1, GENERAL>(q.K0 + 2 * q.Ay, 2 * q.Oy, D[2], Sk[2], qm, qp, px, es, p[3], p[4]);
+  fx_pair<LP1, GENERAL>(q.K0 + 2 * q.Az, 2 * q.Oz, D[3], Sk[3], qm, qp, px, es, p[5], p[6]);
+  const int64_t Kh = q.K0 >> 1;
+  const int64_t Exy = Kh + q.Ax + q.Ay, Exz = Kh + q.Ax + q.Az, Eyz = Kh + q.Ay + q.Az;
+  fx_pair<LP1, GENERAL>(Exy + q.Cxy, q.Ox + q.Oy, D[4], Sk[4], qm, qp, px, es, p[7], p[8]);
+  fx_pair<LP1, GENERAL>(Exy - q.Cxy, q.Ox - q.Oy, D[5], Sk[5], qm, qp, px, es, p[9], p[10]);
+  fx_pair<LP1, GENERAL>(Exz + q.Cxz, q.Ox + q.Oz, D[6], Sk[6], qm, qp, px, es, p[11], p[12]);
+  fx_pair<LP1, GENERAL>(Exz - q.Cxz, q.Ox - q.Oz, D[7], Sk[7], qm, qp, px, es, p[13], p[14]);
+  fx_pair<LP1, GENERAL>(Eyz + q.Cyz, q.Oy + q.Oz, D[8], Sk[8], qm, qp, px, es, p[15], p[16]);
+  fx_pair<LP1, GENERAL>(Eyz - q.Cyz, q.Oy - q.Oz, D[9], Sk[9], qm, qp, px, es, p[17], p[18]);
 }
 
-// Q64 image of a rate constant |x| < 1/2: round(x * 2^64).
-inline int64_t q64_of(double x) { return static_cast<int64_t>(std::llround(std::ldexp(x, 64))); }
+// Q64 image of a rate constant |x| <= 1/2: round(x * 2^64), kept below 2^63 -
+// 2^31 in magnitude for mulhi_q64 (rates within 2^-33 of 0 or 2 alone).
+inline int64_t q64_of(double x) {
+  constexpr int64_t most = INT64_MAX - INT32_MAX - int64_t(1);
+  const double v = std::ldexp(x, 64);
+  if (v >= 9.2233720368e18) return most;
+  if (v <= -9.2233720368e18) return -most;
+  return static_cast<int64_t>(std::llround(v));
+}
+
+// ---- the class values in fixed point ---------------------------------------------------
+//
+// With exact integer moments S = sum d_i and J = sum c_i d_i, the class values
+// of the pair update need no FP64 arithmetic either.  With q = rho u (which is
+// kd (J + G/2), G = rho g, kd = 1 / (1 + s/2)) and F = G - s q, they are
+//   T = K1 u + a+/2 F = l+/4 q + a+/2 F,   O = K2 u + a-/6 F = l-/6 q + a-/6 F,
+//   K0 = l+/18 (S - 3/2 q.u) - 3 a+/18 u.F = l+/18 S - u.T / 3,
+// all linear in q and F with per-launch Q64 constants; only u = q / rho, a
+// factor of second-order products, takes a division (an integer reciprocal of
+// rho, two Newton steps from a float estimate).  GB300 runs FP64 on 2 lanes
+// per SM against 64 integer and 128 FMA lanes, and these terms in FP64 (27 to
+// 50 instructions a node, 16 SM cycles a warp each) were what bound the FP64
+// steps.
+//
+// The pair scale is 2^(es - 1080) with es = emax - kx: kx = 4 for positive
+// PDFs near each other when l+ = 1 (full storage), 2 for other full-storage
+// nodes, and 0 for deviations, whose momentum reaches 12 times their largest
+// member.  Bounds (each checked, in units of the pair scale unless noted):
+// |J_a| < 2^61, |G_a| < 2^59, |u_a| < 1/4, 0 <= s <= 1, and at the moment
+// scale |S| < 2^60 (kx >= 2) or 2^62 (kx = 0).  With l+-, a+- in their ranges
+// (k1 = l+/4 and a+/2 < 1/2, l-/6 < 1/3, a-/6 < 1/6) this gives |q| < 1.13
+// 2^61, |F| < 1.38 2^61, |T| < 1.26 2^61, |c.T| < 2.51 2^61, |O| < 0.61 2^61,
+// |K0| < 0.25 2^61 (0.45 2^61 at kx = 4) and every output below 2^63.
+struct FxColl {
+  int64_t k0a4;              // 4 l+/18 as a Q64 fraction, and so the next
+  int64_t k1h, fsh;          // l+/8, a+/4 (T halved)
+  int64_t k2h, foh;          // l-/12, a-/12 (O halved)
+  int64_t qm, qp;            // (1 - l-)/2, (1 - l+)/2
+  int64_t gm[3];             // body force: gm 2^(ge - 62), 2^62 <= |gm| < 2^63 (or 0)
+  int ge[3];
+  double rho_s;              // density of the storage shift, 0 for full storage
+  int emin;                  // least moment scale (deviation storage: that of the force)
+  bool gx;                   // the force points along x
+};
+
+// The constants are the doubles of the FP64 update (make_coll), so that both
+// updates evaluate the same map; those below 1/4 are exact as Q64 fractions.
+inline FxColl make_fx_coll(double lp, double lm, const double (&g)[3], double rho_s) {
+  FxColl c;
+  const double ap = 1.0 - lp / 2, am = 1.0 - lm / 2;
+  c.k0a4 = q64_of(4.0 * (lp / 18.0));
+  c.k1h = q64_of(lp / 4.0 / 2.0);
+  c.fsh = q64_of(ap / 2.0 / 2.0);
+  c.k2h = q64_of(lm / 6.0 / 2.0);
+  c.foh = q64_of(am / 6.0 / 2.0);
+  c.qm = q64_of((1.0 - lm) / 2);
+  c.qp = q64_of((1.0 - lp) / 2);
+  for (int a = 0; a < 3; ++a) {
+    int e = 0;
+    const double m = std::frexp(g[a], &e);  // g = m 2^e, 1/2 <= |m| < 1
+    c.gm[a] = static_cast<int64_t>(std::ldexp(m, 63));
+    c.ge[a] = g[a] != 0.0 ? e - 1 : -4096;
+  }
+  c.rho_s = rho_s;
+  // deviations may be far below the force (a start from rest, strong drag):
+  // the scale then follows rho g, the larger term of the result
+  c.emin = kFxMinExp;
+  if (rho_s != 0.0)
+    for (int a = 0; a < 3; ++a) {
+      const int e = dexp(rho_s * g[a]);
+      c.emin = e > c.emin && e < kFxMaxExp ? e : c.emin;
+    }
+  c.gx = g[1] == 0.0 && g[2] == 0.0;
+  return c;
+}
+
+__host__ __device__ __forceinline__ uint64_t umulhi64(uint64_t a, uint64_t b) {
+#ifdef __CUDA_ARCH__
+  return __umul64hi(a, b);
+#else
+  return static_cast<uint64_t>((static_cast<unsigned __int128>(a) * b) >> 64);
+#endif
+}
+
+// 2^125 / D for 2^63 <= D < 2^64, within a relative 2^-60, in (2^61, 2^62]: a
+// float estimate of the high word's reciprocal (21 bits or more) and two
+// integer Newton steps.
+__host__ __device__ __forceinline__ int64_t fx_recip(uint64_t D) {
+  const uint32_t dh = static_cast<uint32_t>(D >> 32), dl = static_cast<uint32_t>(D);
+  constexpr int64_t one = int64_t(1) << 62;
+#ifdef __CUDA_ARCH__
+  const uint32_t r0 = __float2uint_rz(__fdividef(4611686018427387904.0f, __uint2float_rz(dh)));  // 2^62 / dh
+  const uint64_t low = __umulhi(dl, r0);
+#else
+  const uint32_t r0 = static_cast<uint32_t>(4611686018427387904.0f / static_cast<float>(dh));
+  const uint64_t low = (static_cast<uint64_t>(dl) * r0) >> 32;
+#endif
+  const int64_t e = one - static_cast<int64_t>(static_cast<uint64_t>(dh) * r0 + low);  // |e| < 2^42
+  const uint64_t r1 = (static_cast<uint64_t>(r0) << 32) +
+                      static_cast<uint64_t>((static_cast<int64_t>(r0 >> 1) * static_cast<int32_t>(e >> 12)) >> 17);
+  const int32_t e2 = static_cast<int32_t>(one - static_cast<int64_t>(umulhi64(D, r1)));
+  return static_cast<int64_t>((r1 + static_cast<uint64_t>((static_cast<int64_t>(r1 >> 33) * e2) >> 29)) >> 1);
+}
+
+// Class values at the pair scale of one node, from its moments at scale emax;
+// false where a bound fails (the caller then takes the FP64 update).  s: the
+// node's Brinkman solid fraction (DRAG only).
+template <bool FORCE, bool DRAG, bool LP1>
+__host__ __device__ __forceinline__ bool fx_class_int(const FxColl& c, int emax, int kx, int64_t S, int64_t Jx,
+                                                      int64_t Jy, int64_t Jz, double s, FxClass& q) {
+  const int es = emax - kx;
+  // the bits of a value's high word that differ from its sign
+  auto mag = [](int64_t v) {
+    const int32_t h = static_cast<int32_t>(v >> 32);
+    return static_cast<uint32_t>(h ^ (h >> 31));
+  };
+  // rho = D 2^(er - 63), 2^63 <= D < 2^64
+  uint64_t D;
+  int er;
+  bool ok;
+  if (c.rho_s != 0.0) {  // uniform: deviation storage
+    const uint64_t b = dbits(c.rho_s + fx_to_double_cvt(S, emax));
+    D = (b << 11) | kSignBit;
+    er = static_cast<int>(b >> 52) - 1023;  // a negative density, Inf or NaN: er >= 1024
+    ok = er > -1000 && er < 1000 && mag(S) < 1u << 30;
+  } else {
+    const int lz = clz64(static_cast<uint64_t>(S));
+    ok = S > 0 && mag(S) < 1u << 28;
+    D = (static_cast<uint64_t>(S) << (lz & 63)) | kSignBit;
+    er = emax - 1017 - lz;
+  }
+  // u = q / rho will be mulhi(q 2^pre, r) 2^(3 - post), shifted left before
+  // the product as far as |u| < 1/4 allows
+  const int sh = es - 1016 - er;
+  const int pre = sh > 1 ? sh - 1 : 0, down = 1 - sh + pre;  // >= 0
+  const int post = down > 63 ? 63 : down;
+  const int nj = (pre > 1 ? 30 - pre : 29) - kx;
+  ok = ok && emax < kFxMaxExp && nj >= 0 && (mag(Jx) | mag(Jy) | mag(Jz)) >> (nj & 31) == 0;
+  const Bal r = bal(fx_recip(D));
+  const uint32_t px = 1u << kx;
+  int64_t qx = static_cast<int64_t>(static_cast<uint64_t>(Jx) * px);
+  int64_t qy = static_cast<int64_t>(static_cast<uint64_t>(Jy) * px);
+  int64_t qz = static_cast<int64_t>(static_cast<uint64_t>(Jz) * px);
+  int64_t Fx = 0, Fy = 0, Fz = 0;
+  if (FORCE || DRAG) {
+    // rho g_a at the pair scale
+    const Bal Dh = bal(static_cast<int64_t>(D >> 2));
+    const int s0 = es - 1020 - er;
+    const int shx = s0 - c.ge[0];
+    ok = ok && shx >= 3 + pre;
+    Fx = mulhi_q64(bal(c.gm[0] >> 1), Dh) >> (((shx > 65 ? 65 : shx) - 2) & 63);
+    qx += Fx >> 1;
+    if (!c.gx) {  // uniform
+      const int shy = s0 - c.ge[1], shz = s0 - c.ge[2];
+      ok = ok && shy >= 3 + pre && shz >= 3 + pre;
+      Fy = mulhi_q64(bal(c.gm[1] >> 1), Dh) >> (((shy > 65 ? 65 : shy) - 2) & 63);
+      Fz = mulhi_q64(bal(c.gm[2] >> 1), Dh) >> (((shz > 65 ? 65 : shz) - 2) & 63);
+      qy += Fy >> 1;
+      qz += Fz >> 1;
+    }
+  }
+  if (DRAG) {
+    const uint64_t b = dbits(s);
+    ok = ok && b <= 0x3ff0000000000000ull;  // 0 <= s <= 1
+    const int e = 1023 - static_cast<int>(b >> 52);
+    // s/2 as a Q64 fraction (at most 2^63)
+    const uint64_t sh2 = e < 64 ? (((b << 11) | kSignBit) >> (e & 63)) : 0u;
+    const Bal kd = bal(fx_recip(kSignBit + (sh2 >> 1)));  // 1 / (1 + s/2), Q62
+    qx = 2 * mulhi_q64(bal(2 * qx), kd);
+    qy = 2 * mulhi_q64(bal(2 * qy), kd);
+    qz = 2 * mulhi_q64(bal(2 * qz), kd);
+    const Bal s4 = bal(static_cast<int64_t>(sh2 >> 1));
+    Fx -= 2 * mulhi_q64(bal(2 * qx), s4);
+    Fy -= 2 * mulhi_q64(bal(2 * qy), s4);
+    Fz -= 2 * mulhi_q64(bal(2 * qz), s4);
+  }
+  const uint32_t pp = 1u << (pre & 31);
+  auto velocity = [&](int64_t v) {
+    const int64_t m = mulhi_q64(bal(static_cast<int64_t>(static_cast<uint64_t>(v) * pp)), r);
+    return static_cast<int64_t>(static_cast<uint64_t>(m) << 3) >> post;
+  };
+  const int64_t ux = velocity(qx), uy = velocity(qy), uz = velocity(qz);
+  ok = ok && (mag(ux) | mag(uy) | mag(uz)) < 1u << 30;
+  int64_t Tx, Ty, Tz;  // halved, as are Ox, Oy, Oz
+  if (LP1) {  // l+/4 and a+/2 are both 1/4
+    Tx = (qx + Fx) >> 3;
+    Ty = (qy + Fy) >> 3;
+    Tz = (qz + Fz) >> 3;
+  } else {
+    const Bal k1 = bal(c.k1h);
+    Tx = mulhi_q64(k1, bal(qx));
+    Ty = mulhi_q64(k1, bal(qy));
+    Tz = mulhi_q64(k1, bal(qz));
+  }
+  const Bal k2 = bal(c.k2h);
+  q.Ox = mulhi_q64(k2, bal(qx));
+  q.Oy = mulhi_q64(k2, bal(qy));
+  q.Oz = mulhi_q64(k2, bal(qz));
+  if (FORCE || DRAG) {
+    const Bal fs = bal(c.fsh), fo = bal(c.foh), fx = bal(Fx);
+    q.Ox += mulhi_q64(fo, fx);
+    if (!LP1) Tx += mulhi_q64(fs, fx);
+    if (DRAG || !c.gx) {
+      const Bal fy = bal(Fy), fz = bal(Fz);
+      q.Oy += mulhi_q64(fo, fy);
+      q.Oz += mulhi_q64(fo, fz);
+      if (!LP1) {
+        Ty += mulhi_q64(fs, fy);
+        Tz += mulhi_q64(fs, fz);
+      }
+    }
+  }
+  fx_even(q, ux, uy, uz, Tx, Ty, Tz);
+  // K0 = l+/18 S - u.T / 3
+  const int64_t S2 = kx ? static_cast<int64_t>(static_cast<uint64_t>(S) << (kx - 2)) : S >> 2;
+  constexpr int64_t third2 = 0x5555555555555555ll;  // 1/3 as a Q64 fraction
+  q.K0 = mulhi_q64(c.k0a4, S2) - 2 * mulhi_q64(third2, q.Ax + q.Ay + q.Az);
+  return ok;
+}
+
+// The post-collision PDFs of one node from its class values (fx_class_int),
+// its moments at scale emax and the rest PDF's image f0.
+template <bool LP1>
+__host__ __device__ __forceinline__ void fx_update(const FxColl& c, const FxClass& q, int emax, int kx,
+                                                   const int64_t (&D)[10], const int64_t (&Sk)[10], int64_t f0,
+                                                   double (&d)[19]) {
+  fx_pairs<LP1>(q, D, Sk, c.qm, c.qp, emax - kx, kx, d);
+  // rest PDF: (1 - l+) f0 + 6 K0
+  int64_t v0 = 6 * q.K0;
+  if (!LP1) v0 += mulhi_q64(c.qp, static_cast<int64_t>(static_cast<uint64_t>(f0) << (kx + 1)));
+  d[0] = fx_to_double_cvt(v0, emax - kx);
+}
+
+// Binades of the pair scale below the moments' (see above).
+template <bool LP1> __host__ __device__ __forceinline__ int fx_kx(const FxColl& c, bool near) {
+  return c.rho_s != 0.0 ? 0 : (LP1 && near) ? 4 : 2;
+}
 
 }  // namespace dev
 }  // namespace lbm

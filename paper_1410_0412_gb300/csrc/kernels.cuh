@@ -52,42 +52,38 @@ constexpr int ctas(int n128, int b = kBlock) { return n128 * 128 / b > 0 ? n128 
 // FP32 is fastest at 10 CTAs (<= 51 registers), FP16 at 12 (<= 42; 16 spills
 // and loses 7 %; OS-NT-R FP16 on the paper's channel 49.1 -> 51.5 GFLUP/s from
 // 10 to 12), with the adjacency list at 8 (AA odd) or 5 (OS-NT).  The
-// double-float path takes 8 (AA odd) and 6 (others).  Native FP64: the AA
-// steps fit 64 registers without spills and are fastest at 8 CTAs (AA-R on the
-// 256^3 bed 12.8 / 13.6 / 14.2 / 14.6 GFLUP/s at 5 / 6 / 7 / 8); OS-NT and
-// the Esoteric Twist step spill at 7 and take 6.
-#ifndef LBM_MIN_CTAS_F64
-#define LBM_MIN_CTAS_F64 6
-#endif
-#ifndef LBM_MIN_CTAS_F64_AA
-#define LBM_MIN_CTAS_F64_AA 8
-#endif
+// double-float path takes 8 (AA odd) and 6 (others).  Native FP64 with l+ = 1
+// fits 64 registers in every form and takes 8 (ms for 10 steps on the 256^3
+// bed at 6 / 7 / 8: AA-R 6.63 / 6.31 / 6.15, OS-NT-R 7.17 / 6.75 / 6.47); the
+// general rates keep the nine pair sums as well and spill there: AA 6 (7.33
+// against 7.41 / 7.57 at 7 / 8), OS-NT 7 (7.45 against 7.46 / 7.59 at 6 / 8),
+// Esoteric Twist 6.
 #ifndef LBM_MIN_CTAS_OSNT_RIA_F16
 #define LBM_MIN_CTAS_OSNT_RIA_F16 12
 #endif
-template <int PREC, bool RIA> struct MinCtasOsnt { static constexpr int value = RIA ? 10 : 5; };
-template <bool RIA> struct MinCtasOsnt<LBM_F16S, RIA> { static constexpr int value = RIA ? LBM_MIN_CTAS_OSNT_RIA_F16 : 5; };
-template <bool RIA> struct MinCtasOsnt<LBM_F64, RIA> { static constexpr int value = LBM_MIN_CTAS_F64; };
-template <bool RIA> struct MinCtasOsnt<LBM_F64_DF, RIA> { static constexpr int value = 6; };
-template <int PREC> struct MinCtasEven { static constexpr int value = 5; };
-template <> struct MinCtasEven<LBM_F64> { static constexpr int value = LBM_MIN_CTAS_F64_AA; };
-template <> struct MinCtasEven<LBM_F64_DF> { static constexpr int value = 6; };
+template <int PREC, bool RIA, bool LP1> struct MinCtasOsnt { static constexpr int value = RIA ? 10 : 5; };
+template <bool RIA, bool LP1> struct MinCtasOsnt<LBM_F16S, RIA, LP1> { static constexpr int value = RIA ? LBM_MIN_CTAS_OSNT_RIA_F16 : 5; };
+template <bool RIA, bool LP1> struct MinCtasOsnt<LBM_F64, RIA, LP1> { static constexpr int value = LP1 ? 8 : 7; };
+template <bool RIA, bool LP1> struct MinCtasOsnt<LBM_F64_DF, RIA, LP1> { static constexpr int value = 6; };
+template <int PREC, bool LP1> struct MinCtasEven { static constexpr int value = 5; };
+template <bool LP1> struct MinCtasEven<LBM_F64, LP1> { static constexpr int value = LP1 ? 8 : 6; };
+template <bool LP1> struct MinCtasEven<LBM_F64_DF, LP1> { static constexpr int value = 6; };
 #ifndef LBM_MIN_CTAS_ODD_RIA
 #define LBM_MIN_CTAS_ODD_RIA 10
 #endif
 #ifndef LBM_MIN_CTAS_ODD_RIA_F16
 #define LBM_MIN_CTAS_ODD_RIA_F16 12
 #endif
-template <int PREC, bool RIA> struct MinCtasOdd { static constexpr int value = RIA ? LBM_MIN_CTAS_ODD_RIA : 8; };
-template <bool RIA> struct MinCtasOdd<LBM_F16S, RIA> { static constexpr int value = RIA ? LBM_MIN_CTAS_ODD_RIA_F16 : 8; };
-template <bool RIA> struct MinCtasOdd<LBM_F64, RIA> { static constexpr int value = LBM_MIN_CTAS_F64_AA; };
-template <bool RIA> struct MinCtasOdd<LBM_F64_DF, RIA> { static constexpr int value = 8; };
+template <int PREC, bool RIA, bool LP1> struct MinCtasOdd { static constexpr int value = RIA ? LBM_MIN_CTAS_ODD_RIA : 8; };
+template <bool RIA, bool LP1> struct MinCtasOdd<LBM_F16S, RIA, LP1> { static constexpr int value = RIA ? LBM_MIN_CTAS_ODD_RIA_F16 : 8; };
+template <bool RIA, bool LP1> struct MinCtasOdd<LBM_F64, RIA, LP1> { static constexpr int value = LP1 ? 8 : 6; };
+template <bool RIA, bool LP1> struct MinCtasOdd<LBM_F64_DF, RIA, LP1> { static constexpr int value = 8; };
 // The Esoteric Twist step: every step is indirect, and a sweep of 6/8/10/12
 // on GB300 put FP32 and FP16 at 10 CTAs (<= 51 registers; +3-5 % over 8),
-// double-float at 8 (+3 % over 6); native FP64 takes 6 (see above).
-template <int PREC> struct MinCtasEt { static constexpr int value = 10; };
-template <> struct MinCtasEt<LBM_F64_DF> { static constexpr int value = 8; };
-template <> struct MinCtasEt<LBM_F64> { static constexpr int value = LBM_MIN_CTAS_F64; };
+// double-float at 8 (+3 % over 6); native FP64: see above.
+template <int PREC, bool LP1> struct MinCtasEt { static constexpr int value = 10; };
+template <bool LP1> struct MinCtasEt<LBM_F64_DF, LP1> { static constexpr int value = 8; };
+template <bool LP1> struct MinCtasEt<LBM_F64, LP1> { static constexpr int value = LP1 ? 8 : 6; };
 static_assert(kBlock % kWarpNodes == 0, "a warp must cover one run-index group");
 
 // ---- storage traits -----------------------------------------------------------------
@@ -302,7 +298,7 @@ template <class R> struct CollConst {
   R abb_in[2], abb_out[2];  // 2 w (rho_bc - rho_s) for w = 1/18 and 1/36
   double abb64_in[2], abb64_out[2];  // the same in double (the double-float odd step's FP64 gather)
   R inv_s;                  // 1 / storage scale of the scaled collision (see make_coll_step)
-  long long qm_fx, qp_fx;   // qm and qp as Q64 fractions (the FP64 fixed-point pair update)
+  FxColl fx;                // constants of the FP64 collision in fixed point (exact64.cuh)
   bool gx;                  // the body force points along x (g_y = g_z = 0)
 };
 
@@ -330,8 +326,7 @@ template <class R> inline CollConst<R> make_coll(const KParams& kp) {
   }
   c.rho_s = R(kp.rho_s);
   c.inv_s = R(1.0f);
-  c.qm_fx = q64_of((1.0 - kp.lm) / 2);
-  c.qp_fx = q64_of((1.0 - kp.lp) / 2);
+  c.fx = make_fx_coll(kp.lp, kp.lm, kp.g, kp.rho_s);
   c.gx = kp.g[1] == 0.0 && kp.g[2] == 0.0;
   for (int k = 0; k < 2; ++k) {
     const double w = k == 0 ? 1.0 / 18.0 : 1.0 / 36.0;
@@ -570,35 +565,31 @@ __device__ __forceinline__ void collide_m(R (&d)[kQ], const CollConst<R>& c, con
   pair_terms<R, LP1>(d, c, node_terms<R, FORCE, DRAG>(c, s, drho, jx, jy, jz), sa, da);
 }
 
-// The FP64 collision: exact fixed-point moments (exact64.cuh), the node terms
-// in FP64, and the pair update in fixed point on the integer pipe when the
-// node's values are in its range (fx_class_ok; a warp-uniform branch),
-// otherwise in FP64 from the moments rounded to double.  NaN or Inf PDFs
-// take the FP64 branch and come out NaN.
+// The FP64 collision: exact fixed-point moments, the class terms and the pair
+// update in fixed point on the integer and FMA pipes (exact64.cuh) when every
+// node of the warp is in its range (fx_class_int; a warp-uniform branch),
+// otherwise in FP64 from the moments rounded to double.  NaN or Inf PDFs take
+// the FP64 branch and come out NaN.
 template <bool FORCE, bool DRAG, bool LP1>
 __device__ __forceinline__ void collide_f64(double (&d)[kQ], const CollConst<double>& c, const double s) {
-  int64_t Sk[10], D[10], S, Jx, Jy, Jz;
+  int64_t Sk[10], D[10], S, Jx, Jy, Jz, f0;
   // the shorter conversions when every node of the warp has positive PDFs
   // within 5 binades of its largest (full-f storage near equilibrium)
   int emax_fast, emax;
-  double drho;
-  if (__all_sync(__activemask(), fx_pos_near(d, emax_fast))) {
-    emax = fx_moments<!LP1, true>(d, Sk, D, S, Jx, Jy, Jz, emax_fast);
-    // positive PDFs: S >= the largest one's image >= 2^57, so the short conversion applies
-    drho = fx_to_double_pos(S, emax);
-  } else {
-    emax = fx_moments<!LP1>(d, Sk, D, S, Jx, Jy, Jz);
-    drho = emax < kFxMaxExp ? fx_to_double(S, emax) : dfrom(0x7ff8000000000000ull);
-  }
-  const NodeTerms<double> t = node_terms<double, FORCE, DRAG>(c, s, drho, fx_to_double(Jx, emax),
-                                                              fx_to_double(Jy, emax), fx_to_double(Jz, emax));
-  const bool ok = fx_class_ok(emax, t.ux, t.uy, t.uz, t.K0a, t.Tx, t.Ty, t.Tz, t.Ox, t.Oy, t.Oz);
+  const bool near = __all_sync(__activemask(), fx_pos_near(d, emax_fast));
+  if (near)
+    emax = fx_moments<!LP1, true>(d, Sk, D, S, Jx, Jy, Jz, emax_fast, &f0);
+  else
+    emax = fx_moments<!LP1>(d, Sk, D, S, Jx, Jy, Jz, 0, &f0, c.fx.emin);
+  const int kx = fx_kx<LP1>(c.fx, near);
+  FxClass q;
+  const bool ok = fx_class_int<FORCE, DRAG, LP1>(c.fx, emax, kx, S, Jx, Jy, Jz, s, q);
   if (__all_sync(__activemask(), ok)) {
-    constexpr int kx = LP1 ? 4 : 2;
-    const FxClass q = fx_class(emax - kx, t.ux, t.uy, t.uz, t.K0a, t.Tx, t.Ty, t.Tz, t.Ox, t.Oy, t.Oz);
-    fx_pairs<LP1, kx>(q, D, Sk, c.qm_fx, c.qp_fx, emax - kx, d);
-    d[0] = LP1 ? 6.0 * t.K0a : ::fma(c.omlp, d[0], 6.0 * t.K0a);
+    fx_update<LP1>(c.fx, q, emax, kx, D, Sk, f0, d);
   } else {
+    const double drho = emax < kFxMaxExp ? fx_to_double(S, emax) : dfrom(0x7ff8000000000000ull);
+    const NodeTerms<double> t = node_terms<double, FORCE, DRAG>(c, s, drho, fx_to_double(Jx, emax),
+                                                                fx_to_double(Jy, emax), fx_to_double(Jz, emax));
     double sa[10], da[10];
 #pragma unroll
     for (int k = 1; k <= 9; ++k) {
@@ -674,7 +665,7 @@ template <int PREC, bool RIA> struct OsntBlock {
 // evict-first stores so the write stream does not push src out of L2.
 template <int PREC, bool RIA, bool FORCE, bool DRAG, bool LP1 = false>
 __global__ void __launch_bounds__(OsntBlock<PREC, RIA>::value,
-                                  ctas(MinCtasOsnt<PREC, RIA>::value, OsntBlock<PREC, RIA>::value))
+                                  ctas(MinCtasOsnt<PREC, RIA, LP1>::value, OsntBlock<PREC, RIA>::value))
     k_osnt(DevTables t, KParams kp, CollConst<typename St<PREC>::R> c, const typename St<PREC>::T* __restrict__ src,
            typename St<PREC>::T* __restrict__ dst, const float* __restrict__ s, int N) {
   using R = typename St<PREC>::R;
@@ -717,7 +708,7 @@ __global__ void __launch_bounds__(OsntBlock<PREC, RIA>::value,
 // AA even step: direct read of the 19 local PDFs, collide, write to the
 // opposite local slots (no index loads at all).
 template <int PREC, bool FORCE, bool DRAG, bool LP1 = false>
-__global__ void __launch_bounds__(kBlock, ctas(MinCtasEven<PREC>::value)) k_aa_even(DevTables t, KParams kp, CollConst<typename St<PREC>::R> c,
+__global__ void __launch_bounds__(kBlock, ctas(MinCtasEven<PREC, LP1>::value)) k_aa_even(DevTables t, KParams kp, CollConst<typename St<PREC>::R> c,
                                                     typename St<PREC>::T* __restrict__ A,
                                                     const float* __restrict__ s, int N) {
   using R = typename St<PREC>::R;
@@ -769,7 +760,7 @@ __global__ void __launch_bounds__(kBlock) k_aa_even_h2(DevTables t, KParams kp, 
 // AA odd step: read f_i from the neighbour's opposite slot A[inv i][m_i], collide,
 // write p_i to A[i][m_{inv i}] -- the same 19 slots, so in place and race-free.
 template <int PREC, bool RIA, bool FORCE, bool DRAG, bool LP1 = false>
-__global__ void __launch_bounds__(kBlock, ctas(MinCtasOdd<PREC, RIA>::value)) k_aa_odd(DevTables t, KParams kp,
+__global__ void __launch_bounds__(kBlock, ctas(MinCtasOdd<PREC, RIA, LP1>::value)) k_aa_odd(DevTables t, KParams kp,
                                                                               CollConst<typename St<PREC>::R> c,
                                                                               typename St<PREC>::T* __restrict__ A,
                                                                               const float* __restrict__ s, int N) {
@@ -997,7 +988,7 @@ __device__ __forceinline__ unsigned et_locate(const DevTables& t, int n, int (&l
 }
 
 template <int PREC, bool RIA, bool ODD, bool FORCE, bool DRAG, bool LP1 = false>
-__global__ void __launch_bounds__(kBlock, ctas(MinCtasEt<PREC>::value)) k_et(DevTables t, KParams kp,
+__global__ void __launch_bounds__(kBlock, ctas(MinCtasEt<PREC, LP1>::value)) k_et(DevTables t, KParams kp,
                                                                           CollConst<typename St<PREC>::R> c,
                                                                           typename St<PREC>::T* __restrict__ A,
                                                                           const float* __restrict__ s, int N) {
