@@ -361,8 +361,13 @@ __device__ __forceinline__ void block_sum_dd(double& hi, double& lo, double (*s_
 }
 
 // J partial sums of rho u_x (compensated), optional dJ/dF_T and the direct dJ/ds.
+// As k_macro, a CTA walks the nodes in strides of the grid and reduces its
+// compensated sums once: the five shuffle rounds of two-sums per 128 nodes were
+// most of the kernel's time (FP64 pipe 85 % busy), and the one-CTA sum of one
+// partial per 128 nodes took another 0.06 ms.  2.1 M FP32 nodes: 0.27 (0.38
+// with dJ/dF_T) + 0.06 ms before, 0.12 (0.15) + 0.02 now.
 template <int PREC, bool RIA>
-__global__ void __launch_bounds__(kBlock) k_objective(DevTables t, KParams kp, CollConst<typename St<PREC>::R> c,
+__global__ void __launch_bounds__(kBlock, LBM_MIN_CTAS_REDUCE) k_objective(DevTables t, KParams kp, CollConst<typename St<PREC>::R> c,
                                                       const typename St<PREC>::T* pdf, int layout,
                                                       const float* __restrict__ s, double invN,
                                                       double* __restrict__ partials,
@@ -370,28 +375,34 @@ __global__ void __launch_bounds__(kBlock) k_objective(DevTables t, KParams kp, C
                                                       double* __restrict__ grad_s, int N) {
   using R = typename St<PREC>::R;
   __shared__ double s_red[kBlock / 32][2];
-  const int n0 = blockIdx.x * kBlock;
-  const int n = n0 + threadIdx.x;
-  double f[kQ];
   double hi = 0.0, lo = 0.0;
-  if (node_canonical<PREC, RIA, false>(t, kp, c, pdf, layout, n, N, f)) {
+  const double h = 0.5 * kp.g[0];
+  const int64_t stride = int64_t(gridDim.x) * kBlock;
+  for (int64_t k = int64_t(blockIdx.x) * kBlock + threadIdx.x; k < N; k += stride) {
+    const int n = int(k);
+    R d[kQ];
+    node_load<PREC, RIA>(t, kp, c, pdf, layout, n, d);
     // rho and j_x from the stored values as exact fixed-point sums, each
     // rounded once (exact64.cuh): the objective's per-node terms carry no
     // summation error, which keeps finite differences of J above round-off
-    int64_t Sk[10], D[10], S, Jx, Jy, Jz;
-    const int emax = fx_moments<false>(f, Sk, D, S, Jx, Jy, Jz);
-    const double r = kp.rho_s + (emax < kFxMaxExp ? fx_to_double(S, emax) : dfrom(0x7ff8000000000000ull));
-    const double jx = fx_to_double(Jx, emax);
-    const double kd = s ? 1.0 / (1.0 + 0.5 * double(s[n])) : 1.0;
-    const double rux = (jx + 0.5 * kp.g[0] * r) * kd;  // rho u_x
-    hi = rux;
-    if (lamT) {
+    int64_t S, Jx, Jy, Jz;
+    const int emax = fx_moments(d, S, Jx, Jy, Jz);
+    const double r = kp.rho_s + (emax < kFxMaxExp ? fx_to_double_cvt(S, emax) : dfrom(0x7ff8000000000000ull));
+    const double jx = fx_to_double_cvt(Jx, emax);
+    const double kd = s ? drag_factor(s[n]) : 1.0;
+    const double rux = ::fma(h, r, jx) * kd;  // rho u_x
+    double sum, err;
+    two_sum(hi, rux, sum, err);
+    hi = sum;
+    lo += err;
+    if (lamT) {  // three values: c_x = -1, 0, 1
+      const double w = kd * invN;
+      const R l0 = R(h * w), lp = R((1.0 + h) * w), lm = R((h - 1.0) * w);
 #pragma unroll
-      for (int i = 0; i < kQ; ++i) lamT[at(i, t.npad, n)] = R((cx(i) + 0.5 * kp.g[0]) * kd * invN);
+      for (int i = 0; i < kQ; ++i) lamT[at(i, t.npad, n)] = cx(i) == 0 ? l0 : cx(i) > 0 ? lp : lm;
     }
     if (grad_s) grad_s[n] = -0.5 * rux * kd * invN;
   }
-  __syncthreads();
   block_sum_dd(hi, lo, s_red);
   if (threadIdx.x == 0) {
     partials[2 * size_t(blockIdx.x)] = hi;
@@ -448,22 +459,22 @@ int launch_objective_t(const lbm_lattice* L, const KParams& kp, const void* pdf,
   using T = typename dev::St<PREC>::T;
   using R = typename dev::St<PREC>::R;
   auto st = static_cast<cudaStream_t>(stream);
-  const int64_t parts = reduce_parts(L);
+  const unsigned g = reduce_grid(reduce_parts(L));
   const double invN = L->N > 0 ? 1.0 / double(L->N) : 0.0;
   if (L->N > 0) {
     const bool ria = !(L->uploaded & LBM_TABLES_ADJ);
     const auto c = dev::make_coll<R>(kp);
     if (ria)
-      dev::k_objective<PREC, true><<<grid_of(L->N), dev::kBlock, 0, st>>>(
+      dev::k_objective<PREC, true><<<g, dev::kBlock, 0, st>>>(
           L->dev, kp, c, static_cast<const T*>(pdf), layout, s, invN, partials, static_cast<R*>(lamT), grad_s,
           int(L->N));
     else
-      dev::k_objective<PREC, false><<<grid_of(L->N), dev::kBlock, 0, st>>>(
+      dev::k_objective<PREC, false><<<g, dev::kBlock, 0, st>>>(
           L->dev, kp, c, static_cast<const T*>(pdf), layout, s, invN, partials, static_cast<R*>(lamT), grad_s,
           int(L->N));
     if (int rc = cuda_check("objective launch")) return rc;
   }
-  dev::k_finish_dd<PREC><<<1, 512, 0, st>>>(partials, L->N > 0 ? parts : 0, invN, J);
+  dev::k_finish_dd<PREC><<<1, 512, 0, st>>>(partials, L->N > 0 ? int64_t(g) : 0, invN, J);
   return cuda_check("objective reduction launch");
 }
 

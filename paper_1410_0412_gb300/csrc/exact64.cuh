@@ -228,6 +228,60 @@ __host__ __device__ __forceinline__ int fx_moments(const double (&d)[19], int64_
   return emax;
 }
 
+// Node scale and fixed-point image of single-precision PDFs, in the terms of the
+// doubles (scale 2^(emax - 1080), emax the double's biased exponent): exact for
+// PDFs within 34 binades of the largest.  An Inf or a NaN gives kFxMaxExp.
+__host__ __device__ __forceinline__ uint32_t fbits(float x) {
+#ifdef __CUDA_ARCH__
+  return __float_as_uint(x);
+#else
+  uint32_t b;
+  std::memcpy(&b, &x, sizeof b);
+  return b;
+#endif
+}
+template <int Q> __host__ __device__ __forceinline__ int fx_scale(const float (&d)[Q]) {
+  uint32_t top = 0x00800000u;
+#pragma unroll
+  for (int i = 0; i < Q; ++i) {
+    const uint32_t m = fbits(d[i]) & 0x7fffffffu;
+    top = m > top ? m : top;
+  }
+  return top >= 0x7f800000u ? kFxMaxExp : static_cast<int>(top >> 23) + 896;
+}
+__host__ __device__ __forceinline__ int64_t fx_of(float x, int emax) {
+  const uint32_t b = fbits(x);
+  const int e = static_cast<int>(b >> 23) & 0xff;
+  const uint32_t m = (b & 0x007fffffu) | (e ? 0x00800000u : 0u);
+  int sh = emax - 896 - (e ? e : 1);
+  sh = sh < 63 ? sh : 63;
+  const uint64_t v = (static_cast<uint64_t>(m << 2) << 32) >> sh;  // m * 2^34 at sh = 0
+  return (b & 0x80000000u) ? -static_cast<int64_t>(v) : static_cast<int64_t>(v);
+}
+// Density deviation and momentum of single-precision PDFs, exact integers at
+// the returned scale.
+__host__ __device__ __forceinline__ int fx_moments(const float (&d)[19], int64_t& S, int64_t& Jx, int64_t& Jy,
+                                                   int64_t& Jz) {
+  const int emax = fx_scale(d);
+  int64_t D[10];
+  S = fx_of(d[0], emax);
+#pragma unroll
+  for (int k = 1; k <= 9; ++k) {
+    const int64_t a = fx_of(d[2 * k - 1], emax), b = fx_of(d[2 * k], emax);
+    S += a + b;
+    D[k] = a - b;
+  }
+  Jx = D[1] + D[4] + D[5] + D[6] + D[7];
+  Jy = D[2] + D[4] - D[5] + D[8] + D[9];
+  Jz = D[3] + D[6] - D[7] + D[8] - D[9];
+  return emax;
+}
+__host__ __device__ __forceinline__ int fx_moments(const double (&d)[19], int64_t& S, int64_t& Jx, int64_t& Jy,
+                                                   int64_t& Jz) {
+  int64_t Sk[10], D[10];
+  return fx_moments<false>(d, Sk, D, S, Jx, Jy, Jz);
+}
+
 // True when the fast conversions of fx_moments apply: every PDF positive and
 // finite-scaled (node scale below kFxMaxExp) and at most 5 binades below the
 // largest (so fx_of_pos_near's shift stays in [0, 5]; PDFs near w_i rho span
@@ -435,6 +489,7 @@ struct FxColl {
   int64_t gm[3];             // body force: gm 2^(ge - 62), 2^62 <= |gm| < 2^63 (or 0)
   int ge[3];
   double rho_s;              // density of the storage shift, 0 for full storage
+  bool shift;                // rho_s != 0 (a flag: the comparison is an FP64-pipe instruction)
   int emin;                  // least moment scale (deviation storage: that of the force)
   bool gx;                   // the force points along x
 };
@@ -458,6 +513,7 @@ inline FxColl make_fx_coll(double lp, double lm, const double (&g)[3], double rh
     c.ge[a] = g[a] != 0.0 ? e - 1 : -4096;
   }
   c.rho_s = rho_s;
+  c.shift = rho_s != 0.0;
   // deviations may be far below the force (a start from rest, strong drag):
   // the scale then follows rho g, the larger term of the result
   c.emin = kFxMinExp;
@@ -514,7 +570,7 @@ __host__ __device__ __forceinline__ bool fx_class_int(const FxColl& c, int emax,
   uint64_t D;
   int er;
   bool ok;
-  if (c.rho_s != 0.0) {  // uniform: deviation storage
+  if (c.shift) {  // uniform: deviation storage
     const uint64_t b = dbits(c.rho_s + fx_to_double_cvt(S, emax));
     D = (b << 11) | kSignBit;
     er = static_cast<int>(b >> 52) - 1023;  // a negative density, Inf or NaN: er >= 1024
@@ -627,9 +683,19 @@ __host__ __device__ __forceinline__ void fx_update(const FxColl& c, const FxClas
   d[0] = fx_to_double_cvt(v0, emax - kx);
 }
 
+// J 2^(emax - 1080) / rho as a double within (1/2 + 2^-4) ulp, for rho = D
+// 2^(er - 63), 2^63 <= D < 2^64, r = fx_recip(D) and 64 <= emax - er < 1900: J is
+// shifted to 63 bits, so that the product keeps 59 or more.
+__host__ __device__ __forceinline__ double fx_quotient(int64_t J, int emax, Bal r, int er) {
+  const uint64_t a = static_cast<uint64_t>(J ^ (J >> 63)) | 1u;
+  const int lz = clz64(a);
+  const int64_t m = mulhi_q64(bal(static_cast<int64_t>(static_cast<uint64_t>(J) << (lz - 1))), r);
+  return fx_to_double_cvt(m, emax - er - lz + 3);  // m 2^(emax - er - lz - 1077)
+}
+
 // Binades of the pair scale below the moments' (see above).
 template <bool LP1> __host__ __device__ __forceinline__ int fx_kx(const FxColl& c, bool near) {
-  return c.rho_s != 0.0 ? 0 : (LP1 && near) ? 4 : 2;
+  return c.shift ? 0 : (LP1 && near) ? 4 : 2;
 }
 
 }  // namespace dev

@@ -1172,18 +1172,13 @@ __global__ void __launch_bounds__(kBlock) k_load_canonical(DevTables t, KParams 
   }
 }
 
-// Canonical pre-collision state of one node, FP64, unshifted.
-// SHIFT: add the storage shift w_i rho_s back (the canonical PDFs); without
-// it F holds the stored deviations, for callers that form exact moments.
-template <int PREC, bool RIA, bool SHIFT = true>
-__device__ __forceinline__ bool node_canonical(const DevTables& t, const KParams& kp,
-                                               const CollConst<typename St<PREC>::R>& c,
-                                               const typename St<PREC>::T* pdf, int layout, int n, int N,
-                                               double (&F)[kQ]) {
-  using R = typename St<PREC>::R;
-  R d[kQ];
+// Stored PDFs of one node's canonical pre-collision state (deviations in
+// shifted storage), in the storage's arithmetic type.  n < N.
+template <int PREC, bool RIA>
+__device__ __forceinline__ void node_load(const DevTables& t, const KParams& kp,
+                                          const CollConst<typename St<PREC>::R>& c, const typename St<PREC>::T* pdf,
+                                          int layout, int n, typename St<PREC>::R (&d)[kQ]) {
   if (layout >= LBM_LAYOUT_ET_EVEN) {
-    if (n >= N) return false;
     int loc[7];
     et_locations(t, n, loc);
     d[0] = St<PREC>::ld(pdf + n, kp.inv_scale);
@@ -1191,43 +1186,72 @@ __device__ __forceinline__ bool node_canonical(const DevTables& t, const KParams
     for (int i = 1; i < kQ; ++i)
       d[i] = St<PREC>::ld(pdf + at(layout == LBM_LAYOUT_ET_ODD ? inv(i) : i, t.spad, loc[et_row(inv(i)) + 1]),
                           kp.inv_scale);
-#pragma unroll
-    for (int i = 0; i < kQ; ++i) F[i] = SHIFT ? double(d[i]) + wgt(i) * kp.rho_s : double(d[i]);
-    return true;
-  }
-  int m[18];
-  if (layout != LBM_LAYOUT_AA_EVEN) {
-    if (RIA) {
-      if (n >= N) return false;
-      nbr_ria(t, ria_locate(t, n), m);
-    } else {
-      if (n >= N) return false;
-      nbr_adj(t, n, m);
-    }
-  } else if (n >= N) {
-    return false;
+    return;
   }
   if (layout == LBM_LAYOUT_AA_EVEN) {
 #pragma unroll
     for (int i = 0; i < kQ; ++i) d[i] = St<PREC>::ld(pdf + at(i, t.npad, n), kp.inv_scale);
-  } else if (layout == LBM_LAYOUT_OSNT) {
-    gather<PREC, false>(pdf, t.npad, n, m, d, kp.inv_scale, c.abb_in, c.abb_out, t.pressure);
-  } else {
-    gather<PREC, true>(pdf, t.npad, n, m, d, kp.inv_scale, c.abb_in, c.abb_out, t.pressure);
+    return;
   }
-#pragma unroll
-  for (int i = 0; i < kQ; ++i) F[i] = SHIFT ? double(d[i]) + wgt(i) * kp.rho_s : double(d[i]);
-  return true;
+  int m[18];
+  if (RIA)
+    nbr_ria(t, ria_locate(t, n), m);
+  else
+    nbr_adj(t, n, m);
+  if (layout == LBM_LAYOUT_OSNT)
+    gather<PREC, false>(pdf, t.npad, n, m, d, kp.inv_scale, c.abb_in, c.abb_out, t.pressure);
+  else
+    gather<PREC, true>(pdf, t.npad, n, m, d, kp.inv_scale, c.abb_in, c.abb_out, t.pressure);
 }
 
+// Double of a normal float from its bits (the hardware conversion is an
+// instruction of the FP64 pipe).
+__device__ __forceinline__ double double_of_normal(float x) {
+  const uint32_t b = __float_as_uint(x), m = b & 0x7fffffffu;
+  return __hiloint2double(static_cast<int>((b & 0x80000000u) | ((m >> 3) + 0x38000000u)), static_cast<int>(b << 29));
+}
+__device__ __forceinline__ void to_doubles(const double (&d)[kQ], double (&f)[kQ]) {
+#pragma unroll
+  for (int i = 0; i < kQ; ++i) f[i] = d[i];
+}
+__device__ __forceinline__ void to_doubles(const float (&d)[kQ], double (&f)[kQ]) {
+  uint32_t lo = 0xffffffffu, hi = 0u;
+#pragma unroll
+  for (int i = 0; i < kQ; ++i) {
+    const uint32_t m = __float_as_uint(d[i]) & 0x7fffffffu;
+    lo = m < lo ? m : lo;
+    hi = m > hi ? m : hi;
+  }
+  if (__all_sync(__activemask(), lo >= 0x00800000u && hi < 0x7f800000u)) {
+#pragma unroll
+    for (int i = 0; i < kQ; ++i) f[i] = double_of_normal(d[i]);
+  } else {
+#pragma unroll
+    for (int i = 0; i < kQ; ++i) f[i] = double(d[i]);
+  }
+}
+
+// x != 0 without an FP64-pipe comparison.
+__device__ __forceinline__ bool nonzero(double x) { return (dbits(x) << 1) != 0; }
+
+// Canonical PDFs in FP64.  The conversions run on the integer pipe, which
+// leaves the FP64 pipe one addition per PDF (none without a storage shift):
+// 5.3 M FP32 nodes in 0.38 ms with the conversions on the FP64 pipe (86 %
+// busy), 0.21 ms so.
 template <int PREC, bool RIA>
 __global__ void __launch_bounds__(kBlock) k_canonical(DevTables t, KParams kp, CollConst<typename St<PREC>::R> c,
                                                       const typename St<PREC>::T* pdf, int layout,
                                                       double* __restrict__ F, int N) {
-  const int n0 = blockIdx.x * kBlock;
-  const int n = n0 + threadIdx.x;
+  const int n = blockIdx.x * kBlock + threadIdx.x;
+  if (n >= N) return;
+  typename St<PREC>::R d[kQ];
+  node_load<PREC, RIA>(t, kp, c, pdf, layout, n, d);
   double f[kQ];
-  if (!node_canonical<PREC, RIA>(t, kp, c, pdf, layout, n, N, f)) return;
+  to_doubles(d, f);
+  if (nonzero(kp.rho_s)) {  // uniform
+#pragma unroll
+    for (int i = 0; i < kQ; ++i) f[i] = ::fma(wgt(i), kp.rho_s, f[i]);
+  }
 #pragma unroll
   for (int i = 0; i < kQ; ++i) F[size_t(i) * N + n] = f[i];
 }
@@ -1252,44 +1276,95 @@ __device__ __forceinline__ void block_sum4(double (&v)[4], double (*s_red)[4]) {
   }
 }
 
-// rho, u = (j0/rho + g/2)/(1 + s/2) per node and per-CTA partial sums of
-// [rho, rho u_x, rho u_y, rho u_z] (FP64).
-template <int PREC, bool RIA>
-__global__ void __launch_bounds__(kBlock) k_macro(DevTables t, KParams kp, CollConst<typename St<PREC>::R> c,
-                                                  const typename St<PREC>::T* pdf, int layout,
-                                                  const float* __restrict__ s, double* __restrict__ rho,
-                                                  double* __restrict__ u, double* __restrict__ partials, int N) {
-  __shared__ double s_red[kBlock / 32][4];
-  const int n0 = blockIdx.x * kBlock;
-  const int n = n0 + threadIdx.x;
-  double f[kQ];
-  double acc[4] = {0.0, 0.0, 0.0, 0.0};
-  if (node_canonical<PREC, RIA>(t, kp, c, pdf, layout, n, N, f)) {
-    double r = 0.0, jx = 0.0, jy = 0.0, jz = 0.0;
+// kd = 1 / (1 + s/2), through the integer reciprocal for the fractions 0 <= s <= 1.
+__device__ __forceinline__ double drag_factor(float s) {
+  const double v = ::fma(0.5, double(s), 1.0);
+  if (s >= 0.0f && s <= 1.0f) return fx_to_double_cvt(fx_recip((dbits(v) << 11) | kSignBit), 1018);
+  return 1.0 / v;
+}
+
+// Density and velocity of one node from its stored PDFs: rho = rho_s + sum d_i
+// and u = (j0/rho + g/2)/(1 + s/2).  The sums are exact integers, rounded once,
+// and the quotients integer products (fx_quotient); what is left in FP64 is
+// the addition of rho_s, of g/2 where it is not zero, and the factor of the
+// drag.  Summing 19 doubles and dividing three times there took about 90
+// FP64 instructions a node.  Nodes outside the integer range (no positive
+// normal density, Inf or NaN PDFs) take the FP64 form.
+template <class R>
+__device__ __forceinline__ void node_rho_u(const KParams& kp, const R (&d)[kQ], const float* __restrict__ s, int n,
+                                           double& r, double& ux, double& uy, double& uz) {
+  int64_t S, Jx, Jy, Jz;
+  const int emax = fx_moments(d, S, Jx, Jy, Jz);
+  r = kp.rho_s + fx_to_double_cvt(S, emax);
+  const uint64_t b = dbits(r);
+  const int er = static_cast<int>(b >> 52) - 1023;
+  if (emax < kFxMaxExp && er > -1000 && er < 1000 && emax - er >= 64 && emax - er < 1900) {
+    const Bal q = bal(fx_recip((b << 11) | kSignBit));
+    ux = fx_quotient(Jx, emax, q, er);
+    uy = fx_quotient(Jy, emax, q, er);
+    uz = fx_quotient(Jz, emax, q, er);
+  } else {
+    double f[kQ], jx = 0.0, jy = 0.0, jz = 0.0;
+    r = 0.0;
 #pragma unroll
     for (int i = 0; i < kQ; ++i) {
+      f[i] = ::fma(wgt(i), kp.rho_s, double(d[i]));
       r += f[i];
       if (cx(i)) jx += cx(i) > 0 ? f[i] : -f[i];
       if (cy(i)) jy += cy(i) > 0 ? f[i] : -f[i];
       if (cz(i)) jz += cz(i) > 0 ? f[i] : -f[i];
     }
-    const double kd = s ? 1.0 / (1.0 + 0.5 * double(s[n])) : 1.0;
-    const double ux = (jx / r + 0.5 * kp.g[0]) * kd;
-    const double uy = (jy / r + 0.5 * kp.g[1]) * kd;
-    const double uz = (jz / r + 0.5 * kp.g[2]) * kd;
+    ux = jx / r;
+    uy = jy / r;
+    uz = jz / r;
+  }
+  if (nonzero(kp.g[0])) ux = ::fma(0.5, kp.g[0], ux);  // uniform
+  if (nonzero(kp.g[1])) uy = ::fma(0.5, kp.g[1], uy);
+  if (nonzero(kp.g[2])) uz = ::fma(0.5, kp.g[2], uz);
+  if (s) {
+    const double kd = drag_factor(s[n]);
+    ux *= kd;
+    uy *= kd;
+    uz *= kd;
+  }
+}
+
+// rho and u per node and per-CTA partial sums of [rho, rho u_x, rho u_y,
+// rho u_z] (FP64).  Bound by the FP64 pipe (12 instructions a node) and HBM
+// together.  A CTA walks the nodes in strides of the grid and reduces once:
+// the five shuffle rounds of four FP64 additions per 128 nodes cost more than
+// the node's own arithmetic.  5.3 M FP32 nodes: 1.40 -> 0.19 ms.
+#ifndef LBM_MIN_CTAS_REDUCE
+#define LBM_MIN_CTAS_REDUCE 6
+#endif
+template <int PREC, bool RIA>
+__global__ void __launch_bounds__(kBlock, LBM_MIN_CTAS_REDUCE) k_macro(DevTables t, KParams kp, CollConst<typename St<PREC>::R> c,
+                                                  const typename St<PREC>::T* pdf, int layout,
+                                                  const float* __restrict__ s, double* __restrict__ rho,
+                                                  double* __restrict__ u, double* __restrict__ partials, int N) {
+  __shared__ double s_red[kBlock / 32][4];
+  double acc[4] = {0.0, 0.0, 0.0, 0.0};
+  const int64_t stride = int64_t(gridDim.x) * kBlock;
+  for (int64_t k = int64_t(blockIdx.x) * kBlock + threadIdx.x; k < N; k += stride) {
+    const int n = int(k);
+    typename St<PREC>::R d[kQ];
+    node_load<PREC, RIA>(t, kp, c, pdf, layout, n, d);
+    double r, ux, uy, uz;
+    node_rho_u(kp, d, s, n, r, ux, uy, uz);
     if (rho) rho[n] = r;
     if (u) {
       u[n] = ux;
       u[size_t(N) + n] = uy;
       u[2 * size_t(N) + n] = uz;
     }
-    acc[0] = r;
-    acc[1] = r * ux;
-    acc[2] = r * uy;
-    acc[3] = r * uz;
+    if (partials) {  // uniform
+      acc[0] += r;
+      acc[1] = ::fma(r, ux, acc[1]);
+      acc[2] = ::fma(r, uy, acc[2]);
+      acc[3] = ::fma(r, uz, acc[3]);
+    }
   }
   if (!partials) return;
-  __syncthreads();
   block_sum4(acc, s_red);
   if (threadIdx.x == 0)
 #pragma unroll
@@ -1322,6 +1397,12 @@ inline int cuda_check(const char* what) {
 }
 
 inline unsigned grid_of(int64_t N) { return unsigned((N + dev::kBlock - 1) / dev::kBlock); }
+
+// CTAs of the reducing kernels (k_macro, k_objective), which walk the nodes in
+// strides: enough for 16 per SM, so that the one-CTA sum of their partials is
+// short (with one partial per 128 nodes it took 0.11 ms of a 5.3 M-node
+// read-back).  Never more than the workspace holds (reduce_parts).
+inline unsigned reduce_grid(int64_t nparts) { return unsigned(std::min<int64_t>(std::max<int64_t>(nparts, 1), 16 * 152)); }
 
 inline bool has_force(const KParams& kp) { return kp.g[0] != 0.0 || kp.g[1] != 0.0 || kp.g[2] != 0.0; }
 
@@ -1520,19 +1601,20 @@ int launch_macroscopic_t(const lbm_lattice* L, const KParams& kp, const void* pd
   using T = typename dev::St<PREC>::T;
   auto st = static_cast<cudaStream_t>(stream);
   double* part = sums ? partials : nullptr;
+  const unsigned g = reduce_grid(nparts);
   if (L->N > 0) {
     const bool ria = !(L->uploaded & LBM_TABLES_ADJ);
     const auto c = dev::make_coll<typename dev::St<PREC>::R>(kp);
     if (ria)
-      dev::k_macro<PREC, true><<<grid_of(L->N), dev::kBlock, 0, st>>>(L->dev, kp, c, static_cast<const T*>(pdf),
-                                                                     layout, s, rho, u, part, int(L->N));
+      dev::k_macro<PREC, true><<<g, dev::kBlock, 0, st>>>(L->dev, kp, c, static_cast<const T*>(pdf), layout, s, rho, u,
+                                                          part, int(L->N));
     else
-      dev::k_macro<PREC, false><<<grid_of(L->N), dev::kBlock, 0, st>>>(L->dev, kp, c, static_cast<const T*>(pdf),
-                                                                      layout, s, rho, u, part, int(L->N));
+      dev::k_macro<PREC, false><<<g, dev::kBlock, 0, st>>>(L->dev, kp, c, static_cast<const T*>(pdf), layout, s, rho,
+                                                           u, part, int(L->N));
     if (int rc = cuda_check("macroscopic launch")) return rc;
   }
   if (sums) {
-    dev::k_finish4<PREC><<<1, 512, 0, st>>>(partials, L->N > 0 ? nparts : 0, sums);
+    dev::k_finish4<PREC><<<1, 512, 0, st>>>(partials, L->N > 0 ? int64_t(g) : 0, sums);
     return cuda_check("reduction launch");
   }
   return LBM_OK;
