@@ -372,6 +372,16 @@ LBM_API int lbm_fx_pairs_host(const double* d, const double* terms, int64_t n, d
 LBM_API int lbm_fx_collide_host(const double* d, const float* s, int64_t n, const lbm_params* params, double* out,
                                 int* ok);
 
+/* Host image of the LBM_F64 adjoint step's arithmetic in fixed point.  d: host
+ * double [n][19], forward PDFs F_n in params' storage; mu: host double [n][19],
+ * the gathered adjoint vector; s: host float [n] or NULL.  lam: host double
+ * [n][19], the adjoint PDFs; grad: host double [n], the nodes' dJ/ds terms; ok:
+ * host int [n], 0 where a node is outside the fixed-point range (its results are
+ * then 0; the kernel takes the FP64 form there).  LBM_ERR_ARG for bad params,
+ * NULL pointers or n < 0. */
+LBM_API int lbm_fx_adjoint_host(const double* d, const double* mu, const float* s, int64_t n, const lbm_params* params,
+                                double* lam, double* grad, int* ok);
+
 /* Check the host tables: entries in range, adjacency reciprocity
  * (adj[i][n] = m >= 0  <=>  adj[inv i][m] = n), run table decoding back to the
  * adjacency list exactly, runs sorted and covering [0, N).  Returns

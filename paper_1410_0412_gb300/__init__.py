@@ -620,6 +620,31 @@ def lbm_fx_collide_host(d, params, s=None):
     return out, ok.astype(bool)
 
 
+def lbm_fx_adjoint_host(d, mu, params, s=None):
+    """Host image of the FP64 adjoint step's arithmetic in fixed point (``lbm_fx_adjoint_host``).
+
+    d, mu: [n, 19] forward PDFs (in the storage of ``params``) and gathered
+    adjoint values; s: [n] Brinkman solid fractions or None.  Returns (lam
+    [n, 19], grad [n], ok [n]).
+    """
+    import numpy as np
+    a = np.ascontiguousarray(np.asarray(d, dtype=np.float64))
+    m = np.ascontiguousarray(np.asarray(mu, dtype=np.float64))
+    if a.ndim != 2 or a.shape[1] != 19 or m.shape != a.shape:
+        raise ValueError("d and mu must have shape [n, 19]")
+    sf = None
+    if s is not None:
+        sf = np.ascontiguousarray(np.asarray(s, dtype=np.float32))
+        if sf.shape != (a.shape[0],):
+            raise ValueError("s must have shape [n]")
+    lam, grad = np.empty_like(a), np.empty(a.shape[0])
+    ok = np.empty(a.shape[0], dtype=np.int32)
+    check(_lib.load().lbm_fx_adjoint_host(a.ctypes.data, m.ctypes.data, None if sf is None else sf.ctypes.data,
+                                          a.shape[0], ctypes.byref(params.c()), lam.ctypes.data, grad.ctypes.data,
+                                          ok.ctypes.data), "lbm_fx_adjoint_host")
+    return lam, grad, ok.astype(bool)
+
+
 def lbm_bandwidth_kernel(kind, dst, src=None, arrays=1, stream=None):
     """One launch of the CNT-kA (kind 0, copy src -> dst with streaming stores) or
     U-kA (kind 1, update dst in place) bandwidth kernel over ``arrays`` equal
@@ -875,7 +900,7 @@ __all__ = [
     "PartitionedSolver", "lbm_halo_exchange", "lbm_partition_run_aa", "lbm_partition_run_osnt",
     "lbm_objective_flux", "lbm_adjoint_step", "lbm_ckpt_workspace_bytes", "lbm_flux_forward", "lbm_flux_backward",
     "flux_objective", "new_adjoint", "lbm_macroscopic_noalloc", "lbm_check_finite", "lbm_bandwidth_kernel", "lbm_fp64_peak_kernel",
-    "lbm_exact_moments_host", "lbm_fx_pairs_host", "lbm_fx_collide_host",
+    "lbm_exact_moments_host", "lbm_fx_pairs_host", "lbm_fx_collide_host", "lbm_fx_adjoint_host",
     "State", "FluxObjective",
 ]
 

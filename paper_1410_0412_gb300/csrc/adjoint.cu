@@ -36,6 +36,7 @@ template <class R> struct AdjConst {
   R nk18ap, k6ap;           // -18 a+, 6 a+
   R k3am, nk3am;            // 3 a-, -3 a-
   bool gx;                  // the body force points along x (g_y = g_z = 0)
+  FxAdj fx;                 // constants of the FP64 step in fixed point (exact64.cuh)
 };
 
 // Storage of the adjoint arrays: IEEE double for both FP64 paths (the
@@ -89,6 +90,7 @@ template <class R> AdjConst<R> make_adj(const KParams& kp) {
   c.k3am = R(3.0 * am);
   c.nk3am = R(-3.0 * am);
   c.gx = kp.g[1] == 0.0 && kp.g[2] == 0.0;
+  c.fx = make_fx_adj(kp.lp, kp.lm, kp.g);
   return c;
 }
 
@@ -99,28 +101,25 @@ template <class R> AdjConst<R> make_adj(const KParams& kp) {
 // w0 mu_0 for M0).  FP64 forms those sums exactly in fixed point on the
 // integer pipe (exact64.cuh) and rounds each once; P_k is converted only when
 // the caller needs it (l+ != 1).
-// NEED_PD: convert P and D to R (the FP64 pair update needs them; the
-// fixed-point one reads the integers Pi, Di at the scale emax instead).
-template <class R, bool NEED_P, bool NEED_PD = true>
+template <class R, bool NEED_P>
 __device__ __forceinline__ void adj_moments(const R (&mu)[kQ], const AdjConst<R>& c, R (&P)[10], R (&D)[10], R& M0,
-                                            R& M1x, R& M1y, R& M1z, R& Mxx, R& Myy, R& Mzz, R& Mxy, R& Mxz,
-                                            R& Myz, int64_t (&Pi)[10], int64_t (&Di)[10], int& emax) {
+                                            R& M1x, R& M1y, R& M1z, R& Mxx, R& Myy, R& Mzz, R& Mxy, R& Mxz, R& Myz) {
   using ::fma;
   const R w2 = c.w[2];
   if constexpr (std::is_same<R, double>::value) {
     uint64_t b[kQ];
 #pragma unroll
     for (int i = 0; i < kQ; ++i) b[i] = dbits(mu[i]);
-    emax = fx_scale(b);
-    int64_t f[kQ];
+    const int emax = fx_scale(b);
+    int64_t f[kQ], Pi[10], Di[10];
 #pragma unroll
     for (int i = 0; i < kQ; ++i) f[i] = fx_of(b[i], emax);
 #pragma unroll
     for (int k = 1; k <= 9; ++k) {
       Pi[k] = f[2 * k - 1] + f[2 * k];
       Di[k] = f[2 * k - 1] - f[2 * k];
-      if (NEED_PD && NEED_P) P[k] = fx_to_double(Pi[k], emax);
-      if (NEED_PD) D[k] = fx_to_double(Di[k], emax);
+      if (NEED_P) P[k] = fx_to_double(Pi[k], emax);
+      D[k] = fx_to_double(Di[k], emax);
     }
     // every integer sum below has at most 24 terms of magnitude < 2^58
     const int64_t A1 = Pi[1] + Pi[2] + Pi[3];
@@ -160,8 +159,18 @@ __device__ __forceinline__ void adj_moments(const R (&mu)[kQ], const AdjConst<R>
 // One adjoint step.  G: OS-NT grid at step n (its pull gather is F_n).
 // lam_next / lam: adjoint of the canonical states F_{n+1} / F_n, layout [19][Npad].
 // LP1: l+ = 1 (FP64-storage paths), where (1 - l+)/2 = 1 - l+ = 0.
+#ifndef LBM_MIN_CTAS_ADJ
+#define LBM_MIN_CTAS_ADJ 8
+#endif
+// Resident CTAs per SM.  FP64 at 3 / 4 / 5 / 6: 13.43 / 12.80 / 13.11 / 14.08 ms
+// for a checkpointed gradient of 60 steps on 0.77 M nodes (above 4 it spills).
+// FP32 and FP16 wait for the gathers: 6 / 7 / 8 / 9 gave 19.67 / 19.61 / 18.99 /
+// 18.98 ms for 100 steps on the 128^3 box.
+template <int PREC> struct MinCtasAdj { static constexpr int value = LBM_MIN_CTAS_ADJ; };
+template <> struct MinCtasAdj<LBM_F64> { static constexpr int value = 4; };
+template <> struct MinCtasAdj<LBM_F64_DF> { static constexpr int value = 3; };
 template <int PREC, bool RIA, bool DRAG, bool LP1 = false>
-__global__ void __launch_bounds__(kBlock) k_adjoint(DevTables t, KParams kp, CollConst<typename St<PREC>::R> cc,
+__global__ void __launch_bounds__(kBlock, MinCtasAdj<PREC>::value) k_adjoint(DevTables t, KParams kp, CollConst<typename St<PREC>::R> cc,
                                                     AdjConst<typename St<PREC>::R> c,
                                                     const typename St<PREC>::T* __restrict__ G,
                                                     const typename Lam<PREC>::T* __restrict__ lam_next,
@@ -209,10 +218,56 @@ __global__ void __launch_bounds__(kBlock) k_adjoint(DevTables t, KParams kp, Col
     }
   }
   R sa[10], da[10], drho, jx, jy, jz;
-  moments<R, false>(d, sa, da, drho, jx, jy, jz);
+  const R sn = DRAG ? R(__ldg(s + n)) : R(0);
+  if constexpr (std::is_same<R, double>::value) {
+    // FP64: the whole step in fixed point (fx_adjoint) where every node of the
+    // warp is in range.  It was bound by the FP64 pipe (about 160 instructions
+    // a node, 80 % busy, DRAM 28 %): 0.175 ms for 0.77 M nodes with drag; now
+    // 0.102 ms.
+    int64_t S, Jx, Jy, Jz, Sk[10], Dk[10];
+    const int ef = fx_moments<false>(d, Sk, Dk, S, Jx, Jy, Jz, 0, nullptr, cc.fx.emin);
+    uint64_t b[kQ];
+#pragma unroll
+    for (int i = 0; i < kQ; ++i) b[i] = dbits(mu[i]);
+    const int em = fx_scale(b, kFxMinExpAdj);
+    int64_t Pi[10], Di[10];
+    const int64_t m0 = fx_of(b[0], em);
+#pragma unroll
+    for (int k = 1; k <= 9; ++k) {
+      const int64_t fa = fx_of(b[2 * k - 1], em), fb = fx_of(b[2 * k], em);
+      Pi[k] = fa + fb;
+      Di[k] = fa - fb;
+    }
+    FxAdjOut o;
+    const bool ok = fx_adjoint<DRAG>(cc.fx, c.fx, ef, S, Jx, Jy, Jz, sn, em, m0, Pi, Di, o);
+    if (__all_sync(__activemask(), ok)) {
+      if (grad_s) {
+        const double rho = c.rho_s + fx_to_double_cvt(S, ef);
+        grad_s[n] = ::fma(rho, fx_to_double_cvt(o.gs, o.eg), grad_s[n]);
+      }
+      // lambda_a,b = e +- o, e = A + qp P_k, o = qm D_k + c_a.B; rest: A + (1 - l+) mu_0
+      const Bal qm = bal(cc.fx.qm), qp = bal(cc.fx.qp);
+      L::st(lam + n, fx_to_double_cvt(LP1 ? o.A : o.A + mulhi_q64(qp, bal(2 * m0)), em));
+#pragma unroll
+      for (int k = 1; k <= 9; ++k) {
+        const int64_t Bc = k == 1 ? o.Bx : k == 2 ? o.By : k == 3 ? o.Bz : k == 4 ? o.Bx + o.By : k == 5 ? o.Bx - o.By
+                         : k == 6 ? o.Bx + o.Bz : k == 7 ? o.Bx - o.Bz : k == 8 ? o.By + o.Bz : o.By - o.Bz;
+        const int64_t e = LP1 ? o.A : o.A + mulhi_q64(qp, bal(Pi[k]));
+        const int64_t odd = mulhi_q64(qm, bal(Di[k])) + Bc;
+        L::st(lam + at(2 * k - 1, t.npad, n), fx_to_double_cvt(e + odd, em));
+        L::st(lam + at(2 * k, t.npad, n), fx_to_double_cvt(e - odd, em));
+      }
+      return;
+    }
+    drho = ef < kFxMaxExp ? fx_to_double(S, ef) : dfrom(0x7ff8000000000000ull);
+    jx = fx_to_double(Jx, ef);
+    jy = fx_to_double(Jy, ef);
+    jz = fx_to_double(Jz, ef);
+  } else {
+    moments<R, false>(d, sa, da, drho, jx, jy, jz);
+  }
   const R rho = c.rho_s + drho;
   const R irho = recip(rho);
-  const R sn = DRAG ? R(__ldg(s + n)) : R(0);
   const R kd = DRAG ? recip(R(1) + halve(sn)) : R(1);
   R ux = fma(jx, irho, c.hg[0]), uy = fma(jy, irho, c.hg[1]), uz = fma(jz, irho, c.hg[2]);
   if (DRAG) {
@@ -221,10 +276,7 @@ __global__ void __launch_bounds__(kBlock) k_adjoint(DevTables t, KParams kp, Col
     uz *= kd;
   }
   R P[10], D[10], M0, M1x, M1y, M1z, Mxx, Myy, Mzz, Mxy, Mxz, Myz;
-  int64_t Pi[10], Di[10];
-  int emax_mu = 0;
-  constexpr bool kFxOut = std::is_same<R, double>::value;  // the fixed-point pair update below
-  adj_moments<R, !LP1, !kFxOut>(mu, c, P, D, M0, M1x, M1y, M1z, Mxx, Myy, Mzz, Mxy, Mxz, Myz, Pi, Di, emax_mu);
+  adj_moments<R, !LP1>(mu, c, P, D, M0, M1x, M1y, M1z, Mxx, Myy, Mzz, Mxy, Mxz, Myz);
   const R M2ux = fma(Mxx, ux, fma(Mxy, uy, Mxz * uz));
   const R M2uy = fma(Mxy, ux, fma(Myy, uy, Myz * uz));
   const R M2uz = fma(Mxz, ux, fma(Myz, uy, Mzz * uz));
@@ -278,40 +330,6 @@ __global__ void __launch_bounds__(kBlock) k_adjoint(DevTables t, KParams kp, Col
     grad_s[n] += L::to_double(gs);
   }
   L::st(lam + n, LP1 ? A : fma(c.omlp, mu[0], A));
-  if constexpr (kFxOut) {
-    // The pair update lambda_a,b = e +- o, e = A + qp P_k, o = qm D_k + c_a.B, in
-    // 64-bit fixed point at one bit finer than the adjoint moments' scale:
-    // P_k and D_k enter exactly, A and B truncated, the products floored,
-    // each output rounded once.  |mu_i| < 2 B_mu gives |D_k|, |P_k| < 4 B_mu;
-    // with |A|, |B_a| < 4 B_mu (checked) every value stays below 16 B_mu, half
-    // the int64 range at this scale.  Otherwise the warp takes the FP64 update.
-    constexpr int kxa = 1;
-    const bool ok = emax_mu < kFxMaxExp && dexp(A) <= emax_mu + 1 && dexp(Bx) <= emax_mu + 1 &&
-                    dexp(By) <= emax_mu + 1 && dexp(Bz) <= emax_mu + 1;
-    if (__all_sync(__activemask(), ok)) {
-      const int es = emax_mu - kxa;
-      const int64_t Af = fx_of(dbits(A), es);
-      const int64_t Bxf = fx_of(dbits(Bx), es), Byf = fx_of(dbits(By), es), Bzf = fx_of(dbits(Bz), es);
-#pragma unroll
-      for (int k = 1; k <= 9; ++k) {
-        const int a = 2 * k - 1;
-        const int64_t Bc = k == 1 ? Bxf : k == 2 ? Byf : k == 3 ? Bzf : k == 4 ? Bxf + Byf : k == 5 ? Bxf - Byf
-                         : k == 6 ? Bxf + Bzf : k == 7 ? Bxf - Bzf : k == 8 ? Byf + Bzf : Byf - Bzf;
-        const int64_t Df = static_cast<int64_t>(static_cast<uint64_t>(Di[k]) << kxa);
-        int64_t e = Af;
-        if (!LP1) e += mulhi_q64(cc.fx.qp, static_cast<int64_t>(static_cast<uint64_t>(Pi[k]) << kxa));
-        const int64_t o = mulhi_q64(cc.fx.qm, Df) + Bc;
-        L::st(lam + at(a, t.npad, n), fx_to_double(e + o, es));
-        L::st(lam + at(a + 1, t.npad, n), fx_to_double(e - o, es));
-      }
-      return;
-    }
-#pragma unroll
-    for (int k = 1; k <= 9; ++k) {
-      if (!LP1) P[k] = fx_to_double(Pi[k], emax_mu);
-      D[k] = fx_to_double(Di[k], emax_mu);
-    }
-  }
 #pragma unroll
   for (int k = 1; k <= 9; ++k) {
     const int a = 2 * k - 1;

@@ -440,6 +440,50 @@ int lbm_fx_collide_host(const double* d, const float* s, int64_t n, const lbm_pa
   return LBM_OK;
 }
 
+int lbm_fx_adjoint_host(const double* d, const double* mu, const float* s, int64_t n, const lbm_params* params,
+                        double* lam, double* grad, int* ok) {
+  KParams kp;
+  if (int rc = make_kparams(params, LBM_F64, &kp)) return rc;
+  if (n < 0 || (n > 0 && (!d || !mu || !lam || !grad || !ok)))
+    return set_error(LBM_ERR_ARG, "d, mu, lam, grad or ok is NULL, or n < 0");
+  const dev::FxColl c = dev::make_fx_coll(kp.lp, kp.lm, kp.g, kp.rho_s);
+  const dev::FxAdj a = dev::make_fx_adj(kp.lp, kp.lm, kp.g);
+  for (int64_t k = 0; k < n; ++k) {
+    double f[19], out[19] = {0.0};
+    std::memcpy(f, d + 19 * k, sizeof f);
+    int64_t Sk[10], Dk[10], S, Jx, Jy, Jz, Pi[10], Di[10];
+    const int ef = dev::fx_moments<false>(f, Sk, Dk, S, Jx, Jy, Jz, 0, nullptr, c.emin);
+    uint64_t b[19];
+    for (int i = 0; i < 19; ++i) b[i] = dev::dbits(mu[19 * k + i]);
+    const int em = dev::fx_scale(b, dev::kFxMinExpAdj);
+    const int64_t m0 = dev::fx_of(b[0], em);
+    for (int q = 1; q <= 9; ++q) {
+      const int64_t fa = dev::fx_of(b[2 * q - 1], em), fb = dev::fx_of(b[2 * q], em);
+      Pi[q] = fa + fb;
+      Di[q] = fa - fb;
+    }
+    dev::FxAdjOut o;
+    ok[k] = s ? dev::fx_adjoint<true>(c, a, ef, S, Jx, Jy, Jz, double(s[k]), em, m0, Pi, Di, o)
+              : dev::fx_adjoint<false>(c, a, ef, S, Jx, Jy, Jz, 0.0, em, m0, Pi, Di, o);
+    grad[k] = 0.0;
+    if (ok[k]) {
+      grad[k] = (kp.rho_s + dev::fx_to_double_cvt(S, ef)) * dev::fx_to_double_cvt(o.gs, o.eg);
+      out[0] = dev::fx_to_double_cvt(o.A + dev::mulhi_q64(c.qp, 2 * m0), em);
+      for (int q = 1; q <= 9; ++q) {
+        const int64_t B[3] = {o.Bx, o.By, o.Bz};
+        int64_t Bc = 0;
+        for (int x = 0; x < 3; ++x)
+          Bc += B[x] * (x == 0 ? kCX[2 * q - 1] : x == 1 ? kCY[2 * q - 1] : kCZ[2 * q - 1]);
+        const int64_t e = o.A + dev::mulhi_q64(c.qp, Pi[q]), odd = dev::mulhi_q64(c.qm, Di[q]) + Bc;
+        out[2 * q - 1] = dev::fx_to_double_cvt(e + odd, em);
+        out[2 * q] = dev::fx_to_double_cvt(e - odd, em);
+      }
+    }
+    std::memcpy(lam + 19 * k, out, sizeof out);
+  }
+  return LBM_OK;
+}
+
 int lbm_validate_tables(const lbm_lattice* L) {
   if (int rc = check_lat(L)) return rc;
   try {

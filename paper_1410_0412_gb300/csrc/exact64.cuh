@@ -698,5 +698,181 @@ template <bool LP1> __host__ __device__ __forceinline__ int fx_kx(const FxColl& 
   return c.shift ? 0 : (LP1 && near) ? 4 : 2;
 }
 
+// ---- the adjoint step in fixed point ----------------------------------------------------
+//
+// With the weighted moments M0, M1, M2 of the gathered adjoint vector mu and
+// K = 9 M2 - 3 M0, the terms of the adjoint collision (adjoint.cu) collapse to
+//   X = K u, Y = K g, P = dPsi/du = (l+ - 2 a+ s) X + a+ Y + 3 (l- - a- s) M1,
+//   A = l+ M0 - (l+/2 - a+ s) u.X + 3 a- M1.g + kd P.g / 2,   B = kd P,
+//   dJ/ds / rho = -a+ u.X - 3 a- M1.u - kd P.u / 2,
+// all linear in mu: products of the integer moments (w = 1/36 and 1/18 make them
+// integers over 36) with u, g and per-launch constants as Q64 fractions.  u is
+// kept normalised, u = u' 2^-p with 1/32 < |u'| < 0.28 for its largest
+// component, and what enters dJ/ds only
+// through u (K u, M1.u, Y.u) is carried p bits finer than mu, so that the
+// gradient of a slow flow keeps its relative accuracy.
+//
+// Bounds: |mu_i| < 2^58 at mu's scale, so |36 M0| / 2 < 18, |36 M1| < 12,
+// |36 M2_aa| < 12, |36 M2_ab| < 4 and |4 K_aa| < 24 (times 2^58 each); |J 2^z| <
+// 2^62, |G| < 2^59 and p >= 0 give |u'| < 0.28 2^64 and |4 X| < 9 2^58; |g_a| < 2^-6
+// (checked on the host) makes Y small; then |P| < 7 2^58, |A| < 5 2^58 and every
+// output is below 2^62.  Each product is within 3/4 of a unit.
+struct FxAdj {
+  int64_t l18;           // l+/18 as a Q64 fraction, and so the next
+  int64_t c1, c1s;       // l+/4, a+/2  (c1 - c1s s)
+  int64_t c3, c3s;       // l-/12, a-/12 (c3 - c3s s)
+  int64_t ap4;           // a+/4
+  int64_t g[3];
+  bool ok;               // the force is in range
+};
+
+inline FxAdj make_fx_adj(double lp, double lm, const double (&g)[3]) {
+  FxAdj c;
+  const double ap = 1.0 - lp / 2, am = 1.0 - lm / 2;
+  c.l18 = q64_of(lp / 18.0);
+  c.c1 = q64_of(lp / 4.0);
+  c.c1s = q64_of(ap / 2.0);
+  c.c3 = q64_of(lm / 12.0);
+  c.c3s = q64_of(am / 12.0);
+  c.ap4 = q64_of(ap / 4.0);
+  c.ok = true;
+  for (int a = 0; a < 3; ++a) {
+    c.ok = c.ok && std::fabs(g[a]) < 0.015625;
+    c.g[a] = c.ok ? q64_of(g[a]) : 0;
+  }
+  return c;
+}
+
+// Least moment scale of the adjoint vector: leaves room below it for the finer
+// scale of the gradient (adjoint values below 2^-880 flush to zero).
+constexpr int kFxMinExpAdj = 200;
+
+struct FxAdjOut {
+  int64_t A, Bx, By, Bz;  // at mu's scale
+  int64_t gs;             // dJ/ds / rho at the scale em - p
+  int eg;                 // em - p
+};
+
+// A, B and the gradient term of one node: from the forward moments (S, J at
+// scale ef) and the adjoint pair sums and differences Pi, Di and rest value m0 at
+// scale em.  False where a bound fails (the caller takes the FP64 form).
+template <bool DRAG>
+__host__ __device__ __forceinline__ bool fx_adjoint(const FxColl& c, const FxAdj& a, int ef, int64_t S, int64_t Jx,
+                                                    int64_t Jy, int64_t Jz, double s, int em, int64_t m0,
+                                                    const int64_t (&Pi)[10], const int64_t (&Di)[10], FxAdjOut& o) {
+  // rho = D 2^(er - 63)
+  uint64_t D;
+  int er;
+  bool ok = a.ok && ef < kFxMaxExp && em < kFxMaxExp;
+  if (c.shift) {  // uniform
+    const uint64_t b = dbits(c.rho_s + fx_to_double_cvt(S, ef));
+    D = (b << 11) | kSignBit;
+    er = static_cast<int>(b >> 52) - 1023;
+    ok = ok && er > -1000 && er < 1000;
+  } else {
+    const int lz = clz64(static_cast<uint64_t>(S));
+    ok = ok && S > 0;
+    D = (static_cast<uint64_t>(S) << (lz & 63)) | kSignBit;
+    er = ef - 1017 - lz;
+  }
+  // q = rho u at z bits below the forward scale: J 2^z < 2^62, G < 2^59
+  const uint64_t mj = static_cast<uint64_t>((Jx ^ (Jx >> 63)) | (Jy ^ (Jy >> 63)) | (Jz ^ (Jz >> 63)));
+  int z = mj ? clz64(mj) - 2 : 4096;
+  const int zg = ef - 1023 - er;
+  z = zg - c.ge[0] < z ? zg - c.ge[0] : z;
+  if (!c.gx) {  // uniform
+    z = zg - c.ge[1] < z ? zg - c.ge[1] : z;
+    z = zg - c.ge[2] < z ? zg - c.ge[2] : z;
+  }
+  ok = ok && z >= 0;
+  const Bal Dh = bal(static_cast<int64_t>(D >> 2)), r = bal(fx_recip(D));
+  const int s0 = ef - z - 1020 - er;
+  const int shx = s0 - c.ge[0];
+  int64_t qx = static_cast<int64_t>(static_cast<uint64_t>(Jx) << (z & 63)) +
+               (mulhi_q64(bal(c.gm[0] >> 1), Dh) >> (((shx > 64 ? 64 : shx) - 1) & 63));
+  int64_t qy = static_cast<int64_t>(static_cast<uint64_t>(Jy) << (z & 63));
+  int64_t qz = static_cast<int64_t>(static_cast<uint64_t>(Jz) << (z & 63));
+  if (!c.gx) {  // uniform
+    const int shy = s0 - c.ge[1], shz = s0 - c.ge[2];
+    qy += mulhi_q64(bal(c.gm[1] >> 1), Dh) >> (((shy > 64 ? 64 : shy) - 1) & 63);
+    qz += mulhi_q64(bal(c.gm[2] >> 1), Dh) >> (((shz > 64 ? 64 : shz) - 1) & 63);
+  }
+  Bal kd = Bal{1 << 30, 0};  // Q62
+  int64_t c1 = a.c1, c3 = a.c3;
+  if (DRAG) {
+    const uint64_t b = dbits(s);
+    ok = ok && b <= 0x3ff0000000000000ull;  // 0 <= s <= 1
+    const int e = 1023 - static_cast<int>(b >> 52);
+    const uint64_t sh2 = e < 64 ? (((b << 11) | kSignBit) >> (e & 63)) : 0u;  // s/2, Q64
+    kd = bal(fx_recip(kSignBit + (sh2 >> 1)));
+    qx = 4 * mulhi_q64(bal(qx), kd);
+    qy = 4 * mulhi_q64(bal(qy), kd);
+    qz = 4 * mulhi_q64(bal(qz), kd);
+    const Bal s4 = bal(static_cast<int64_t>(sh2 >> 1));  // s/4
+    c1 -= 4 * mulhi_q64(bal(a.c1s), s4);
+    c3 -= 4 * mulhi_q64(bal(a.c3s), s4);
+  }
+  // u' = mulhi(q, r) 4, u = u' 2^-p (Q64)
+  const Bal ux = bal(4 * mulhi_q64(bal(qx), r)), uy = bal(4 * mulhi_q64(bal(qy), r)), uz = bal(4 * mulhi_q64(bal(qz), r));
+  int p = z + 1016 + er - ef;
+  p = (ux.h | ux.l | uy.h | uy.l | uz.h | uz.l) ? p : 0;
+  ok = ok && p >= 0 && em - p >= 64;
+  const int ps = p < 63 ? (p & 63) : 63;
+  auto fine = [&](Bal v) { return bal(((static_cast<int64_t>(v.h) << 32) + v.l) >> ps); };  // Q64 u
+  // moments over 36 (M0 halved) and 4 K
+  const int64_t A1 = Pi[1] + Pi[2] + Pi[3];
+  const int64_t m0h = 6 * m0 + A1 + ((Pi[4] + Pi[5] + Pi[6] + Pi[7] + Pi[8] + Pi[9]) >> 1);
+  const int64_t t0 = 2 * mulhi_q64(int64_t(0x5555555555555555ll), m0h);  // 36 M0 / 3
+  const Bal kxx = bal(2 * Pi[1] + Pi[4] + Pi[5] + Pi[6] + Pi[7] - t0);
+  const Bal kyy = bal(2 * Pi[2] + Pi[4] + Pi[5] + Pi[8] + Pi[9] - t0);
+  const Bal kzz = bal(2 * Pi[3] + Pi[6] + Pi[7] + Pi[8] + Pi[9] - t0);
+  const Bal kxy = bal(Pi[4] - Pi[5]), kxz = bal(Pi[6] - Pi[7]), kyz = bal(Pi[8] - Pi[9]);
+  const Bal nx = bal(2 * Di[1] + Di[4] + Di[5] + Di[6] + Di[7]);
+  const Bal ny = bal(2 * Di[2] + Di[4] - Di[5] + Di[8] + Di[9]);
+  const Bal nz = bal(2 * Di[3] + Di[6] - Di[7] + Di[8] - Di[9]);
+  // 4 X and M1.u (36), p bits finer
+  const int64_t Xx = mulhi_q64(kxx, ux) + mulhi_q64(kxy, uy) + mulhi_q64(kxz, uz);
+  const int64_t Xy = mulhi_q64(kxy, ux) + mulhi_q64(kyy, uy) + mulhi_q64(kyz, uz);
+  const int64_t Xz = mulhi_q64(kxz, ux) + mulhi_q64(kyz, uy) + mulhi_q64(kzz, uz);
+  const int64_t nu = mulhi_q64(nx, ux) + mulhi_q64(ny, uy) + mulhi_q64(nz, uz);
+  const int64_t uX = mulhi_q64(fine(ux), bal(Xx)) + mulhi_q64(fine(uy), bal(Xy)) + mulhi_q64(fine(uz), bal(Xz));
+  // 4 Y, Y.u (p bits finer) and M1.g (36)
+  const Bal gx = bal(a.g[0]);
+  int64_t Yx = mulhi_q64(kxx, gx), Yy = mulhi_q64(kxy, gx), Yz = mulhi_q64(kxz, gx), ng = mulhi_q64(nx, gx);
+  if (!c.gx) {  // uniform
+    const Bal gy = bal(a.g[1]), gz = bal(a.g[2]);
+    Yx += mulhi_q64(kxy, gy) + mulhi_q64(kxz, gz);
+    Yy += mulhi_q64(kyy, gy) + mulhi_q64(kyz, gz);
+    Yz += mulhi_q64(kyz, gy) + mulhi_q64(kzz, gz);
+    ng += mulhi_q64(ny, gy) + mulhi_q64(nz, gz);
+  }
+  const Bal yx = bal(Yx), yy = bal(Yy), yz = bal(Yz);
+  const int64_t uY = mulhi_q64(ux, yx) + mulhi_q64(uy, yy) + mulhi_q64(uz, yz);
+  const Bal b1 = bal(c1), b3 = bal(c3), ap4 = bal(a.ap4);
+  const int64_t Px = mulhi_q64(b1, bal(Xx >> ps)) + mulhi_q64(ap4, yx) + mulhi_q64(b3, nx);
+  const int64_t Py = mulhi_q64(b1, bal(Xy >> ps)) + mulhi_q64(ap4, yy) + mulhi_q64(b3, ny);
+  const int64_t Pz = mulhi_q64(b1, bal(Xz >> ps)) + mulhi_q64(ap4, yz) + mulhi_q64(b3, nz);
+  int64_t Pg = mulhi_q64(gx, bal(Px));
+  if (!c.gx) Pg += mulhi_q64(bal(a.g[1]), bal(Py)) + mulhi_q64(bal(a.g[2]), bal(Pz));
+  o.A = mulhi_q64(bal(a.l18), bal(m0h)) - (mulhi_q64(b1, bal(uX >> ps)) >> 1) + mulhi_q64(bal(a.c3s), bal(ng));
+  if (DRAG) {
+    o.A += 2 * mulhi_q64(kd, bal(Pg));
+    o.Bx = 2 * mulhi_q64(kd, bal(2 * Px));
+    o.By = 2 * mulhi_q64(kd, bal(2 * Py));
+    o.Bz = 2 * mulhi_q64(kd, bal(2 * Pz));
+  } else {
+    o.A += Pg >> 1;
+    o.Bx = Px;
+    o.By = Py;
+    o.Bz = Pz;
+  }
+  // -(a-/12 + kd/2 c3) M1.u - (a+/4 + kd/2 c1) u.X - kd/2 a+/4 u.Y
+  const int64_t h3 = DRAG ? 2 * mulhi_q64(kd, b3) : c3 >> 1, h1 = DRAG ? 2 * mulhi_q64(kd, b1) : c1 >> 1;
+  const int64_t hy = DRAG ? 2 * mulhi_q64(kd, ap4) : a.ap4 >> 1;
+  o.gs = -(mulhi_q64(bal(a.c3s + h3), bal(nu)) + mulhi_q64(bal(a.ap4 + h1), bal(uX)) + mulhi_q64(bal(hy), bal(uY)));
+  o.eg = em - p;
+  return ok;
+}
+
 }  // namespace dev
 }  // namespace lbm
