@@ -169,7 +169,7 @@ __device__ __forceinline__ void adj_moments(const R (&mu)[kQ], const AdjConst<R>
 template <int PREC> struct MinCtasAdj { static constexpr int value = LBM_MIN_CTAS_ADJ; };
 template <> struct MinCtasAdj<LBM_F64> { static constexpr int value = 4; };
 template <> struct MinCtasAdj<LBM_F64_DF> { static constexpr int value = 3; };
-template <int PREC, bool RIA, bool DRAG, bool LP1 = false>
+template <int PREC, int TAB, bool DRAG, bool LP1 = false>
 __global__ void __launch_bounds__(kBlock, MinCtasAdj<PREC>::value) k_adjoint(DevTables t, KParams kp, CollConst<typename St<PREC>::R> cc,
                                                     AdjConst<typename St<PREC>::R> c,
                                                     const typename St<PREC>::T* __restrict__ G,
@@ -185,27 +185,23 @@ __global__ void __launch_bounds__(kBlock, MinCtasAdj<PREC>::value) k_adjoint(Dev
   // the post-collision state is pulled by node m_{inv j} (fluid) or, through a
   // marker, by this node's inv j slot (sign -1 for anti-bounce-back).
   R d[kQ], mu[kQ];
-  if (RIA && t.run_slot) {
-    // Run slots (no pressure faces, the grid below 2^31 slots): the pull slots
-    // of F_n are run_slot_osnt(i, r) + off, and the slot of lambda_{n+1} that
-    // direction j reads is the AA odd table's run_slot(inv j, r) + off.
+  if constexpr (TAB == kSlot) {
+    // Run slots: the pull slots of F_n are run_slot_osnt(i, r) + off, and the
+    // slot of lambda_{n+1} that direction j reads is the AA odd table's
+    // run_slot(inv j, r) + off.
     const RiaCursor cur = ria_locate<kKeepIdx<PREC>>(t, n);
-    unsigned sl[18];
-    run_slots<kKeepIdx<PREC>>(t.run_slot_osnt, t.rpad, cur.r, cur.off, sl);
+    NodeSlots q;
+    run_slots<kKeepIdx<PREC>, false>(t.run_slot_osnt, cur.r, cur.off, q);
     d[0] = St<PREC>::ld(G + n, kp.inv_scale);
 #pragma unroll
-    for (int i = 1; i < kQ; ++i) d[i] = St<PREC>::ld(G + sl[i - 1], kp.inv_scale);
-    run_slots<kKeepIdx<PREC>>(t.run_slot, t.rpad, cur.r, cur.off, sl);
+    for (int i = 1; i < kQ; ++i) d[i] = St<PREC>::ld(G + q.sl[i - 1], kp.inv_scale);
+    run_slots<kKeepIdx<PREC>, false>(t.run_slot, cur.r, cur.off, q);
     mu[0] = L::ld(lam_next + n);
 #pragma unroll
-    for (int j = 1; j < kQ; ++j) mu[j] = L::ld(lam_next + sl[inv(j) - 1]);
+    for (int j = 1; j < kQ; ++j) mu[j] = L::ld(lam_next + q.sl[inv(j) - 1]);
   } else {
     int m[18];
-    if (RIA) {
-      nbr_ria(t, ria_locate(t, n), m);
-    } else {
-      nbr_adj(t, n, m);
-    }
+    node_entries<TAB, true>(t, n, m);
     gather<PREC, false>(G, t.npad, n, m, d, kp.inv_scale, cc.abb_in, cc.abb_out, t.pressure);
     mu[0] = L::ld(lam_next + n);
 #pragma unroll
@@ -461,12 +457,20 @@ int launch_adjoint_t(const lbm_lattice* L, const KParams& kp, const void* G, con
   LT* lo = static_cast<LT*>(lam);
   const int N = int(L->N);
   const bool lp1 = use_lp1<PREC>(kp);
-#define LBM_ADJ(R_, D_) LBM_LAUNCH_LP1(k_adjoint, LBM_TARGS2(R_, D_), (L->dev, kp, cc, ac, Gp, ln, lo, s, grad_s, N))
-  if (s) {
-    if (ria) LBM_ADJ(true, true); else LBM_ADJ(false, true);
-  } else {
-    if (ria) LBM_ADJ(true, false); else LBM_ADJ(false, false);
-  }
+#define LBM_ADJ(T_)                                                                                             \
+  do {                                                                                                          \
+    if (s)                                                                                                      \
+      LBM_LAUNCH_LP1(k_adjoint, LBM_TARGS2(T_, true), (L->dev, kp, cc, ac, Gp, ln, lo, s, grad_s, N));          \
+    else                                                                                                        \
+      LBM_LAUNCH_LP1(k_adjoint, LBM_TARGS2(T_, false), (L->dev, kp, cc, ac, Gp, ln, lo, s, grad_s, N));         \
+  } while (0)
+  // lattices with pressure faces decode the adjacency entries in either table
+  if (!ria)
+    LBM_ADJ(dev::kAdjAny);
+  else if (table_kind(L, ria) == dev::kSlot)
+    LBM_ADJ(dev::kSlot);
+  else
+    LBM_ADJ(dev::kRunAny);
 #undef LBM_ADJ
   return cuda_check("adjoint step launch");
 }

@@ -120,7 +120,7 @@ TableLayout table_layout(const lbm_lattice* L, int which) {
     off = align256(off + size_t(std::max<int64_t>(L->nwarps, 1)) * 4);
     t.warp_head0 = off;
     off = align256(off + size_t(std::max<int64_t>(L->nwarps, 1)) * 4);
-    if (L->run_slot_state == 1) {
+    if (L->run_slot_state > 0) {
       t.run_slot = off;
       t.has_run_slot = true;
       off = align256(off + run_slot_words(L->Rpad) * 4);
@@ -739,7 +739,7 @@ int lbm_export_run_slots(lbm_lattice* L, int kind, int32_t* out, int* available)
   const TableVec& t = kind == 0 ? L->run_slot : L->run_slot_osnt;
   for (int64_t r = 0; r < L->R; ++r)
     for (int j = 0; j < 18; ++j)
-      out[r * 18 + j] = LBM_SLOT_AOS ? t[size_t(r) * kSlotStride + j] : t[size_t(j) * L->Rpad + size_t(r)];
+      out[r * 18 + j] = t[size_t(r) * kSlotStride + j];
   return LBM_OK;
 }
 

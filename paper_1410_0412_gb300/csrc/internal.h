@@ -54,15 +54,12 @@ template <class T> struct NoInitAlloc : std::allocator<T> {
 };
 using TableVec = std::vector<int32_t, NoInitAlloc<int32_t>>;
 
-// Run slot tables (derive_run_slots): run-major, kSlotStride int32 per run
-// (18 slots and 2 words of padding, 80 bytes), so that a thread fetches its
-// run's 18 slots with five aligned vector loads instead of 18 scalar ones.
-// With LBM_SLOT_AOS=0 they are direction-major, [18][Rpad].
-#ifndef LBM_SLOT_AOS
-#define LBM_SLOT_AOS 1
-#endif
+// Run slot tables (derive_run_slots): run-major, kSlotStride int32 per run (18
+// slots and the masks of the directions that meet an inlet and an outlet, 80
+// bytes), so that a thread fetches its run's slots with five aligned vector
+// loads instead of 18 scalar ones.
 constexpr int kSlotStride = 20;
-inline size_t run_slot_words(int64_t Rpad) { return size_t(LBM_SLOT_AOS ? kSlotStride : 18) * size_t(Rpad); }
+inline size_t run_slot_words(int64_t Rpad) { return size_t(kSlotStride) * size_t(Rpad); }
 
 // Device addresses of the uploaded tables (all inside one caller buffer).
 struct DevTables {
@@ -130,8 +127,8 @@ struct lbm_lattice {
   std::vector<int32_t> warp_run0;  // [nwarps]  run holding node 32w
   std::vector<int32_t> warp_head0; // [nwarps]  first node of that run
   int64_t hist[33] = {0};
-  // The AA odd step's slots per run (derive_run_slots): -1 not derived yet,
-  // 0 the lattice does not qualify, 1 run_slot holds them
+  // The run slot tables (derive_run_slots): -1 not derived yet, 0 the lattice
+  // does not qualify, 1 run_slot holds them, 2 they hold pressure faces too
   int run_slot_state = -1;
   lbm::TableVec run_slot;          // [Rpad][kSlotStride] AA odd step
   lbm::TableVec run_slot_osnt;     // [Rpad][kSlotStride] OS-NT step

@@ -187,44 +187,58 @@ template <bool KEEP = true, class T> __device__ __forceinline__ T ld_idx(const T
 }
 template <int PREC> constexpr bool kKeepIdx = PREC != LBM_F64_DF;
 
-// The 18 slots of run r of a run slot table (derive_run_slots), each plus
-// off: sl[j] belongs to direction j + 1.  Run-major tables take four 16-byte
-// and one 8-byte load (the row is 80-byte aligned: the table starts on a
-// 256-byte boundary).  With a stash column (the AA odd step's [18][kBlock]
-// shared array at this thread's lane), each slot is also parked there as soon
-// as it is formed; parking all 18 after the loads made the FP16 step spill
-// 152 instead of 64 bytes and lose the gain.
-template <bool KEEP>
-__device__ __forceinline__ void run_slots(const int32_t* tbl, uint32_t rpad, int r, int off, unsigned (&sl)[18],
-                                          int* stash = nullptr) {
-#if LBM_SLOT_AOS
+// How a step kernel finds the slots of its nodes' PDFs: one instantiation each,
+// chosen by table_kind, so that the common ones carry neither the registers nor
+// the code of the others (a run-time choice of table in one kernel, with the
+// pressure masks of kSlotFace, cost 3-8 % in every form).
+//  kSlot      RIA through the run slot table, no pressure faces
+//  kSlotFace  the same with pressure faces (masks in the table's last two words)
+//  kAdj       the adjacency list, no pressure faces, grid below 2^32 slots
+//  kRunAny    RIA through the runs' adjacency entries: any grid, any markers
+//  kAdjAny    the adjacency list: any grid, any markers
+enum Table { kSlot, kSlotFace, kAdj, kRunAny, kAdjAny };
+__host__ __device__ constexpr bool is_run(int tab) { return tab == kSlot || tab == kSlotFace || tab == kRunAny; }
+__host__ __device__ constexpr bool is_any(int tab) { return tab == kRunAny || tab == kAdjAny; }
+
+// The slots of one node's 18 moving PDFs in the flat grid, sl[j] for direction
+// j + 1, and (kSlotFace) the directions that meet a pressure face: bit j of in /
+// out when the pull of direction j + 1 meets an inlet / outlet.
+struct NodeSlots {
+  unsigned sl[18], in, out;
+};
+
+// ... from row r of a run slot table (derive_run_slots), plus off.  Run-major
+// tables take four 16-byte loads and one of 8 bytes, or of 16 with FACE (the row
+// is 80-byte aligned: the table starts on a 256-byte boundary).  With a stash column (the AA odd step's shared array at this
+// thread's lane), each slot is also parked there as soon as it is formed;
+// parking all 18 after the loads made the FP16 step spill 152 instead of 64
+// bytes and lose the gain.
+template <bool KEEP, bool FACE>
+__device__ __forceinline__ void run_slots(const int32_t* tbl, int r, int off, NodeSlots& q, int* stash = nullptr) {
   const int4* p = reinterpret_cast<const int4*>(tbl + static_cast<size_t>(static_cast<unsigned>(r)) * kSlotStride);
 #pragma unroll
-  for (int q = 0; q < 5; ++q) {
+  for (int k4 = 0; k4 < 5; ++k4) {
     int w[4];
-    if (q < 4) {
-      const int4 v = ld_idx<KEEP>(p + q);
+    if (k4 < 4 || FACE) {
+      const int4 v = ld_idx<KEEP>(p + k4);
       w[0] = v.x, w[1] = v.y, w[2] = v.z, w[3] = v.w;
     } else {
       const int2 v = ld_idx<KEEP>(reinterpret_cast<const int2*>(p + 4));
       w[0] = v.x, w[1] = v.y, w[2] = w[3] = 0;
     }
+    if (FACE && k4 == 4) {
+      q.in = static_cast<unsigned>(w[2]);
+      q.out = static_cast<unsigned>(w[3]);
+    }
 #pragma unroll
     for (int k = 0; k < 4; ++k) {
-      const int j = 4 * q + k;
+      const int j = 4 * k4 + k;
       if (j < 18) {
-        sl[j] = static_cast<unsigned>(w[k] + off);
-        if (stash) stash[j * kBlock] = static_cast<int>(sl[j]);
+        q.sl[j] = static_cast<unsigned>(w[k] + off);
+        if (stash) stash[j * kBlock] = static_cast<int>(q.sl[j]);
       }
     }
   }
-#else
-#pragma unroll
-  for (int j = 0; j < 18; ++j) {
-    sl[j] = static_cast<unsigned>(ld_idx<KEEP>(tbl + at(j, rpad, r)) + off);
-    if (stash) stash[j * kBlock] = static_cast<int>(sl[j]);
-  }
-#endif
 }
 
 // ---- neighbour addressing --------------------------------------------------------------
@@ -271,6 +285,37 @@ template <bool KEEP = true> __device__ __forceinline__ void nbr_ria(const DevTab
     const int a = ld_idx<KEEP>(t.run_adj + at(i, t.rpad, c.r));
     m[i] = a >= 0 ? a + c.off : a;
   }
+}
+
+// The slots that the OS-NT (AA_ODD = false) or the AA odd step reads, by the
+// run slot table or (kAdj) resolved from the adjacency list: once, where
+// decoding the marker and the direction again at each store takes twice the
+// integer instructions.
+template <int TAB, bool AA_ODD, bool KEEP>
+__device__ __forceinline__ void node_slots(const DevTables& t, int n, NodeSlots& q, int* stash = nullptr) {
+  if constexpr (is_run(TAB)) {
+    const RiaCursor cur = ria_locate<KEEP>(t, n);
+    run_slots<KEEP, TAB == kSlotFace>(AA_ODD ? t.run_slot : t.run_slot_osnt, cur.r, cur.off, q, stash);
+  } else {
+    int m[18];
+    nbr_adj(t, n, m);
+#pragma unroll
+    for (int i = 1; i < kQ; ++i) {
+      const int mi = m[i - 1];
+      const unsigned dir = static_cast<unsigned>((mi >= 0) == AA_ODD ? inv(i) : i);
+      q.sl[i - 1] = dir * t.npad + static_cast<unsigned>(mi >= 0 ? mi : n);
+      if (stash) stash[(i - 1) * kBlock] = static_cast<int>(q.sl[i - 1]);
+    }
+  }
+}
+
+// The node's adjacency entries (kRunAny, kAdjAny).
+template <int TAB, bool KEEP>
+__device__ __forceinline__ void node_entries(const DevTables& t, int n, int (&m)[18]) {
+  if constexpr (is_run(TAB))
+    nbr_ria<KEEP>(t, ria_locate<KEEP>(t, n), m);
+  else
+    nbr_adj(t, n, m);
 }
 
 // ---- TRT collision (Sect. 2) in pair form ------------------------------------------------
@@ -656,6 +701,64 @@ __device__ __forceinline__ void gather(const typename St<PREC>::T* g, uint32_t n
   }
 }
 
+// Anti-bounce-back of pulled values at pressure faces (a warp-uniform branch
+// that warps away from the faces skip).
+template <int TAB, class V>
+__device__ __forceinline__ void face_pull(const NodeSlots& q, V (&d)[kQ], const V (&abb_in)[2],
+                                          const V (&abb_out)[2]) {
+  if constexpr (TAB == kSlotFace) {
+    if (warp_any((q.in | q.out) != 0u)) {
+#pragma unroll
+      for (int i = 1; i < kQ; ++i) {
+        if ((q.in >> (i - 1)) & 1u) d[i] = abb_in[wclass(i) - 1] - d[i];
+        if ((q.out >> (i - 1)) & 1u) d[i] = abb_out[wclass(i) - 1] - d[i];
+      }
+    }
+  }
+}
+
+// The stored PDFs of a node through its slots (storage units for LBM_F16S).
+template <int PREC, int TAB>
+__device__ __forceinline__ void slot_pull(const KParams& kp, const CollConst<typename St<PREC>::R>& c,
+                                          const typename St<PREC>::T* g, int n, const NodeSlots& q,
+                                          typename St<PREC>::R (&d)[kQ]) {
+  d[0] = ld_step<PREC>(g + n, kp.inv_scale);
+#pragma unroll
+  for (int i = 1; i < kQ; ++i) d[i] = ld_step<PREC>(g + q.sl[i - 1], kp.inv_scale);
+  face_pull<TAB>(q, d, c.abb_in, c.abb_out);
+}
+
+// Rows of the AA odd step's stash: the 18 slots, and the face masks.
+template <int TAB> constexpr int kStashRows = TAB == kSlotFace ? 20 : 18;
+
+template <int TAB> __device__ __forceinline__ void stash_faces(const NodeSlots& q, int* sm) {
+  if constexpr (TAB == kSlotFace) {
+    sm[18 * kBlock] = static_cast<int>(q.in);
+    sm[19 * kBlock] = static_cast<int>(q.out);
+  }
+}
+
+// The AA odd step's stores: P_i goes back to the slot f_inv(i) came from
+// (parked in sm, this thread's lane of the stash).
+template <int PREC, int TAB>
+__device__ __forceinline__ void slot_push(const KParams& kp, const CollConst<typename St<PREC>::R>& c,
+                                          typename St<PREC>::T* A, int n, const int* sm,
+                                          typename St<PREC>::R (&d)[kQ]) {
+  st_step<PREC>(A + n, d[0], kp.scale);
+  if constexpr (TAB == kSlotFace) {
+    const unsigned in = static_cast<unsigned>(sm[18 * kBlock]), out = static_cast<unsigned>(sm[19 * kBlock]);
+    if (warp_any((in | out) != 0u)) {
+#pragma unroll
+      for (int i = 1; i < kQ; ++i) {
+        if ((in >> (inv(i) - 1)) & 1u) d[i] = c.abb_in[wclass(i) - 1] - d[i];
+        if ((out >> (inv(i) - 1)) & 1u) d[i] = c.abb_out[wclass(i) - 1] - d[i];
+      }
+    }
+  }
+#pragma unroll
+  for (int i = 1; i < kQ; ++i) st_step<PREC>(A + static_cast<unsigned>(sm[(inv(i) - 1) * kBlock]), d[i], kp.scale);
+}
+
 // ---- kernels -----------------------------------------------------------------------------
 template <int PREC, bool RIA> struct OsntBlock {
   static constexpr int value = PREC == LBM_F16S && RIA ? LBM_OSNT_BLOCK_F16R : kBlock;
@@ -663,42 +766,24 @@ template <int PREC, bool RIA> struct OsntBlock {
 
 // OS-NT step: pull (indirect) from src, collide, store locally into dst with
 // evict-first stores so the write stream does not push src out of L2.
-template <int PREC, bool RIA, bool FORCE, bool DRAG, bool LP1 = false>
-__global__ void __launch_bounds__(OsntBlock<PREC, RIA>::value,
-                                  ctas(MinCtasOsnt<PREC, RIA, LP1>::value, OsntBlock<PREC, RIA>::value))
+template <int PREC, int TAB, bool FORCE, bool DRAG, bool LP1 = false>
+__global__ void __launch_bounds__(OsntBlock<PREC, is_run(TAB)>::value,
+                                  ctas(MinCtasOsnt<PREC, is_run(TAB), LP1>::value, OsntBlock<PREC, is_run(TAB)>::value))
     k_osnt(DevTables t, KParams kp, CollConst<typename St<PREC>::R> c, const typename St<PREC>::T* __restrict__ src,
            typename St<PREC>::T* __restrict__ dst, const float* __restrict__ s, int N) {
   using R = typename St<PREC>::R;
-  const int n0 = blockIdx.x * OsntBlock<PREC, RIA>::value;
-  const int n = n0 + threadIdx.x;
-  if (RIA && t.run_slot_osnt) {
-    // Pre-resolved run slots (no pressure faces; the grid below 2^31 slots):
-    // P_i (or P_inv(i) through a bounce-back marker) is pulled from slot
-    // run_slot_osnt(i, r) + off of the flat source grid.
-    if (n >= N) return;
-    const RiaCursor cur = ria_locate<kKeepIdx<PREC>>(t, n);
-    unsigned sl[18];
-    run_slots<kKeepIdx<PREC>>(t.run_slot_osnt, t.rpad, cur.r, cur.off, sl);
-    R d[kQ];
-    d[0] = ld_step<PREC>(src + n, kp.inv_scale);
-#pragma unroll
-    for (int i = 1; i < kQ; ++i) d[i] = ld_step<PREC>(src + sl[i - 1], kp.inv_scale);
-    const R sn = DRAG ? R(__ldg(s + n)) : R(0);
-    collide<R, FORCE, DRAG, LP1, kScaled<PREC>>(d, c, sn);
-#pragma unroll
-    for (int i = 0; i < kQ; ++i) st_stream_step<PREC>(dst + at(i, t.npad, n), d[i], kp.scale);
-    return;
-  }
-  int m[18];
-  if (RIA) {
-    if (n >= N) return;
-    nbr_ria<kKeepIdx<PREC>>(t, ria_locate<kKeepIdx<PREC>>(t, n), m);
-  } else {
-    if (n >= N) return;
-    nbr_adj(t, n, m);
-  }
+  const int n = blockIdx.x * OsntBlock<PREC, is_run(TAB)>::value + threadIdx.x;
+  if (n >= N) return;
   R d[kQ];
-  gather<PREC, false, kScaled<PREC>>(src, t.npad, n, m, d, kp.inv_scale, c.abb_in, c.abb_out, t.pressure);
+  if constexpr (is_any(TAB)) {
+    int m[18];
+    node_entries<TAB, kKeepIdx<PREC>>(t, n, m);
+    gather<PREC, false, kScaled<PREC>>(src, t.npad, n, m, d, kp.inv_scale, c.abb_in, c.abb_out, t.pressure);
+  } else {
+    NodeSlots q;
+    node_slots<TAB, false, kKeepIdx<PREC>>(t, n, q);
+    slot_pull<PREC, TAB>(kp, c, src, n, q, d);
+  }
   const R sn = DRAG ? R(__ldg(s + n)) : R(0);
   collide<R, FORCE, DRAG, LP1, kScaled<PREC>>(d, c, sn);
 #pragma unroll
@@ -757,123 +842,94 @@ __global__ void __launch_bounds__(kBlock) k_aa_even_h2(DevTables t, KParams kp, 
   }
 }
 
+// The double-float odd step's collision from its gathered doubles: it takes
+// the moments on the FP64 pipe, which it leaves mostly idle, and converts only
+// those 13 (or 23) values to double-float.
+template <bool FORCE, bool DRAG, bool LP1>
+__device__ __forceinline__ void collide_odd_df(const double (&g64)[kQ], const CollConst<df>& c, df sn, df (&d)[kQ]) {
+  double sa64[10], da64[10], drho64, jx64, jy64, jz64;
+  moments<double, !LP1, true>(g64, sa64, da64, drho64, jx64, jy64, jz64);
+  df sa[10], da[10];
+#pragma unroll
+  for (int k = 1; k <= 9; ++k) {
+    if (!LP1) sa[k] = df_from_double(sa64[k]);
+    da[k] = df_from_double(da64[k]);
+  }
+  if (!LP1) d[0] = df_from_double(g64[0]);
+  collide_m<df, FORCE, DRAG, LP1>(d, c, sn, sa, da, df_from_double(drho64), df_from_double(jx64),
+                                  df_from_double(jy64), df_from_double(jz64));
+}
+
 // AA odd step: read f_i from the neighbour's opposite slot A[inv i][m_i], collide,
 // write p_i to A[i][m_{inv i}] -- the same 19 slots, so in place and race-free.
-template <int PREC, bool RIA, bool FORCE, bool DRAG, bool LP1 = false>
-__global__ void __launch_bounds__(kBlock, ctas(MinCtasOdd<PREC, RIA, LP1>::value)) k_aa_odd(DevTables t, KParams kp,
+template <int PREC, int TAB, bool FORCE, bool DRAG, bool LP1 = false>
+__global__ void __launch_bounds__(kBlock, ctas(MinCtasOdd<PREC, is_run(TAB), LP1>::value)) k_aa_odd(DevTables t, KParams kp,
                                                                               CollConst<typename St<PREC>::R> c,
                                                                               typename St<PREC>::T* __restrict__ A,
                                                                               const float* __restrict__ s, int N) {
   using R = typename St<PREC>::R;
-  // The 18 resolved entries must survive the collision: they are parked in
-  // shared memory ([18][kBlock], lane-consecutive, conflict-free) rather than
-  // held in registers across it or read again from L1 after it (measured
-  // faster for every precision on GB300).
-  __shared__ int s_m[18][kBlock];
+  // The 18 resolved slots (kRunAny, kAdjAny: adjacency entries) must survive the
+  // collision: they are parked in shared memory (lane-consecutive,
+  // conflict-free) rather than held in registers across it or read again from
+  // L1 after it (measured faster for every precision on GB300).
+  __shared__ int s_m[kStashRows<TAB>][kBlock];
+  int* const sm = &s_m[0][threadIdx.x];
   const int n = blockIdx.x * kBlock + threadIdx.x;
   if (n >= N) return;
+  const R sn = DRAG ? R(__ldg(s + n)) : R(0);
   R d[kQ];
-  if (RIA && t.run_slot) {
-    // Pre-resolved run slots (no pressure faces; the grid below 2^31 slots):
-    // f_i is read from slot run_slot(i, r) + off of the flat grid, and P_i
-    // goes back to the slot f_inv(i) came from.
-    const RiaCursor cur = ria_locate<kKeepIdx<PREC>>(t, n);
-    unsigned sl[18];
-    run_slots<kKeepIdx<PREC>>(t.run_slot, t.rpad, cur.r, cur.off, sl, &s_m[0][threadIdx.x]);
+  if constexpr (!is_any(TAB)) {
+    NodeSlots q;
+    node_slots<TAB, true, kKeepIdx<PREC>>(t, n, q, sm);
+    stash_faces<TAB>(q, sm);
     if constexpr (PREC == LBM_F64_DF) {
       const double* g = reinterpret_cast<const double*>(A);
       double g64[kQ];
       g64[0] = __ldg(g + n);
 #pragma unroll
-      for (int i = 1; i < kQ; ++i) g64[i] = __ldg(g + sl[i - 1]);
-      double sa64[10], da64[10], drho64, jx64, jy64, jz64;
-      moments<double, !LP1, true>(g64, sa64, da64, drho64, jx64, jy64, jz64);
-      R sa[10], da[10];
-#pragma unroll
-      for (int k = 1; k <= 9; ++k) {
-        if (!LP1) sa[k] = df_from_double(sa64[k]);
-        da[k] = df_from_double(da64[k]);
-      }
-      if (!LP1) d[0] = df_from_double(g64[0]);
-      const R sn = DRAG ? R(__ldg(s + n)) : R(0);
-      collide_m<R, FORCE, DRAG, LP1>(d, c, sn, sa, da, df_from_double(drho64), df_from_double(jx64),
-                                     df_from_double(jy64), df_from_double(jz64));
+      for (int i = 1; i < kQ; ++i) g64[i] = __ldg(g + q.sl[i - 1]);
+      face_pull<TAB>(q, g64, c.abb64_in, c.abb64_out);
+      collide_odd_df<FORCE, DRAG, LP1>(g64, c, sn, d);
     } else {
-      d[0] = ld_step<PREC>(A + n, kp.inv_scale);
-#pragma unroll
-      for (int i = 1; i < kQ; ++i) d[i] = ld_step<PREC>(A + sl[i - 1], kp.inv_scale);
-      const R sn = DRAG ? R(__ldg(s + n)) : R(0);
+      slot_pull<PREC, TAB>(kp, c, A, n, q, d);
       collide<R, FORCE, DRAG, LP1, kScaled<PREC>>(d, c, sn);
     }
-    st_step<PREC>(A + n, d[0], kp.scale);
-#pragma unroll
-    for (int i = 1; i < kQ; ++i) st_step<PREC>(A + static_cast<unsigned>(s_m[inv(i) - 1][threadIdx.x]), d[i], kp.scale);
-    return;
-  }
-  {
+    slot_push<PREC, TAB>(kp, c, A, n, sm, d);
+  } else {
     int m[18];
-    if (RIA) {
-      nbr_ria<kKeepIdx<PREC>>(t, ria_locate<kKeepIdx<PREC>>(t, n), m);
-    } else {
-      nbr_adj(t, n, m);
-    }
+    node_entries<TAB, kKeepIdx<PREC>>(t, n, m);
 #pragma unroll
-    for (int j = 0; j < 18; ++j) s_m[j][threadIdx.x] = m[j];
+    for (int j = 0; j < 18; ++j) sm[j * kBlock] = m[j];
     if constexpr (PREC == LBM_F64_DF) {
-      // The double-float odd step leaves its FP64 pipe mostly idle: it takes
-      // the moments there, in IEEE double from the loaded doubles, and
-      // converts only those 13 (or 23) values to double-float.
       double g64[kQ];
       gather<LBM_F64, true>(reinterpret_cast<const double*>(A), t.npad, n, m, g64, kp.inv_scale, c.abb64_in,
                             c.abb64_out, t.pressure);
-      double sa64[10], da64[10], drho64, jx64, jy64, jz64;
-      moments<double, !LP1, true>(g64, sa64, da64, drho64, jx64, jy64, jz64);
-      R sa[10], da[10];
-#pragma unroll
-      for (int k = 1; k <= 9; ++k) {
-        if (!LP1) sa[k] = df_from_double(sa64[k]);
-        da[k] = df_from_double(da64[k]);
-      }
-      if (!LP1) d[0] = df_from_double(g64[0]);
-      const R sn = DRAG ? R(__ldg(s + n)) : R(0);
-      collide_m<R, FORCE, DRAG, LP1>(d, c, sn, sa, da, df_from_double(drho64), df_from_double(jx64),
-                                     df_from_double(jy64), df_from_double(jz64));
+      collide_odd_df<FORCE, DRAG, LP1>(g64, c, sn, d);
     } else {
       gather<PREC, true, kScaled<PREC>>(A, t.npad, n, m, d, kp.inv_scale, c.abb_in, c.abb_out, t.pressure);
+      collide<R, FORCE, DRAG, LP1, kScaled<PREC>>(d, c, sn);
     }
-  }
-  if constexpr (PREC != LBM_F64_DF) {
-    const R sn = DRAG ? R(__ldg(s + n)) : R(0);
-    collide<R, FORCE, DRAG, LP1, kScaled<PREC>>(d, c, sn);
-  }
-  st_step<PREC>(A + n, d[0], kp.scale);
-  // p_i goes to the slot node m_{inv i} pulls it from next (or, through a
-  // marker, to this node's own opposite slot)
-  int mo_[18];
+    st_step<PREC>(A + n, d[0], kp.scale);
+    // p_i goes to the slot node m_{inv i} pulls it from next (or, through a
+    // marker, to this node's own opposite slot)
 #pragma unroll
-  for (int j = 0; j < 18; ++j) mo_[j] = s_m[j][threadIdx.x];
-  bool face = false;
-  if (t.pressure) {
+    for (int j = 0; j < 18; ++j) m[j] = sm[j * kBlock];
+    bool face = false;
+    if (t.pressure) {
 #pragma unroll
-    for (int j = 0; j < 18; ++j) face |= mo_[j] < -1;
-  }
-  if (t.pressure && warp_any(face)) {
+      for (int j = 0; j < 18; ++j) face |= m[j] < -1;
+    }
+    if (t.pressure && warp_any(face)) {
+#pragma unroll
+      for (int i = 1; i < kQ; ++i) {
+        const int mo = m[inv(i) - 1];
+        if (mo < -1) d[i] = (mo == LBM_MARK_INLET ? c.abb_in[wclass(i) - 1] : c.abb_out[wclass(i) - 1]) - d[i];
+      }
+    }
 #pragma unroll
     for (int i = 1; i < kQ; ++i) {
-      const int mo = mo_[inv(i) - 1];
-      R v = d[i];
-      if (mo < -1) v = (mo == LBM_MARK_INLET ? c.abb_in[wclass(i) - 1] : c.abb_out[wclass(i) - 1]) - v;
-      const int dir = mo >= 0 ? i : inv(i);
-      const int node = mo >= 0 ? mo : n;
-      st_step<PREC>(A + at(dir, t.npad, node), v, kp.scale);
-    }
-  } else {
-#pragma unroll
-    for (int i = 1; i < kQ; ++i) {
-      const int mo = mo_[inv(i) - 1];
-      const int dir = mo >= 0 ? i : inv(i);
-      const int node = mo >= 0 ? mo : n;
-      st_step<PREC>(A + at(dir, t.npad, node), d[i], kp.scale);
+      const int mo = m[inv(i) - 1];
+      st_step<PREC>(A + at(mo >= 0 ? i : inv(i), t.npad, mo >= 0 ? mo : n), d[i], kp.scale);
     }
   }
 }
@@ -890,14 +946,16 @@ __global__ void __launch_bounds__(kBlock, ctas(MinCtasOdd<PREC, RIA, LP1>::value
 #ifndef LBM_MIN_CTAS_ODD_X2
 #define LBM_MIN_CTAS_ODD_X2 8
 #endif
-template <int PREC, bool FORCE, bool DRAG>
+template <int PREC, int TAB, bool FORCE, bool DRAG>
 __global__ void __launch_bounds__(kBlock, ctas(LBM_MIN_CTAS_ODD_X2)) k_aa_odd_x2(DevTables t, KParams kp,
                                                                          CollConst<typename St<PREC>::R> c,
                                                                          typename St<PREC>::T* __restrict__ A,
                                                                          const float* __restrict__ s, int N) {
   using R = typename St<PREC>::R;
   static_assert(std::is_same<R, float>::value, "float-collision precisions only");
-  __shared__ int s_sl[2][18][kBlock];
+  __shared__ int s_sl[2][kStashRows<TAB>][kBlock];
+  int* const sm0 = &s_sl[0][0][threadIdx.x];
+  int* const sm1 = &s_sl[1][0][threadIdx.x];
   const int n0 = blockIdx.x * (2 * kBlock) + threadIdx.x;
   if (n0 >= N) return;
   const int n1 = n0 + kBlock;
@@ -906,35 +964,33 @@ __global__ void __launch_bounds__(kBlock, ctas(LBM_MIN_CTAS_ODD_X2)) k_aa_odd_x2
   {
     const RiaCursor c0 = ria_locate(t, n0);
     const RiaCursor c1 = ria_locate(t, has1 ? n1 : n0);
-    unsigned sl0[18], sl1[18];
-    run_slots<true>(t.run_slot, t.rpad, c0.r, c0.off, sl0);
-    run_slots<true>(t.run_slot, t.rpad, c1.r, c1.off, sl1);
+    NodeSlots q0, q1;
+    run_slots<true, TAB == kSlotFace>(t.run_slot, c0.r, c0.off, q0);
+    run_slots<true, TAB == kSlotFace>(t.run_slot, c1.r, c1.off, q1);
 #pragma unroll
     for (int j = 0; j < 18; ++j) {
-      s_sl[0][j][threadIdx.x] = static_cast<int>(sl0[j]);
-      s_sl[1][j][threadIdx.x] = static_cast<int>(sl1[j]);
+      sm0[j * kBlock] = static_cast<int>(q0.sl[j]);
+      sm1[j * kBlock] = static_cast<int>(q1.sl[j]);
     }
+    stash_faces<TAB>(q0, sm0);
+    stash_faces<TAB>(q1, sm1);
     d0[0] = ld_step<PREC>(A + n0, kp.inv_scale);
     d1[0] = ld_step<PREC>(A + (has1 ? n1 : n0), kp.inv_scale);
 #pragma unroll
     for (int i = 1; i < kQ; ++i) {
-      d0[i] = ld_step<PREC>(A + sl0[i - 1], kp.inv_scale);
-      d1[i] = ld_step<PREC>(A + sl1[i - 1], kp.inv_scale);
+      d0[i] = ld_step<PREC>(A + q0.sl[i - 1], kp.inv_scale);
+      d1[i] = ld_step<PREC>(A + q1.sl[i - 1], kp.inv_scale);
     }
+    face_pull<TAB>(q0, d0, c.abb_in, c.abb_out);
+    face_pull<TAB>(q1, d1, c.abb_in, c.abb_out);
   }
   const R s0 = DRAG ? R(__ldg(s + n0)) : R(0);
   collide<R, FORCE, DRAG, false, kScaled<PREC>>(d0, c, s0);
-  st_step<PREC>(A + n0, d0[0], kp.scale);
-#pragma unroll
-  for (int i = 1; i < kQ; ++i)
-    st_step<PREC>(A + static_cast<unsigned>(s_sl[0][inv(i) - 1][threadIdx.x]), d0[i], kp.scale);
+  slot_push<PREC, TAB>(kp, c, A, n0, sm0, d0);
   if (has1) {
     const R s1 = DRAG ? R(__ldg(s + n1)) : R(0);
     collide<R, FORCE, DRAG, false, kScaled<PREC>>(d1, c, s1);
-    st_step<PREC>(A + n1, d1[0], kp.scale);
-#pragma unroll
-    for (int i = 1; i < kQ; ++i)
-      st_step<PREC>(A + static_cast<unsigned>(s_sl[1][inv(i) - 1][threadIdx.x]), d1[i], kp.scale);
+    slot_push<PREC, TAB>(kp, c, A, n1, sm1, d1);
   }
 }
 
@@ -1404,6 +1460,29 @@ inline unsigned grid_of(int64_t N) { return unsigned((N + dev::kBlock - 1) / dev
 // read-back).  Never more than the workspace holds (reduce_parts).
 inline unsigned reduce_grid(int64_t nparts) { return unsigned(std::min<int64_t>(std::max<int64_t>(nparts, 1), 16 * 152)); }
 
+// The table a step of this lattice reads (dev::Table).  Grids of 2^32 slots or
+// more (above 226 M nodes) have no 32-bit slot index.
+inline int table_kind(const lbm_lattice* L, int ria) {
+  if (ria) return !L->dev.run_slot ? dev::kRunAny : L->dev.pressure ? dev::kSlotFace : dev::kSlot;
+  const bool wide = int64_t(kQ) * L->Npad >= (int64_t(1) << 32);
+  return wide || L->dev.pressure ? dev::kAdjAny : dev::kAdj;
+}
+
+// Run BODY(TAB) for the lattice's table; SLOTS: whether the kernel has the run
+// slot instantiations.
+#define LBM_BY_TABLE(BODY, SLOTS)                           \
+  switch (table_kind(L, ria)) {                             \
+    case dev::kSlot:                                        \
+      if constexpr (SLOTS) BODY(dev::kSlot);                \
+      break;                                                \
+    case dev::kSlotFace:                                    \
+      if constexpr (SLOTS) BODY(dev::kSlotFace);            \
+      break;                                                \
+    case dev::kAdj: BODY(dev::kAdj); break;                 \
+    case dev::kRunAny: BODY(dev::kRunAny); break;           \
+    default: BODY(dev::kAdjAny); break;                     \
+  }
+
 inline bool has_force(const KParams& kp) { return kp.g[0] != 0.0 || kp.g[1] != 0.0 || kp.g[2] != 0.0; }
 
 // The l+ = 1 collision (see collide) is instantiated for the FP64-storage
@@ -1441,22 +1520,19 @@ int launch_osnt_t(const lbm_lattice* L, const KParams& kp, const void* src, void
   const bool f = has_force(kp);
   const auto c = dev::make_coll_step<PREC>(kp);
   const bool lp1 = use_lp1<PREC>(kp);
-#define LBM_OSNT(R_, F_, D_) LBM_LAUNCH_LP1(k_osnt, LBM_TARGS3(R_, F_, D_), (L->dev, kp, c, a, b, s, N))
-  if (s) {
-    if (ria) LBM_OSNT(true, true, true); else LBM_OSNT(false, true, true);
-  } else if (f) {
-    if (ria) LBM_OSNT(true, true, false); else LBM_OSNT(false, true, false);
-  } else {
-    if (ria) LBM_OSNT(true, false, false); else LBM_OSNT(false, false, false);
-  }
+#define LBM_OSNT(T_)                                                                                    \
+  do {                                                                                                  \
+    if (s)                                                                                              \
+      LBM_LAUNCH_LP1(k_osnt, LBM_TARGS3(T_, true, true), (L->dev, kp, c, a, b, s, N));                  \
+    else if (f)                                                                                         \
+      LBM_LAUNCH_LP1(k_osnt, LBM_TARGS3(T_, true, false), (L->dev, kp, c, a, b, s, N));                 \
+    else                                                                                                \
+      LBM_LAUNCH_LP1(k_osnt, LBM_TARGS3(T_, false, false), (L->dev, kp, c, a, b, s, N));                \
+  } while (0)
+  LBM_BY_TABLE(LBM_OSNT, true)
 #undef LBM_OSNT
   return cuda_check("OS-NT step launch");
 }
-
-#ifndef LBM_ODD_X2
-#define LBM_ODD_X2 1
-#endif
-constexpr bool kOddX2 = LBM_ODD_X2 != 0;
 
 template <int PREC>
 int launch_aa_t(const lbm_lattice* L, const KParams& kp, void* pdf, int parity, const float* s, int ria,
@@ -1488,22 +1564,32 @@ int launch_aa_t(const lbm_lattice* L, const KParams& kp, void* pdf, int parity, 
     return cuda_check("AA even step launch");
   }
   if constexpr (PREC == LBM_F32) {
-    if (ria && L->dev.run_slot && kOddX2) {
+    if (ria && L->dev.run_slot) {
       const unsigned g2 = unsigned((L->N + 2 * dev::kBlock - 1) / (2 * dev::kBlock));
-      if (s) dev::k_aa_odd_x2<PREC, true, true><<<g2, dev::kBlock, 0, st>>>(L->dev, kp, c, A, s, N);
-      else if (f) dev::k_aa_odd_x2<PREC, true, false><<<g2, dev::kBlock, 0, st>>>(L->dev, kp, c, A, s, N);
-      else dev::k_aa_odd_x2<PREC, false, false><<<g2, dev::kBlock, 0, st>>>(L->dev, kp, c, A, s, N);
+#define LBM_AAODD2(T_)                                                                                   \
+  do {                                                                                                   \
+    if (s) dev::k_aa_odd_x2<PREC, T_, true, true><<<g2, dev::kBlock, 0, st>>>(L->dev, kp, c, A, s, N);   \
+    else if (f) dev::k_aa_odd_x2<PREC, T_, true, false><<<g2, dev::kBlock, 0, st>>>(L->dev, kp, c, A, s, N); \
+    else dev::k_aa_odd_x2<PREC, T_, false, false><<<g2, dev::kBlock, 0, st>>>(L->dev, kp, c, A, s, N);   \
+  } while (0)
+      if (L->dev.pressure)
+        LBM_AAODD2(dev::kSlotFace);
+      else
+        LBM_AAODD2(dev::kSlot);
+#undef LBM_AAODD2
       return cuda_check("AA odd step launch");
     }
   }
-#define LBM_AAODD(R_, F_, D_) LBM_LAUNCH_LP1(k_aa_odd, LBM_TARGS3(R_, F_, D_), (L->dev, kp, c, A, s, N))
-  if (s) {
-    if (ria) LBM_AAODD(true, true, true); else LBM_AAODD(false, true, true);
-  } else if (f) {
-    if (ria) LBM_AAODD(true, true, false); else LBM_AAODD(false, true, false);
-  } else {
-    if (ria) LBM_AAODD(true, false, false); else LBM_AAODD(false, false, false);
-  }
+#define LBM_AAODD(T_)                                                                                   \
+  do {                                                                                                  \
+    if (s)                                                                                              \
+      LBM_LAUNCH_LP1(k_aa_odd, LBM_TARGS3(T_, true, true), (L->dev, kp, c, A, s, N));                   \
+    else if (f)                                                                                         \
+      LBM_LAUNCH_LP1(k_aa_odd, LBM_TARGS3(T_, true, false), (L->dev, kp, c, A, s, N));                  \
+    else                                                                                                \
+      LBM_LAUNCH_LP1(k_aa_odd, LBM_TARGS3(T_, false, false), (L->dev, kp, c, A, s, N));                 \
+  } while (0)
+  LBM_BY_TABLE(LBM_AAODD, (PREC != LBM_F32))  // FP32 took k_aa_odd_x2 above
 #undef LBM_AAODD
   return cuda_check("AA odd step launch");
 }

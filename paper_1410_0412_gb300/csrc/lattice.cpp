@@ -476,9 +476,16 @@ int derive_et_tables(lbm_lattice* L);
 // spends one add per access.  Lattices
 // with pressure markers (whose anti-bounce-back needs the marker kind) or a
 // grid of 2^31 or more slots do not qualify: run_slot_state = 0.
+// Run slot tables, for grids below 2^31 slots.  Row r holds the AA odd step's
+// (run_slot) and the OS-NT step's (run_slot_osnt) slots of run r's first node;
+// words 18 and 19 hold the directions whose pull meets an inlet or an outlet
+// (bit i - 1).  A lattice with pressure faces has them when its runs number at
+// most half its nodes: 160 bytes a run are then no more than the adjacency list,
+// while at one run per node (a Hilbert order) the rows read as many bytes as the
+// runs' adjacency entries and would double the tables of a large lattice.
 int derive_run_slots(lbm_lattice* L) {
   if (L->run_slot_state >= 0) return LBM_OK;
-  if (int64_t(19) * L->Npad >= (int64_t(1) << 31) || L->bc.x_pressure) {
+  if (int64_t(19) * L->Npad >= (int64_t(1) << 31)) {
     L->run_slot_state = 0;
     return LBM_OK;
   }
@@ -491,39 +498,40 @@ int derive_run_slots(lbm_lattice* L) {
           return;
         }
     });
-    if (marker) {
+    const bool pressure = marker || L->bc.x_pressure;
+    if (pressure && 2 * L->R > L->N) {
       L->run_slot_state = 0;
       return LBM_OK;
     }
     L->run_slot.resize(run_slot_words(L->Rpad));
     L->run_slot_osnt.resize(run_slot_words(L->Rpad));
-    // element (i, r): run-major r * kSlotStride + i - 1, or direction-major (i - 1) * Rpad + r
-    const size_t rs_r = LBM_SLOT_AOS ? kSlotStride : 1, rs_i = LBM_SLOT_AOS ? 1 : size_t(L->Rpad);
     parallel_for(L->Rpad, [&](int64_t rb, int64_t re) {
       for (int64_t r = rb; r < re; ++r) {
+        int32_t* aa = &L->run_slot[size_t(r) * kSlotStride];
+        int32_t* os = &L->run_slot_osnt[size_t(r) * kSlotStride];
+        uint32_t in = 0, out = 0;
         for (int i = 1; i <= 18; ++i) {
-          const size_t k = size_t(r) * rs_r + size_t(i - 1) * rs_i;
           if (r >= L->R) {
-            L->run_slot[k] = L->run_slot_osnt[k] = 0;  // padding
+            aa[i - 1] = os[i - 1] = 0;  // padding
           } else {
             const int32_t a = L->run_adj[size_t(i - 1) * L->Rpad + size_t(r)];
             const int64_t head = L->run_start[size_t(r)];
-            L->run_slot[k] = a >= 0 ? int32_t(int64_t(kInv[i]) * L->Npad + a) : int32_t(int64_t(i) * L->Npad + head);
-            L->run_slot_osnt[k] =
-                a >= 0 ? int32_t(int64_t(i) * L->Npad + a) : int32_t(int64_t(kInv[i]) * L->Npad + head);
+            aa[i - 1] = a >= 0 ? int32_t(int64_t(kInv[i]) * L->Npad + a) : int32_t(int64_t(i) * L->Npad + head);
+            os[i - 1] = a >= 0 ? int32_t(int64_t(i) * L->Npad + a) : int32_t(int64_t(kInv[i]) * L->Npad + head);
+            in |= a == LBM_MARK_INLET ? 1u << (i - 1) : 0u;
+            out |= a == LBM_MARK_OUTLET ? 1u << (i - 1) : 0u;
           }
         }
-        if (LBM_SLOT_AOS)
-          for (int w = 18; w < kSlotStride; ++w)
-            L->run_slot[size_t(r) * kSlotStride + w] = L->run_slot_osnt[size_t(r) * kSlotStride + w] = 0;
+        aa[18] = os[18] = int32_t(in);
+        aa[19] = os[19] = int32_t(out);
       }
     });
+    L->run_slot_state = pressure ? 2 : 1;
   } catch (const std::bad_alloc&) {
     L->run_slot.clear();
     L->run_slot_osnt.clear();
     return set_error(LBM_ERR_ALLOC, "out of host memory for the run slot table");
   }
-  L->run_slot_state = 1;
   return LBM_OK;
 }
 
