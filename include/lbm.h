@@ -447,6 +447,13 @@ LBM_API int lbm_step_aa(const lbm_lattice* lat, int prec, const lbm_params* para
 LBM_API int lbm_run_aa(const lbm_lattice* lat, int prec, const lbm_params* params, void* pdf,
                int start_parity, int steps, const float* s, int ria, void* stream);
 
+/* Run `steps` OS-NT steps from grid0, the state ping-ponging between the two
+ * grids: it ends in grid0 after an even number of steps, in grid1 after an odd
+ * one (the other grid is overwritten).  Errors as lbm_step_osnt, and for
+ * steps < 0. */
+LBM_API int lbm_run_osnt(const lbm_lattice* lat, int prec, const lbm_params* params, void* grid0, void* grid1,
+                         int steps, const float* s, int ria, void* stream);
+
 /* ---- Esoteric Twist: the third single-grid form (named in Sect. 1 and Sect. 4) ----
  * The paper lists Geier's Esoteric Twist with OS-NT and the AA pattern as the
  * lowest-loop-balance propagation schemes but does not evaluate it.  Layout

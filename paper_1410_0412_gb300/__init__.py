@@ -435,6 +435,15 @@ def lbm_step_osnt(lat, prec, params, src, dst, s=None, ria=False, stream=None):
                                     _ptr(_check_s(lat, s)), 1 if ria else 0, _stream(stream)), "lbm_step_osnt")
 
 
+def lbm_run_osnt(lat, prec, params, grid0, grid1, steps, s=None, ria=False, stream=None):
+    """``steps`` OS-NT steps from grid0; the state ends in grid0 (even) or grid1 (odd)."""
+    prec = _prec(prec)
+    _check_grid(lat, prec, grid0, "grid0")
+    _check_grid(lat, prec, grid1, "grid1")
+    check(_lib.load().lbm_run_osnt(lat.handle, prec, ctypes.byref(params.c()), _ptr(grid0), _ptr(grid1), int(steps),
+                                   _ptr(_check_s(lat, s)), 1 if ria else 0, _stream(stream)), "lbm_run_osnt")
+
+
 def lbm_step_aa(lat, prec, params, pdf, parity, s=None, ria=False, stream=None):
     prec = _prec(prec)
     _check_grid(lat, prec, pdf, "pdf")
@@ -831,10 +840,11 @@ class Solver:
 
     def step(self, n=1, stream=None):
         if self.form == "osnt":
-            for _ in range(n):
-                lbm_step_osnt(self.lat, self.prec, self.params, self.grids[0], self.grids[1], self.s, self.ria, stream)
+            n = len(range(n))
+            lbm_run_osnt(self.lat, self.prec, self.params, self.grids[0], self.grids[1], n, self.s, self.ria, stream)
+            if n % 2:
                 self.grids.reverse()
-                self.t += 1
+            self.t += n
         elif self.form == "et":
             lbm_run_et(self.lat, self.prec, self.params, self.grids[0], self.t % 2, n, self.s, self.ria, stream)
             self.t += n
@@ -842,14 +852,20 @@ class Solver:
             lbm_run_aa(self.lat, self.prec, self.params, self.grids[0], self.t % 2, n, self.s, self.ria, stream)
             self.t += n
 
+    # Step pairs of the longer of step_graph's two graphs: consecutive steps of
+    # one graph overlap their launches, consecutive graphs do not (100 OS-NT-R
+    # FP32 steps on 46 k nodes: 424 us with one pair per graph, 250 with 16).
+    _GRAPH_PAIRS = 16
+
     def step_graph(self, n):
-        """Advance n steps (n even) by replaying a CUDA graph of one step pair.
+        """Advance n steps (n even) by replaying CUDA graphs of step pairs.
 
         For small lattices, where a step takes a few microseconds, launch
-        overhead dominates; the pair (even + odd AA step, or two OS-NT steps
-        ping-ponging the grids) is captured once and replayed n / 2 times on
-        the current stream.  The graph is rebuilt when the solver's grids or
-        parameters change (call ``reset_graph``).
+        overhead dominates; one pair (even + odd AA step, or two OS-NT steps
+        ping-ponging the grids) and, for long advances, a block of 16 pairs are
+        each captured once and replayed on the current stream.  The graphs are
+        rebuilt when the solver's grids or parameters change (call
+        ``reset_graph``).
         """
         torch = _torch()
         if n % 2:
@@ -865,21 +881,38 @@ class Solver:
                 self.step(2)
             torch.cuda.current_stream().wait_stream(side)
             n -= 2
-            g = torch.cuda.CUDAGraph()
-            with torch.cuda.graph(g):
-                st = torch.cuda.current_stream()
-                if self.form == "osnt":
-                    lbm_step_osnt(self.lat, self.prec, self.params, self.grids[0], self.grids[1], self.s, self.ria, st)
-                    lbm_step_osnt(self.lat, self.prec, self.params, self.grids[1], self.grids[0], self.s, self.ria, st)
-                elif self.form == "et":
-                    lbm_run_et(self.lat, self.prec, self.params, self.grids[0], 0, 2, self.s, self.ria, st)
-                else:
-                    lbm_step_aa(self.lat, self.prec, self.params, self.grids[0], 0, self.s, self.ria, st)
-                    lbm_step_aa(self.lat, self.prec, self.params, self.grids[0], 1, self.s, self.ria, st)
-            self._graph = g
-        for _ in range(n // 2):
-            self._graph.replay()
-        self.t += n
+            self._graph = {}
+        left = n // 2
+        if left >= self._GRAPH_PAIRS:
+            if "block" not in self._graph:
+                self._graph["block"] = self._capture(2 * self._GRAPH_PAIRS)
+            while left >= self._GRAPH_PAIRS:
+                self._graph["block"].replay()
+                left -= self._GRAPH_PAIRS
+                self.t += 2 * self._GRAPH_PAIRS
+            if "pair" not in self._graph:  # the rest of a long advance is not worth a capture
+                self.step(2 * left)
+                return
+        if left and "pair" not in self._graph:
+            self._graph["pair"] = self._capture(2)
+        for _ in range(left):
+            self._graph["pair"].replay()
+        self.t += 2 * left
+
+    def _capture(self, steps):
+        """A CUDA graph of an even number of steps from the current (even) state."""
+        torch = _torch()
+        g = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(g):
+            st = torch.cuda.current_stream()
+            if self.form == "osnt":
+                lbm_run_osnt(self.lat, self.prec, self.params, self.grids[0], self.grids[1], steps, self.s, self.ria,
+                             st)
+            elif self.form == "et":
+                lbm_run_et(self.lat, self.prec, self.params, self.grids[0], 0, steps, self.s, self.ria, st)
+            else:
+                lbm_run_aa(self.lat, self.prec, self.params, self.grids[0], 0, steps, self.s, self.ria, st)
+        return g
 
     def reset_graph(self):
         self._graph = None
@@ -894,7 +927,7 @@ class Solver:
 
 __all__ = [
     "Params", "Lattice", "Solver", "LbmError", "lbm_init_equilibrium", "lbm_load_canonical", "lbm_canonical_pdfs",
-    "lbm_step_osnt", "lbm_step_aa", "lbm_run_aa", "lbm_macroscopic", "LBM_F64", "LBM_F32", "LBM_F16S", "LBM_F64_DF",
+    "lbm_step_osnt", "lbm_run_osnt", "lbm_step_aa", "lbm_run_aa", "lbm_macroscopic", "LBM_F64", "LBM_F32", "LBM_F16S", "LBM_F64_DF",
     "LBM_LAYOUT_OSNT", "LBM_LAYOUT_AA_EVEN", "LBM_LAYOUT_AA_ODD", "LBM_TABLES_ADJ", "LBM_TABLES_RIA",
     "LBM_LAYOUT_ET_EVEN", "LBM_LAYOUT_ET_ODD", "LBM_TABLES_ET", "lbm_step_et", "lbm_run_et", "Partitioning",
     "PartitionedSolver", "lbm_halo_exchange", "lbm_partition_run_aa", "lbm_partition_run_osnt",

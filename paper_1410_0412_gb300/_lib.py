@@ -102,6 +102,7 @@ SIGNATURES = {
     "lbm_canonical_pdfs": [_P, _I, ctypes.POINTER(lbm_params), _P, _I, _P, _P],
     "lbm_step_osnt": [_P, _I, ctypes.POINTER(lbm_params), _P, _P, _P, _I, _P],
     "lbm_step_aa": [_P, _I, ctypes.POINTER(lbm_params), _P, _I, _P, _I, _P],
+    "lbm_run_osnt": [_P, _I, ctypes.POINTER(lbm_params), _P, _P, _I, _P, _I, _P],
     "lbm_run_aa": [_P, _I, ctypes.POINTER(lbm_params), _P, _I, _I, _P, _I, _P],
     "lbm_et_info": [_P, _PI64, _PI64, _P],
     "lbm_export_et_tables": [_P, _P, _P],

@@ -648,6 +648,23 @@ int lbm_step_osnt(const lbm_lattice* L, int prec, const lbm_params* params, cons
   return LBM_DISPATCH_STEP(prec, launch_osnt_t, L, kp, src, dst, s, ria ? 1 : 0, stream);
 }
 
+int lbm_run_osnt(const lbm_lattice* L, int prec, const lbm_params* params, void* grid0, void* grid1, int steps,
+                 const float* s, int ria, void* stream) {
+  if (int rc = check_lat(L)) return rc;
+  KParams kp;
+  if (int rc = make_kparams(params, prec, &kp)) return rc;
+  if (!grid0 || !grid1) return set_error(LBM_ERR_ARG, "grid0 or grid1 is NULL");
+  if (grid0 == grid1) return set_error(LBM_ERR_ARG, "OS-NT needs two distinct grids");
+  if (steps < 0) return set_error(LBM_ERR_ARG, "steps must be >= 0");
+  if (L->N == 0 || steps == 0) return LBM_OK;
+  if (int rc = check_tables(L, ria)) return rc;
+  for (int t = 0; t < steps; ++t)
+    if (int rc = LBM_DISPATCH_STEP(prec, launch_osnt_t, L, kp, t & 1 ? grid1 : grid0, t & 1 ? grid0 : grid1, s,
+                                   ria ? 1 : 0, stream))
+      return rc;
+  return LBM_OK;
+}
+
 int lbm_step_aa(const lbm_lattice* L, int prec, const lbm_params* params, void* pdf, int parity, const float* s,
                 int ria, void* stream) {
   if (int rc = check_lat(L)) return rc;
