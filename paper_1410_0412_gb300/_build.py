@@ -21,7 +21,13 @@ LIB = os.path.join(PKG, "liblbm.so")
 
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 COMMON = ["-O3", "-std=c++17", "-lineinfo", "-Xcompiler", "-fPIC,-fvisibility=hidden", "-I" + os.path.join(ROOT, "include")]
-SOURCES = ["api.cpp", "lattice.cpp", "kernels_f64.cu", "kernels_f64df.cu", "kernels_f32.cu", "kernels_f16s.cu", "adjoint.cu", "noalloc.cu", "bandwidth.cu", "partition.cpp", "halo.cu"]
+# the longest compilations first
+SOURCES = [
+    "kernels_f64_aa.cu", "kernels_f64_osnt.cu", "kernels_f64_et.cu", "adjoint.cu", "kernels_f32_osnt.cu",
+    "kernels_f32_aa.cu", "kernels_f32_et.cu", "kernels_f16s_osnt.cu", "kernels_f16s_aa.cu",
+    "kernels_f16s_et.cu", "kernels_f64df_osnt.cu", "kernels_f64df_aa.cu", "kernels_f64df_et.cu",
+    "kernels_state.cu", "noalloc.cu", "bandwidth.cu", "halo.cu", "api.cpp", "lattice.cpp", "partition.cpp",
+]
 
 
 def nvcc() -> str:
@@ -62,7 +68,7 @@ def build(verbose: bool = False, force: bool = False, ptxas_info: bool = False) 
             raise RuntimeError(f"nvcc failed on {src}:\n{r.stderr}")
         return obj, r.stderr
 
-    with ThreadPoolExecutor(max_workers=min(8, len(srcs))) as ex:
+    with ThreadPoolExecutor(max_workers=min(os.cpu_count() or 8, 16, len(srcs))) as ex:
         results = list(ex.map(compile_one, srcs))
     if verbose or ptxas_info:
         for (obj, err), src in zip(results, srcs):

@@ -43,19 +43,19 @@ template <class R> struct AdjConst {
 // double-float one converts on load and store), float otherwise.
 template <int PREC> struct Lam {
   using T = float;
-  static __device__ __forceinline__ float ld(const T* p) { return *p; }
+  template <bool DEP = false> static __device__ __forceinline__ float ld(const T* p) { return ld_grid<DEP>(p); }
   static __device__ __forceinline__ void st(T* p, float v) { *p = v; }
   static __device__ __forceinline__ double to_double(float v) { return double(v); }
 };
 template <> struct Lam<LBM_F64> {
   using T = double;
-  static __device__ __forceinline__ double ld(const T* p) { return *p; }
+  template <bool DEP = false> static __device__ __forceinline__ double ld(const T* p) { return ld_grid<DEP>(p); }
   static __device__ __forceinline__ void st(T* p, double v) { *p = v; }
   static __device__ __forceinline__ double to_double(double v) { return v; }
 };
 template <> struct Lam<LBM_F64_DF> {
   using T = double;
-  static __device__ __forceinline__ df ld(const T* p) { return df_from_double(*p); }
+  template <bool DEP = false> static __device__ __forceinline__ df ld(const T* p) { return df_from_double(ld_grid<DEP>(p)); }
   static __device__ __forceinline__ void st(T* p, df v) { *p = double_from_df(v); }
   static __device__ __forceinline__ double to_double(df v) { return double_from_df(v); }
 };
@@ -169,7 +169,7 @@ __device__ __forceinline__ void adj_moments(const R (&mu)[kQ], const AdjConst<R>
 template <int PREC> struct MinCtasAdj { static constexpr int value = LBM_MIN_CTAS_ADJ; };
 template <> struct MinCtasAdj<LBM_F64> { static constexpr int value = 4; };
 template <> struct MinCtasAdj<LBM_F64_DF> { static constexpr int value = 3; };
-template <int PREC, int TAB, bool DRAG, bool LP1 = false>
+template <int PREC, bool DEP, int TAB, bool DRAG, bool LP1 = false>
 __global__ void __launch_bounds__(kBlock, MinCtasAdj<PREC>::value) k_adjoint(DevTables t, KParams kp, CollConst<typename St<PREC>::R> cc,
                                                     AdjConst<typename St<PREC>::R> c,
                                                     const typename St<PREC>::T* __restrict__ G,
@@ -192,29 +192,31 @@ __global__ void __launch_bounds__(kBlock, MinCtasAdj<PREC>::value) k_adjoint(Dev
     const RiaCursor cur = ria_locate<kKeepIdx<PREC>>(t, n);
     NodeSlots q;
     run_slots<kKeepIdx<PREC>, false>(t.run_slot_osnt, cur.r, cur.off, q);
-    d[0] = St<PREC>::ld(G + n, kp.inv_scale);
+    if (DEP) step_wait();
+    d[0] = St<PREC>::template ld<DEP>(G + n, kp.inv_scale);
 #pragma unroll
-    for (int i = 1; i < kQ; ++i) d[i] = St<PREC>::ld(G + q.sl[i - 1], kp.inv_scale);
+    for (int i = 1; i < kQ; ++i) d[i] = St<PREC>::template ld<DEP>(G + q.sl[i - 1], kp.inv_scale);
     run_slots<kKeepIdx<PREC>, false>(t.run_slot, cur.r, cur.off, q);
-    mu[0] = L::ld(lam_next + n);
+    mu[0] = L::template ld<DEP>(lam_next + n);
 #pragma unroll
-    for (int j = 1; j < kQ; ++j) mu[j] = L::ld(lam_next + q.sl[inv(j) - 1]);
+    for (int j = 1; j < kQ; ++j) mu[j] = L::template ld<DEP>(lam_next + q.sl[inv(j) - 1]);
   } else {
     int m[18];
     node_entries<TAB, true>(t, n, m);
-    gather<PREC, false>(G, t.npad, n, m, d, kp.inv_scale, cc.abb_in, cc.abb_out, t.pressure);
-    mu[0] = L::ld(lam_next + n);
+    if (DEP) step_wait();
+    gather<PREC, false, false, DEP>(G, t.npad, n, m, d, kp.inv_scale, cc.abb_in, cc.abb_out, t.pressure);
+    mu[0] = L::template ld<DEP>(lam_next + n);
 #pragma unroll
     for (int j = 1; j < kQ; ++j) {
       const int mp = m[inv(j) - 1];
       const int dir = mp >= 0 ? j : inv(j);
       const int node = mp >= 0 ? mp : n;
-      const R v = L::ld(lam_next + at(dir, t.npad, node));
+      const R v = L::template ld<DEP>(lam_next + at(dir, t.npad, node));
       mu[j] = mp < -1 ? -v : v;
     }
   }
   R sa[10], da[10], drho, jx, jy, jz;
-  const R sn = DRAG ? R(__ldg(s + n)) : R(0);
+  const R sn = DRAG ? R(ld_grid<DEP>(s + n)) : R(0);
   if constexpr (std::is_same<R, double>::value) {
     // FP64: the whole step in fixed point (fx_adjoint) where every node of the
     // warp is in range.  It was bound by the FP64 pipe (about 160 instructions
@@ -456,22 +458,25 @@ int launch_adjoint_t(const lbm_lattice* L, const KParams& kp, const void* G, con
   const LT* ln = static_cast<const LT*>(lam_next);
   LT* lo = static_cast<LT*>(lam);
   const int N = int(L->N);
-  const bool lp1 = use_lp1<PREC>(kp);
-#define LBM_ADJ(T_)                                                                                             \
-  do {                                                                                                          \
-    if (s)                                                                                                      \
-      LBM_LAUNCH_LP1(k_adjoint, LBM_TARGS2(T_, true), (L->dev, kp, cc, ac, Gp, ln, lo, s, grad_s, N));          \
-    else                                                                                                        \
-      LBM_LAUNCH_LP1(k_adjoint, LBM_TARGS2(T_, false), (L->dev, kp, cc, ac, Gp, ln, lo, s, grad_s, N));         \
-  } while (0)
-  // lattices with pressure faces decode the adjacency entries in either table
-  if (!ria)
-    LBM_ADJ(dev::kAdjAny);
-  else if (table_kind(L, ria) == dev::kSlot)
-    LBM_ADJ(dev::kSlot);
-  else
-    LBM_ADJ(dev::kRunAny);
-#undef LBM_ADJ
+  // dependent launches as the OS-NT steps around it; without a run slot table,
+  // and with pressure faces, it reads the adjacency entries
+  by_dep<PREC, kFormOsnt>(L, [&](auto dep) {
+    auto go = [&](auto tab) {
+      by_bool(s != nullptr, [&](auto drag) {
+        by_lp1<PREC>(use_lp1<PREC>(kp), [&](auto lp1) {
+          constexpr bool kDep = decltype(dep)::value, kD = decltype(drag)::value;
+          launch_step<kDep>(dev::k_adjoint<PREC, kDep, decltype(tab)::value, kD, decltype(lp1)::value>, g, blk, st,
+                            L->dev, kp, cc, ac, Gp, ln, lo, s, grad_s, N);
+        });
+      });
+    };
+    if (!ria)
+      go(TableC<dev::kAdjAny>{});
+    else if (table_kind(L, ria) == dev::kSlot)
+      go(TableC<dev::kSlot>{});
+    else
+      go(TableC<dev::kRunAny>{});
+  });
   return cuda_check("adjoint step launch");
 }
 

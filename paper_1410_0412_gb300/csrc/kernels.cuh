@@ -86,6 +86,59 @@ template <bool LP1> struct MinCtasEt<LBM_F64_DF, LP1> { static constexpr int val
 template <bool LP1> struct MinCtasEt<LBM_F64, LP1> { static constexpr int value = LP1 ? 8 : 6; };
 static_assert(kBlock % kWarpNodes == 0, "a warp must cover one run-index group");
 
+// ---- programmatic dependent launch ---------------------------------------------------
+// A step kernel launched as a dependent one (DEP, see dependent_launch) may
+// start as soon as the last CTA of the kernel before it has ended, before that
+// kernel's results are complete: it finds its slots in the tables, which no
+// kernel writes, and then waits (step_wait) before it touches a grid, the drag
+// field or an adjoint array.  Launch latency, the flush of one step and the round
+// of table loads of the next overlap: 2 to 3 us a step.  No kernel triggers its
+// dependents early: with the trigger at the top of the kernels the 46 k-node box
+// took 3.5 us a step, without it 2.7 (5.1 as plain launches).  Behind the wait,
+// data is read with ld_dep: an ordinary load, never the non-coherent path, which
+// assumes data that is constant while the kernel runs, and volatile, so that it
+// stays there.
+__device__ __forceinline__ void step_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
+__device__ __forceinline__ double ld_dep(const double* p) {
+  double v;
+  asm volatile("ld.global.f64 %0, [%1];" : "=d"(v) : "l"(p));
+  return v;
+}
+__device__ __forceinline__ float ld_dep(const float* p) {
+  float v;
+  asm volatile("ld.global.f32 %0, [%1];" : "=f"(v) : "l"(p));
+  return v;
+}
+__device__ __forceinline__ __half ld_dep(const __half* p) {
+  unsigned short v;
+  asm volatile("ld.global.b16 %0, [%1];" : "=h"(v) : "l"(p));
+  return __ushort_as_half(v);
+}
+__device__ __forceinline__ __half2 ld_dep(const __half2* p) {
+  unsigned v;
+  asm volatile("ld.global.b32 %0, [%1];" : "=r"(v) : "l"(p));
+  return *reinterpret_cast<__half2*>(&v);
+}
+// DEP: behind step_wait; otherwise the non-coherent load.
+template <bool DEP, class V> __device__ __forceinline__ V ld_grid(const V* p) {
+  if constexpr (DEP)
+    return ld_dep(p);
+  else
+    return __ldg(p);
+}
+
+// Two scheduling fences of the DEP kernels, each kept where it measured faster.
+// slots_first: every slot is resolved before the first PDF load, so that the 19
+// loads leave back to back (OS-NT-R, 10 steps at 200^3 without -> with, us: FP64
+// 3217 -> 3106, FP32 1636 -> 1610, FP16S 1106 -> 1064; the AA odd step's stash
+// orders it already).
+__device__ __forceinline__ void slots_first() { asm volatile("bar.warp.sync %0;" ::"r"(__activemask()) : "memory"); }
+// kLoadsFirst: the collision starts after all 19 loads have been issued (a branch
+// that is never taken ends their basic block): FP64 AA-R at 200^3 3132 -> 3025 us,
+// FP32 OS-NT-R 1610 -> 1569; FP32 AA-R and FP16S lose 5-17 %.
+template <int PREC, bool AA> constexpr bool kLoadsFirst = AA ? PREC == LBM_F64 : PREC == LBM_F32;
+
 // ---- storage traits -----------------------------------------------------------------
 // Value stored for PDF i: f_i - w_i rho_s (rho_s = 0 when unshifted), in the
 // storage type; LBM_F16S additionally multiplies by the scale.
@@ -94,7 +147,7 @@ template <int PREC> struct St;
 template <> struct St<LBM_F64> {
   using T = double;
   using R = double;
-  static __device__ __forceinline__ R ld(const T* p, float) { return __ldg(p); }
+  template <bool DEP = false> static __device__ __forceinline__ R ld(const T* p, float) { return ld_grid<DEP>(p); }
   static __device__ __forceinline__ void st(T* p, R v, float) { *p = v; }
   static __device__ __forceinline__ void st_stream(T* p, R v, float) { __stcs(p, v); }
 };
@@ -103,7 +156,9 @@ template <> struct St<LBM_F64> {
 template <> struct St<LBM_F64_DF> {
   using T = double;
   using R = df;
-  static __device__ __forceinline__ R ld(const T* p, float) { return df_from_double(__ldg(p)); }
+  template <bool DEP = false> static __device__ __forceinline__ R ld(const T* p, float) {
+    return df_from_double(ld_grid<DEP>(p));
+  }
   static __device__ __forceinline__ void st(T* p, R v, float) { *p = double_from_df(v); }
   static __device__ __forceinline__ void st_stream(T* p, R v, float) { __stcs(p, double_from_df(v)); }
 };
@@ -111,7 +166,7 @@ template <> struct St<LBM_F64_DF> {
 template <> struct St<LBM_F32> {
   using T = float;
   using R = float;
-  static __device__ __forceinline__ R ld(const T* p, float) { return __ldg(p); }
+  template <bool DEP = false> static __device__ __forceinline__ R ld(const T* p, float) { return ld_grid<DEP>(p); }
   static __device__ __forceinline__ void st(T* p, R v, float) { *p = v; }
   static __device__ __forceinline__ void st_stream(T* p, R v, float) { __stcs(p, v); }
 };
@@ -119,8 +174,8 @@ template <> struct St<LBM_F32> {
 template <> struct St<LBM_F16S> {
   using T = __half;
   using R = float;
-  static __device__ __forceinline__ R ld(const T* p, float inv_scale) {
-    return __half2float(__ldg(p)) * inv_scale;
+  template <bool DEP = false> static __device__ __forceinline__ R ld(const T* p, float inv_scale) {
+    return __half2float(ld_grid<DEP>(p)) * inv_scale;
   }
   static __device__ __forceinline__ void st(T* p, R v, float scale) { *p = __float2half_rn(v * scale); }
   static __device__ __forceinline__ void st_stream(T* p, R v, float scale) {
@@ -419,12 +474,12 @@ template <int PREC> inline CollConst<typename St<PREC>::R> make_coll_step(const 
 
 // PDF loads and stores of the step kernels: storage units for LBM_F16S
 // (no scale), the storage traits otherwise.
-template <int PREC>
+template <int PREC, bool DEP = false>
 __device__ __forceinline__ typename St<PREC>::R ld_step(const typename St<PREC>::T* p, float inv_scale) {
   if constexpr (kScaled<PREC>)
-    return __half2float(__ldg(p));
+    return __half2float(ld_grid<DEP>(p));
   else
-    return St<PREC>::ld(p, inv_scale);
+    return St<PREC>::template ld<DEP>(p, inv_scale);
 }
 template <int PREC>
 __device__ __forceinline__ void st_step(typename St<PREC>::T* p, typename St<PREC>::R v, float scale) {
@@ -674,18 +729,19 @@ __device__ __forceinline__ bool warp_any(bool flag) { return __any_sync(__active
 //   AA grid after an odd count:      A[inv i][m]  | marker: A[i][n]
 // a pressure marker (-2 / -3) turns the bounce-back value v into
 // 2 w_i (rho_bc - rho_s) - v (anti-bounce-back, in deviation form).
-template <int PREC, bool AA_ODD, bool SC = false>
+template <int PREC, bool AA_ODD, bool SC = false, bool DEP = false>
 __device__ __forceinline__ void gather(const typename St<PREC>::T* g, uint32_t npad, int n, const int (&m)[18],
                                        typename St<PREC>::R (&d)[kQ], float inv_scale,
                                        const typename St<PREC>::R (&abb_in)[2],
                                        const typename St<PREC>::R (&abb_out)[2], int pressure) {
-  d[0] = SC ? ld_step<PREC>(g + n, inv_scale) : St<PREC>::ld(g + n, inv_scale);
+  d[0] = SC ? ld_step<PREC, DEP>(g + n, inv_scale) : St<PREC>::template ld<DEP>(g + n, inv_scale);
 #pragma unroll
   for (int i = 1; i < kQ; ++i) {
     const int mi = m[i - 1];
     const int dir = (mi >= 0) == AA_ODD ? inv(i) : i;
     const int node = mi >= 0 ? mi : n;
-    d[i] = SC ? ld_step<PREC>(g + at(dir, npad, node), inv_scale) : St<PREC>::ld(g + at(dir, npad, node), inv_scale);
+    const typename St<PREC>::T* p = g + at(dir, npad, node);
+    d[i] = SC ? ld_step<PREC, DEP>(p, inv_scale) : St<PREC>::template ld<DEP>(p, inv_scale);
   }
   if (pressure) {  // uniform: only lattices with pressure faces pay for the check
     bool face = false;
@@ -718,14 +774,15 @@ __device__ __forceinline__ void face_pull(const NodeSlots& q, V (&d)[kQ], const 
 }
 
 // The stored PDFs of a node through its slots (storage units for LBM_F16S).
-template <int PREC, int TAB>
-__device__ __forceinline__ void slot_pull(const KParams& kp, const CollConst<typename St<PREC>::R>& c,
-                                          const typename St<PREC>::T* g, int n, const NodeSlots& q,
-                                          typename St<PREC>::R (&d)[kQ]) {
-  d[0] = ld_step<PREC>(g + n, kp.inv_scale);
+template <int PREC, bool DEP, int TAB>
+__device__ __forceinline__ void slot_pull(const KParams& kp, const typename St<PREC>::R (&abb_in)[2],
+                                          const typename St<PREC>::R (&abb_out)[2], const typename St<PREC>::T* g,
+                                          int n, const NodeSlots& q, typename St<PREC>::R (&d)[kQ]) {
+  if (DEP) step_wait();
+  d[0] = ld_step<PREC, DEP>(g + n, kp.inv_scale);
 #pragma unroll
-  for (int i = 1; i < kQ; ++i) d[i] = ld_step<PREC>(g + q.sl[i - 1], kp.inv_scale);
-  face_pull<TAB>(q, d, c.abb_in, c.abb_out);
+  for (int i = 1; i < kQ; ++i) d[i] = ld_step<PREC, DEP>(g + q.sl[i - 1], kp.inv_scale);
+  face_pull<TAB>(q, d, abb_in, abb_out);
 }
 
 // Rows of the AA odd step's stash: the 18 slots, and the face masks.
@@ -766,7 +823,7 @@ template <int PREC, bool RIA> struct OsntBlock {
 
 // OS-NT step: pull (indirect) from src, collide, store locally into dst with
 // evict-first stores so the write stream does not push src out of L2.
-template <int PREC, int TAB, bool FORCE, bool DRAG, bool LP1 = false>
+template <int PREC, bool DEP, int TAB, bool FORCE, bool DRAG, bool LP1 = false>
 __global__ void __launch_bounds__(OsntBlock<PREC, is_run(TAB)>::value,
                                   ctas(MinCtasOsnt<PREC, is_run(TAB), LP1>::value, OsntBlock<PREC, is_run(TAB)>::value))
     k_osnt(DevTables t, KParams kp, CollConst<typename St<PREC>::R> c, const typename St<PREC>::T* __restrict__ src,
@@ -778,13 +835,16 @@ __global__ void __launch_bounds__(OsntBlock<PREC, is_run(TAB)>::value,
   if constexpr (is_any(TAB)) {
     int m[18];
     node_entries<TAB, kKeepIdx<PREC>>(t, n, m);
-    gather<PREC, false, kScaled<PREC>>(src, t.npad, n, m, d, kp.inv_scale, c.abb_in, c.abb_out, t.pressure);
+    if (DEP) step_wait();
+    gather<PREC, false, kScaled<PREC>, DEP>(src, t.npad, n, m, d, kp.inv_scale, c.abb_in, c.abb_out, t.pressure);
   } else {
     NodeSlots q;
     node_slots<TAB, false, kKeepIdx<PREC>>(t, n, q);
-    slot_pull<PREC, TAB>(kp, c, src, n, q, d);
+    if (DEP) slots_first();
+    slot_pull<PREC, DEP, TAB>(kp, c.abb_in, c.abb_out, src, n, q, d);
+    if (DEP && kLoadsFirst<PREC, false> && t.npad == 0u) return;
   }
-  const R sn = DRAG ? R(__ldg(s + n)) : R(0);
+  const R sn = DRAG ? R(ld_grid<DEP>(s + n)) : R(0);
   collide<R, FORCE, DRAG, LP1, kScaled<PREC>>(d, c, sn);
 #pragma unroll
   for (int i = 0; i < kQ; ++i) st_stream_step<PREC>(dst + at(i, t.npad, n), d[i], kp.scale);
@@ -792,7 +852,7 @@ __global__ void __launch_bounds__(OsntBlock<PREC, is_run(TAB)>::value,
 
 // AA even step: direct read of the 19 local PDFs, collide, write to the
 // opposite local slots (no index loads at all).
-template <int PREC, bool FORCE, bool DRAG, bool LP1 = false>
+template <int PREC, bool DEP, bool FORCE, bool DRAG, bool LP1 = false>
 __global__ void __launch_bounds__(kBlock, ctas(MinCtasEven<PREC, LP1>::value)) k_aa_even(DevTables t, KParams kp, CollConst<typename St<PREC>::R> c,
                                                     typename St<PREC>::T* __restrict__ A,
                                                     const float* __restrict__ s, int N) {
@@ -800,9 +860,11 @@ __global__ void __launch_bounds__(kBlock, ctas(MinCtasEven<PREC, LP1>::value)) k
   const int n = blockIdx.x * kBlock + threadIdx.x;
   if (n >= N) return;
   R d[kQ];
+  if (DEP) step_wait();
 #pragma unroll
-  for (int i = 0; i < kQ; ++i) d[i] = ld_step<PREC>(A + at(i, t.npad, n), kp.inv_scale);
-  const R sn = DRAG ? R(__ldg(s + n)) : R(0);
+  for (int i = 0; i < kQ; ++i) d[i] = ld_step<PREC, DEP>(A + at(i, t.npad, n), kp.inv_scale);
+  if (DEP && kLoadsFirst<PREC, true> && t.npad == 0u) return;
+  const R sn = DRAG ? R(ld_grid<DEP>(s + n)) : R(0);
   collide<R, FORCE, DRAG, LP1, kScaled<PREC>>(d, c, sn);
 #pragma unroll
   for (int i = 0; i < kQ; ++i) st_step<PREC>(A + at(inv(i), t.npad, n), d[i], kp.scale);
@@ -813,21 +875,22 @@ __global__ void __launch_bounds__(kBlock, ctas(MinCtasEven<PREC, LP1>::value)) k
 // of the one-node form (Npad is a multiple of 128, so every pair is aligned;
 // a pair's second node may lie past N: it is loaded and computed but not
 // stored).
-template <bool FORCE, bool DRAG>
+template <bool DEP, bool FORCE, bool DRAG>
 __global__ void __launch_bounds__(kBlock) k_aa_even_h2(DevTables t, KParams kp, CollConst<float> c,
                                                        __half* __restrict__ A, const float* __restrict__ s,
                                                        int N) {
   const int n = 2 * (blockIdx.x * kBlock + threadIdx.x);
   if (n >= N) return;
   float d0[kQ], d1[kQ];
+  if (DEP) step_wait();
 #pragma unroll
   for (int i = 0; i < kQ; ++i) {
-    const float2 v = __half22float2(__ldg(reinterpret_cast<const __half2*>(A + at(i, t.npad, n))));
+    const float2 v = __half22float2(ld_grid<DEP>(reinterpret_cast<const __half2*>(A + at(i, t.npad, n))));
     d0[i] = v.x;  // storage units: the scale is folded into c (make_coll_step)
     d1[i] = v.y;
   }
-  const float s0 = DRAG ? __ldg(s + n) : 0.0f;
-  const float s1 = DRAG ? (n + 1 < N ? __ldg(s + n + 1) : 0.0f) : 0.0f;
+  const float s0 = DRAG ? ld_grid<DEP>(s + n) : 0.0f;
+  const float s1 = DRAG ? (n + 1 < N ? ld_grid<DEP>(s + n + 1) : 0.0f) : 0.0f;
   collide<float, FORCE, DRAG, false, true>(d0, c, s0);
   collide<float, FORCE, DRAG, false, true>(d1, c, s1);
   // the pair's second node may lie past N (odd N): write node slots only, as
@@ -862,7 +925,7 @@ __device__ __forceinline__ void collide_odd_df(const double (&g64)[kQ], const Co
 
 // AA odd step: read f_i from the neighbour's opposite slot A[inv i][m_i], collide,
 // write p_i to A[i][m_{inv i}] -- the same 19 slots, so in place and race-free.
-template <int PREC, int TAB, bool FORCE, bool DRAG, bool LP1 = false>
+template <int PREC, bool DEP, int TAB, bool FORCE, bool DRAG, bool LP1 = false>
 __global__ void __launch_bounds__(kBlock, ctas(MinCtasOdd<PREC, is_run(TAB), LP1>::value)) k_aa_odd(DevTables t, KParams kp,
                                                                               CollConst<typename St<PREC>::R> c,
                                                                               typename St<PREC>::T* __restrict__ A,
@@ -876,22 +939,20 @@ __global__ void __launch_bounds__(kBlock, ctas(MinCtasOdd<PREC, is_run(TAB), LP1
   int* const sm = &s_m[0][threadIdx.x];
   const int n = blockIdx.x * kBlock + threadIdx.x;
   if (n >= N) return;
-  const R sn = DRAG ? R(__ldg(s + n)) : R(0);
   R d[kQ];
   if constexpr (!is_any(TAB)) {
     NodeSlots q;
     node_slots<TAB, true, kKeepIdx<PREC>>(t, n, q, sm);
     stash_faces<TAB>(q, sm);
     if constexpr (PREC == LBM_F64_DF) {
-      const double* g = reinterpret_cast<const double*>(A);
       double g64[kQ];
-      g64[0] = __ldg(g + n);
-#pragma unroll
-      for (int i = 1; i < kQ; ++i) g64[i] = __ldg(g + q.sl[i - 1]);
-      face_pull<TAB>(q, g64, c.abb64_in, c.abb64_out);
+      slot_pull<LBM_F64, DEP, TAB>(kp, c.abb64_in, c.abb64_out, reinterpret_cast<const double*>(A), n, q, g64);
+      const R sn = DRAG ? R(ld_grid<DEP>(s + n)) : R(0);
       collide_odd_df<FORCE, DRAG, LP1>(g64, c, sn, d);
     } else {
-      slot_pull<PREC, TAB>(kp, c, A, n, q, d);
+      slot_pull<PREC, DEP, TAB>(kp, c.abb_in, c.abb_out, A, n, q, d);
+      if (DEP && kLoadsFirst<PREC, true> && t.npad == 0u) return;
+      const R sn = DRAG ? R(ld_grid<DEP>(s + n)) : R(0);
       collide<R, FORCE, DRAG, LP1, kScaled<PREC>>(d, c, sn);
     }
     slot_push<PREC, TAB>(kp, c, A, n, sm, d);
@@ -900,13 +961,15 @@ __global__ void __launch_bounds__(kBlock, ctas(MinCtasOdd<PREC, is_run(TAB), LP1
     node_entries<TAB, kKeepIdx<PREC>>(t, n, m);
 #pragma unroll
     for (int j = 0; j < 18; ++j) sm[j * kBlock] = m[j];
+    if (DEP) step_wait();
+    const R sn = DRAG ? R(ld_grid<DEP>(s + n)) : R(0);
     if constexpr (PREC == LBM_F64_DF) {
       double g64[kQ];
-      gather<LBM_F64, true>(reinterpret_cast<const double*>(A), t.npad, n, m, g64, kp.inv_scale, c.abb64_in,
+      gather<LBM_F64, true, false, DEP>(reinterpret_cast<const double*>(A), t.npad, n, m, g64, kp.inv_scale, c.abb64_in,
                             c.abb64_out, t.pressure);
       collide_odd_df<FORCE, DRAG, LP1>(g64, c, sn, d);
     } else {
-      gather<PREC, true, kScaled<PREC>>(A, t.npad, n, m, d, kp.inv_scale, c.abb_in, c.abb_out, t.pressure);
+      gather<PREC, true, kScaled<PREC>, DEP>(A, t.npad, n, m, d, kp.inv_scale, c.abb_in, c.abb_out, t.pressure);
       collide<R, FORCE, DRAG, LP1, kScaled<PREC>>(d, c, sn);
     }
     st_step<PREC>(A + n, d[0], kp.scale);
@@ -946,7 +1009,7 @@ __global__ void __launch_bounds__(kBlock, ctas(MinCtasOdd<PREC, is_run(TAB), LP1
 #ifndef LBM_MIN_CTAS_ODD_X2
 #define LBM_MIN_CTAS_ODD_X2 8
 #endif
-template <int PREC, int TAB, bool FORCE, bool DRAG>
+template <int PREC, bool DEP, int TAB, bool FORCE, bool DRAG>
 __global__ void __launch_bounds__(kBlock, ctas(LBM_MIN_CTAS_ODD_X2)) k_aa_odd_x2(DevTables t, KParams kp,
                                                                          CollConst<typename St<PREC>::R> c,
                                                                          typename St<PREC>::T* __restrict__ A,
@@ -974,21 +1037,22 @@ __global__ void __launch_bounds__(kBlock, ctas(LBM_MIN_CTAS_ODD_X2)) k_aa_odd_x2
     }
     stash_faces<TAB>(q0, sm0);
     stash_faces<TAB>(q1, sm1);
-    d0[0] = ld_step<PREC>(A + n0, kp.inv_scale);
-    d1[0] = ld_step<PREC>(A + (has1 ? n1 : n0), kp.inv_scale);
+    if (DEP) step_wait();
+    d0[0] = ld_step<PREC, DEP>(A + n0, kp.inv_scale);
+    d1[0] = ld_step<PREC, DEP>(A + (has1 ? n1 : n0), kp.inv_scale);
 #pragma unroll
     for (int i = 1; i < kQ; ++i) {
-      d0[i] = ld_step<PREC>(A + q0.sl[i - 1], kp.inv_scale);
-      d1[i] = ld_step<PREC>(A + q1.sl[i - 1], kp.inv_scale);
+      d0[i] = ld_step<PREC, DEP>(A + q0.sl[i - 1], kp.inv_scale);
+      d1[i] = ld_step<PREC, DEP>(A + q1.sl[i - 1], kp.inv_scale);
     }
     face_pull<TAB>(q0, d0, c.abb_in, c.abb_out);
     face_pull<TAB>(q1, d1, c.abb_in, c.abb_out);
   }
-  const R s0 = DRAG ? R(__ldg(s + n0)) : R(0);
+  const R s0 = DRAG ? R(ld_grid<DEP>(s + n0)) : R(0);
   collide<R, FORCE, DRAG, false, kScaled<PREC>>(d0, c, s0);
   slot_push<PREC, TAB>(kp, c, A, n0, sm0, d0);
   if (has1) {
-    const R s1 = DRAG ? R(__ldg(s + n1)) : R(0);
+    const R s1 = DRAG ? R(ld_grid<DEP>(s + n1)) : R(0);
     collide<R, FORCE, DRAG, false, kScaled<PREC>>(d1, c, s1);
     slot_push<PREC, TAB>(kp, c, A, n1, sm1, d1);
   }
@@ -1043,7 +1107,7 @@ __device__ __forceinline__ unsigned et_locate(const DevTables& t, int n, int (&l
   return __ldg(t.et_run_mask + c.r);
 }
 
-template <int PREC, bool RIA, bool ODD, bool FORCE, bool DRAG, bool LP1 = false>
+template <int PREC, bool DEP, bool RIA, bool ODD, bool FORCE, bool DRAG, bool LP1 = false>
 __global__ void __launch_bounds__(kBlock, ctas(MinCtasEt<PREC, LP1>::value)) k_et(DevTables t, KParams kp,
                                                                           CollConst<typename St<PREC>::R> c,
                                                                           typename St<PREC>::T* __restrict__ A,
@@ -1059,16 +1123,17 @@ __global__ void __launch_bounds__(kBlock, ctas(MinCtasEt<PREC, LP1>::value)) k_e
   int loc[7];
   unsigned mask = et_locate<RIA>(t, n, loc);
   R d[kQ];
-  d[0] = ld_step<PREC>(A + n, kp.inv_scale);
+  if (DEP) step_wait();
+  d[0] = ld_step<PREC, DEP>(A + n, kp.inv_scale);
 #pragma unroll
   for (int i = 1; i < kQ; ++i)
-    d[i] = ld_step<PREC>(A + at(ODD ? inv(i) : i, t.spad, loc[et_row(inv(i)) + 1]), kp.inv_scale);
+    d[i] = ld_step<PREC, DEP>(A + at(ODD ? inv(i) : i, t.spad, loc[et_row(inv(i)) + 1]), kp.inv_scale);
   if (kStash) {
 #pragma unroll
     for (int k = 1; k < 7; ++k) s_loc[k - 1][threadIdx.x] = loc[k];
     s_loc[6][threadIdx.x] = int(mask);
   }
-  const R sn = DRAG ? R(__ldg(s + n)) : R(0);
+  const R sn = DRAG ? R(ld_grid<DEP>(s + n)) : R(0);
   collide<R, FORCE, DRAG, LP1, kScaled<PREC>>(d, c, sn);
   st_step<PREC>(A + n, d[0], kp.scale);
   if (kStash) {
@@ -1468,21 +1533,6 @@ inline int table_kind(const lbm_lattice* L, int ria) {
   return wide || L->dev.pressure ? dev::kAdjAny : dev::kAdj;
 }
 
-// Run BODY(TAB) for the lattice's table; SLOTS: whether the kernel has the run
-// slot instantiations.
-#define LBM_BY_TABLE(BODY, SLOTS)                           \
-  switch (table_kind(L, ria)) {                             \
-    case dev::kSlot:                                        \
-      if constexpr (SLOTS) BODY(dev::kSlot);                \
-      break;                                                \
-    case dev::kSlotFace:                                    \
-      if constexpr (SLOTS) BODY(dev::kSlotFace);            \
-      break;                                                \
-    case dev::kAdj: BODY(dev::kAdj); break;                 \
-    case dev::kRunAny: BODY(dev::kRunAny); break;           \
-    default: BODY(dev::kAdjAny); break;                     \
-  }
-
 inline bool has_force(const KParams& kp) { return kp.g[0] != 0.0 || kp.g[1] != 0.0 || kp.g[2] != 0.0; }
 
 // The l+ = 1 collision (see collide) is instantiated for the FP64-storage
@@ -1491,21 +1541,86 @@ inline bool has_force(const KParams& kp) { return kp.g[0] != 0.0 || kp.g[1] != 0
 template <int PREC> constexpr bool kLp1Path = PREC == LBM_F64 || PREC == LBM_F64_DF;
 template <int PREC> inline bool use_lp1(const KParams& kp) { return kLp1Path<PREC> && kp.lp == 1.0; }
 
-// Launch KERNEL<PREC, ARGS..., LP1> with LP1 = lp1 where that instantiation
-// exists, on grid g of blk-thread CTAs.
-#define LBM_LAUNCH_LP1(KERNEL, TARGS, LAUNCH_ARGS)                             \
-  do {                                                                         \
-    if constexpr (kLp1Path<PREC>) {                                            \
-      if (lp1) {                                                               \
-        dev::KERNEL<PREC, TARGS, true><<<g, blk, 0, st>>> LAUNCH_ARGS;         \
-        break;                                                                 \
-      }                                                                        \
-    }                                                                          \
-    dev::KERNEL<PREC, TARGS, false><<<g, blk, 0, st>>> LAUNCH_ARGS;            \
-  } while (0)
-#define LBM_TARGS3(A_, B_, C_) A_, B_, C_
-#define LBM_TARGS4(A_, B_, C_, D_) A_, B_, C_, D_
-#define LBM_TARGS2(A_, B_) A_, B_
+// Which steps are launched as dependent kernels.  FP64 and the two-grid and
+// Esoteric Twist steps of FP32, and OS-NT of FP16S: always, faster at every size
+// measured (10 steps, plain -> dependent, us, on beds of 96^3 / 200^3: FP64 AA-R
+// 383 -> 359 / 3040 -> 3025, OS-NT-R 412 -> 371 / 3207 -> 3106; FP32 OS-NT-R
+// 188 -> 157 / 1638 -> 1569, ET-R 204 -> 178 / 2146 -> 2104; FP16S OS-NT-R 127 ->
+// 118 / 1089 -> 1064).  The others lose the non-coherent loads, 1-3 % of a large
+// step, and are dependent when a step moves at most 256 MB of PDFs: FP32 AA-R
+// 151 -> 132 at 83 MB, 424 -> 412 at 198, 805 -> 804 at 386, 1570 -> 1591 at 754;
+// FP16S AA-R 123 -> 98 at 42, 507 -> 498 at 193, 960 -> 969 at 377; FP16S ET-R
+// 398 -> 371 at 99, 1657 -> 1685 at 377.  The double-float steps are plain.
+enum Form { kFormOsnt, kFormAa, kFormEt };
+template <int PREC, int FORM>
+constexpr int kDependent = PREC == LBM_F64_DF                                                                  ? 0
+                           : PREC == LBM_F64 || (PREC == LBM_F32 && FORM != kFormAa) || FORM == kFormOsnt ? 2
+                                                                                                            : 1;
+// f gets DEP as the rule says.
+template <int PREC, int FORM, class F> inline void by_dep(const lbm_lattice* L, F f) {
+  if constexpr (kDependent<PREC, FORM> == 0)
+    f(std::false_type{});
+  else if constexpr (kDependent<PREC, FORM> == 2)
+    f(std::true_type{});
+  else if (2 * kQ * int64_t(sizeof(typename dev::St<PREC>::T)) * L->N <= (int64_t(256) << 20))
+    f(std::true_type{});
+  else
+    f(std::false_type{});
+}
+
+// Launch of a step kernel.
+template <bool DEP, class... P, class... A>
+inline void launch_step(void (*k)(P...), unsigned g, unsigned b, cudaStream_t st, A... a) {
+  if constexpr (!DEP) {
+    k<<<g, b, 0, st>>>(static_cast<P>(a)...);
+    return;
+  }
+  cudaLaunchAttribute attr;
+  attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr.val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(g);
+  cfg.blockDim = dim3(b);
+  cfg.stream = st;
+  cfg.attrs = &attr;
+  cfg.numAttrs = 1;
+  cudaLaunchKernelEx(&cfg, k, static_cast<P>(a)...);
+}
+
+// Compile-time choices from run-time values: f gets std::integral_constants.
+template <class F> inline void by_bool(bool v, F f) {
+  if (v)
+    f(std::true_type{});
+  else
+    f(std::false_type{});
+}
+// (FORCE, DRAG) of a step: the drag kernels hold the force as well.
+template <class F> inline void by_terms(bool drag, bool force, F f) {
+  if (drag)
+    f(std::true_type{}, std::true_type{});
+  else if (force)
+    f(std::true_type{}, std::false_type{});
+  else
+    f(std::false_type{}, std::false_type{});
+}
+// LP1 where that instantiation exists.
+template <int PREC, class F> inline void by_lp1(bool lp1, F f) {
+  if constexpr (kLp1Path<PREC>)
+    by_bool(lp1, f);
+  else
+    f(std::false_type{});
+}
+// TAB: the lattice's table.
+template <int T> using TableC = std::integral_constant<int, T>;
+template <class F> inline void by_table(int tab, F f) {
+  switch (tab) {
+    case dev::kSlot: f(TableC<dev::kSlot>{}); break;
+    case dev::kSlotFace: f(TableC<dev::kSlotFace>{}); break;
+    case dev::kAdj: f(TableC<dev::kAdj>{}); break;
+    case dev::kRunAny: f(TableC<dev::kRunAny>{}); break;
+    default: f(TableC<dev::kAdjAny>{}); break;
+  }
+}
 
 template <int PREC>
 int launch_osnt_t(const lbm_lattice* L, const KParams& kp, const void* src, void* dst, const float* s, int ria,
@@ -1517,20 +1632,18 @@ int launch_osnt_t(const lbm_lattice* L, const KParams& kp, const void* src, void
   const T* a = static_cast<const T*>(src);
   T* b = static_cast<T*>(dst);
   const int N = int(L->N);
-  const bool f = has_force(kp);
   const auto c = dev::make_coll_step<PREC>(kp);
-  const bool lp1 = use_lp1<PREC>(kp);
-#define LBM_OSNT(T_)                                                                                    \
-  do {                                                                                                  \
-    if (s)                                                                                              \
-      LBM_LAUNCH_LP1(k_osnt, LBM_TARGS3(T_, true, true), (L->dev, kp, c, a, b, s, N));                  \
-    else if (f)                                                                                         \
-      LBM_LAUNCH_LP1(k_osnt, LBM_TARGS3(T_, true, false), (L->dev, kp, c, a, b, s, N));                 \
-    else                                                                                                \
-      LBM_LAUNCH_LP1(k_osnt, LBM_TARGS3(T_, false, false), (L->dev, kp, c, a, b, s, N));                \
-  } while (0)
-  LBM_BY_TABLE(LBM_OSNT, true)
-#undef LBM_OSNT
+  by_dep<PREC, kFormOsnt>(L, [&](auto dep) {
+    by_table(table_kind(L, ria), [&](auto tab) {
+      by_terms(s != nullptr, has_force(kp), [&](auto force, auto drag) {
+        by_lp1<PREC>(use_lp1<PREC>(kp), [&](auto lp1) {
+          constexpr bool kDep = decltype(dep)::value, kF = decltype(force)::value, kD = decltype(drag)::value;
+          launch_step<kDep>(dev::k_osnt<PREC, kDep, decltype(tab)::value, kF, kD, decltype(lp1)::value>, g, blk, st,
+                            L->dev, kp, c, a, b, s, N);
+        });
+      });
+    });
+  });
   return cuda_check("OS-NT step launch");
 }
 
@@ -1539,58 +1652,40 @@ int launch_aa_t(const lbm_lattice* L, const KParams& kp, void* pdf, int parity, 
                 void* stream) {
   using T = typename dev::St<PREC>::T;
   auto st = static_cast<cudaStream_t>(stream);
-  const unsigned blk = dev::kBlock;
-  const unsigned g = grid_of(L->N);
   T* A = static_cast<T*>(pdf);
   const int N = int(L->N);
-  const bool f = has_force(kp);
-  const bool lp1 = use_lp1<PREC>(kp);
+  const unsigned blk = dev::kBlock, g = grid_of(L->N), g2 = unsigned((L->N + 2 * blk - 1) / (2 * blk));
   const auto c = dev::make_coll_step<PREC>(kp);
-  if constexpr (PREC == LBM_F16S) {
-    if (parity == 0) {
-    const unsigned g2 = unsigned((L->N + 2 * dev::kBlock - 1) / (2 * dev::kBlock));
-    __half* H = reinterpret_cast<__half*>(pdf);
-    const auto cf = dev::make_coll_step<LBM_F16S>(kp);
-    if (s) dev::k_aa_even_h2<true, true><<<g2, dev::kBlock, 0, st>>>(L->dev, kp, cf, H, s, N);
-    else if (f) dev::k_aa_even_h2<true, false><<<g2, dev::kBlock, 0, st>>>(L->dev, kp, cf, H, s, N);
-    else dev::k_aa_even_h2<false, false><<<g2, dev::kBlock, 0, st>>>(L->dev, kp, cf, H, s, N);
-    return cuda_check("AA even step launch");
-    }
-  }
   if (parity == 0) {
-    if (s) LBM_LAUNCH_LP1(k_aa_even, LBM_TARGS2(true, true), (L->dev, kp, c, A, s, N));
-    else if (f) LBM_LAUNCH_LP1(k_aa_even, LBM_TARGS2(true, false), (L->dev, kp, c, A, s, N));
-    else LBM_LAUNCH_LP1(k_aa_even, LBM_TARGS2(false, false), (L->dev, kp, c, A, s, N));
+    by_dep<PREC, kFormAa>(L, [&](auto dep) {
+      by_terms(s != nullptr, has_force(kp), [&](auto force, auto drag) {
+        constexpr bool kDep = decltype(dep)::value, kF = decltype(force)::value, kD = decltype(drag)::value;
+        if constexpr (PREC == LBM_F16S)
+          launch_step<kDep>(dev::k_aa_even_h2<kDep, kF, kD>, g2, blk, st, L->dev, kp, c, A, s, N);
+        else
+          by_lp1<PREC>(use_lp1<PREC>(kp), [&](auto lp1) {
+            launch_step<kDep>(dev::k_aa_even<PREC, kDep, kF, kD, decltype(lp1)::value>, g, blk, st, L->dev, kp, c, A,
+                              s, N);
+          });
+      });
+    });
     return cuda_check("AA even step launch");
   }
-  if constexpr (PREC == LBM_F32) {
-    if (ria && L->dev.run_slot) {
-      const unsigned g2 = unsigned((L->N + 2 * dev::kBlock - 1) / (2 * dev::kBlock));
-#define LBM_AAODD2(T_)                                                                                   \
-  do {                                                                                                   \
-    if (s) dev::k_aa_odd_x2<PREC, T_, true, true><<<g2, dev::kBlock, 0, st>>>(L->dev, kp, c, A, s, N);   \
-    else if (f) dev::k_aa_odd_x2<PREC, T_, true, false><<<g2, dev::kBlock, 0, st>>>(L->dev, kp, c, A, s, N); \
-    else dev::k_aa_odd_x2<PREC, T_, false, false><<<g2, dev::kBlock, 0, st>>>(L->dev, kp, c, A, s, N);   \
-  } while (0)
-      if (L->dev.pressure)
-        LBM_AAODD2(dev::kSlotFace);
-      else
-        LBM_AAODD2(dev::kSlot);
-#undef LBM_AAODD2
-      return cuda_check("AA odd step launch");
-    }
-  }
-#define LBM_AAODD(T_)                                                                                   \
-  do {                                                                                                  \
-    if (s)                                                                                              \
-      LBM_LAUNCH_LP1(k_aa_odd, LBM_TARGS3(T_, true, true), (L->dev, kp, c, A, s, N));                   \
-    else if (f)                                                                                         \
-      LBM_LAUNCH_LP1(k_aa_odd, LBM_TARGS3(T_, true, false), (L->dev, kp, c, A, s, N));                  \
-    else                                                                                                \
-      LBM_LAUNCH_LP1(k_aa_odd, LBM_TARGS3(T_, false, false), (L->dev, kp, c, A, s, N));                 \
-  } while (0)
-  LBM_BY_TABLE(LBM_AAODD, (PREC != LBM_F32))  // FP32 took k_aa_odd_x2 above
-#undef LBM_AAODD
+  by_dep<PREC, kFormAa>(L, [&](auto dep) {
+    by_table(table_kind(L, ria), [&](auto tab) {
+      by_terms(s != nullptr, has_force(kp), [&](auto force, auto drag) {
+        constexpr bool kDep = decltype(dep)::value, kF = decltype(force)::value, kD = decltype(drag)::value;
+        constexpr int kTab = decltype(tab)::value;
+        if constexpr (PREC == LBM_F32 && (kTab == dev::kSlot || kTab == dev::kSlotFace))
+          launch_step<kDep>(dev::k_aa_odd_x2<PREC, kDep, kTab, kF, kD>, g2, blk, st, L->dev, kp, c, A, s, N);
+        else
+          by_lp1<PREC>(use_lp1<PREC>(kp), [&](auto lp1) {
+            launch_step<kDep>(dev::k_aa_odd<PREC, kDep, kTab, kF, kD, decltype(lp1)::value>, g, blk, st, L->dev, kp,
+                              c, A, s, N);
+          });
+      });
+    });
+  });
   return cuda_check("AA odd step launch");
 }
 
@@ -1599,30 +1694,24 @@ int launch_et_t(const lbm_lattice* L, const KParams& kp, void* pdf, int parity, 
                 void* stream) {
   using T = typename dev::St<PREC>::T;
   auto st = static_cast<cudaStream_t>(stream);
-  const unsigned blk = dev::kBlock;
   const unsigned g = grid_of(L->N);
   T* A = static_cast<T*>(pdf);
   const int N = int(L->N);
-  const bool f = has_force(kp);
   const auto c = dev::make_coll_step<PREC>(kp);
-  const bool lp1 = use_lp1<PREC>(kp);
-#define LBM_ET(R_, O_, F_, D_) LBM_LAUNCH_LP1(k_et, LBM_TARGS4(R_, O_, F_, D_), (L->dev, kp, c, A, s, N))
-#define LBM_ET_R(O_, F_, D_) \
-  do {                       \
-    if (ria)                 \
-      LBM_ET(true, O_, F_, D_); \
-    else                     \
-      LBM_ET(false, O_, F_, D_); \
-  } while (0)
-  if (s) {
-    if (parity) LBM_ET_R(true, true, true); else LBM_ET_R(false, true, true);
-  } else if (f) {
-    if (parity) LBM_ET_R(true, true, false); else LBM_ET_R(false, true, false);
-  } else {
-    if (parity) LBM_ET_R(true, false, false); else LBM_ET_R(false, false, false);
-  }
-#undef LBM_ET_R
-#undef LBM_ET
+  by_dep<PREC, kFormEt>(L, [&](auto dep) {
+    by_bool(ria != 0, [&](auto run) {
+      by_bool(parity != 0, [&](auto odd) {
+        by_terms(s != nullptr, has_force(kp), [&](auto force, auto drag) {
+          by_lp1<PREC>(use_lp1<PREC>(kp), [&](auto lp1) {
+            constexpr bool kDep = decltype(dep)::value, kF = decltype(force)::value, kD = decltype(drag)::value;
+            launch_step<kDep>(
+                dev::k_et<PREC, kDep, decltype(run)::value, decltype(odd)::value, kF, kD, decltype(lp1)::value>, g,
+                dev::kBlock, st, L->dev, kp, c, A, s, N);
+          });
+        });
+      });
+    });
+  });
   return cuda_check("Esoteric Twist step launch");
 }
 
@@ -1706,19 +1795,19 @@ int launch_macroscopic_t(const lbm_lattice* L, const KParams& kp, const void* pd
   return LBM_OK;
 }
 
-#define LBM_INSTANTIATE_STEP_LAUNCHERS(P)                                                                          \
-  template int launch_osnt_t<P>(const lbm_lattice*, const KParams&, const void*, void*, const float*, int, void*); \
-  template int launch_aa_t<P>(const lbm_lattice*, const KParams&, void*, int, const float*, int, void*);           \
+// Explicit instantiations, one translation unit each (kernels_*.cu) so that
+// they compile in parallel.
+#define LBM_INSTANTIATE_OSNT(P) \
+  template int launch_osnt_t<P>(const lbm_lattice*, const KParams&, const void*, void*, const float*, int, void*);
+#define LBM_INSTANTIATE_AA(P) \
+  template int launch_aa_t<P>(const lbm_lattice*, const KParams&, void*, int, const float*, int, void*);
+#define LBM_INSTANTIATE_ET(P) \
   template int launch_et_t<P>(const lbm_lattice*, const KParams&, void*, int, const float*, int, void*);
-
-#define LBM_INSTANTIATE_LAUNCHERS(P)                                                                               \
-  template int launch_osnt_t<P>(const lbm_lattice*, const KParams&, const void*, void*, const float*, int, void*); \
-  template int launch_aa_t<P>(const lbm_lattice*, const KParams&, void*, int, const float*, int, void*);           \
-  template int launch_et_t<P>(const lbm_lattice*, const KParams&, void*, int, const float*, int, void*);                \
-  template int launch_init_eq_t<P>(const lbm_lattice*, const KParams&, void*, int, double, const double*, void*);  \
-  template int launch_load_canonical_t<P>(const lbm_lattice*, const KParams&, const double*, void*, int, void*);   \
-  template int launch_canonical_t<P>(const lbm_lattice*, const KParams&, const void*, int, double*, void*);        \
-  template int launch_macroscopic_t<P>(const lbm_lattice*, const KParams&, const void*, int, const float*,          \
+#define LBM_INSTANTIATE_STATE(P)                                                                                  \
+  template int launch_init_eq_t<P>(const lbm_lattice*, const KParams&, void*, int, double, const double*, void*); \
+  template int launch_load_canonical_t<P>(const lbm_lattice*, const KParams&, const double*, void*, int, void*);  \
+  template int launch_canonical_t<P>(const lbm_lattice*, const KParams&, const void*, int, double*, void*);       \
+  template int launch_macroscopic_t<P>(const lbm_lattice*, const KParams&, const void*, int, const float*,        \
                                        double*, double*, double*, double*, int64_t, void*);
 
 }  // namespace lbm
