@@ -74,6 +74,8 @@ template <bool LP1> struct MinCtasEven<LBM_F64_DF, LP1> { static constexpr int v
 #ifndef LBM_MIN_CTAS_ODD_RIA_F16
 #define LBM_MIN_CTAS_ODD_RIA_F16 12
 #endif
+// (the FP16 step with pressure faces, FP16S foam of 7.7 M nodes, 10 steps at 10 /
+// 12 / 14 / 16: 1225 / 1197 / 1169 / 1168 us)
 template <int PREC, bool RIA, bool LP1> struct MinCtasOdd { static constexpr int value = RIA ? LBM_MIN_CTAS_ODD_RIA : 8; };
 template <bool RIA, bool LP1> struct MinCtasOdd<LBM_F16S, RIA, LP1> { static constexpr int value = RIA ? LBM_MIN_CTAS_ODD_RIA_F16 : 8; };
 template <bool RIA, bool LP1> struct MinCtasOdd<LBM_F64, RIA, LP1> { static constexpr int value = LP1 ? 8 : 6; };
@@ -926,7 +928,9 @@ __device__ __forceinline__ void collide_odd_df(const double (&g64)[kQ], const Co
 // AA odd step: read f_i from the neighbour's opposite slot A[inv i][m_i], collide,
 // write p_i to A[i][m_{inv i}] -- the same 19 slots, so in place and race-free.
 template <int PREC, bool DEP, int TAB, bool FORCE, bool DRAG, bool LP1 = false>
-__global__ void __launch_bounds__(kBlock, ctas(MinCtasOdd<PREC, is_run(TAB), LP1>::value)) k_aa_odd(DevTables t, KParams kp,
+__global__ void __launch_bounds__(kBlock, ctas(PREC == LBM_F16S && TAB == kSlotFace
+                                                   ? 14
+                                                   : MinCtasOdd<PREC, is_run(TAB), LP1>::value)) k_aa_odd(DevTables t, KParams kp,
                                                                               CollConst<typename St<PREC>::R> c,
                                                                               typename St<PREC>::T* __restrict__ A,
                                                                               const float* __restrict__ s, int N) {
