@@ -36,7 +36,7 @@ template <class R> struct AdjConst {
   R nk18ap, k6ap;           // -18 a+, 6 a+
   R k3am, nk3am;            // 3 a-, -3 a-
   bool gx;                  // the body force points along x (g_y = g_z = 0)
-  FxAdj fx;                 // constants of the FP64 step in fixed point (exact64.cuh)
+  FxAdj fx = {};            // constants of the FP64 step in fixed point (exact64.cuh)
 };
 
 // Storage of the adjoint arrays: IEEE double for both FP64 paths (the
@@ -90,7 +90,7 @@ template <class R> AdjConst<R> make_adj(const KParams& kp) {
   c.k3am = R(3.0 * am);
   c.nk3am = R(-3.0 * am);
   c.gx = kp.g[1] == 0.0 && kp.g[2] == 0.0;
-  c.fx = make_fx_adj(kp.lp, kp.lm, kp.g);
+  if (std::is_same<R, double>::value) c.fx = make_fx_adj(kp.lp, kp.lm, kp.g);
   return c;
 }
 
@@ -159,18 +159,22 @@ __device__ __forceinline__ void adj_moments(const R (&mu)[kQ], const AdjConst<R>
 // One adjoint step.  G: OS-NT grid at step n (its pull gather is F_n).
 // lam_next / lam: adjoint of the canonical states F_{n+1} / F_n, layout [19][Npad].
 // LP1: l+ = 1 (FP64-storage paths), where (1 - l+)/2 = 1 - l+ = 0.
-#ifndef LBM_MIN_CTAS_ADJ
-#define LBM_MIN_CTAS_ADJ 8
-#endif
-// Resident CTAs per SM.  FP64 at 3 / 4 / 5 / 6: 13.43 / 12.80 / 13.11 / 14.08 ms
-// for a checkpointed gradient of 60 steps on 0.77 M nodes (above 4 it spills).
-// FP32 and FP16 wait for the gathers: 6 / 7 / 8 / 9 gave 19.67 / 19.61 / 18.99 /
-// 18.98 ms for 100 steps on the 128^3 box.
-template <int PREC> struct MinCtasAdj { static constexpr int value = LBM_MIN_CTAS_ADJ; };
-template <> struct MinCtasAdj<LBM_F64> { static constexpr int value = 4; };
-template <> struct MinCtasAdj<LBM_F64_DF> { static constexpr int value = 3; };
+// Resident CTAs per SM, by table, from sweeps of checkpointed gradients (ms).
+// Run slots, FP64 at 3 / 4 / 5 / 6: 13.43 / 12.80 / 13.11 / 14.08 (60 steps on
+// 0.77 M nodes; above 4 it spills); FP32 at 6 / 7 / 8 / 9: 19.67 / 19.61 / 18.99
+// / 18.98 (100 steps on the 128^3 box).  Adjacency list (60 steps on the box):
+// FP32 at 6 / 7 / 8: 17.0 / 15.8 / 17.0, FP64 at 4 / 5 / 6: 37.5 / 36.1 / 40.5.
+// Run entries (60 steps on a 128^3 foam): FP32 at 5 / 6 / 7 / 8: 12.0 / 11.6 /
+// 13.4 / 13.6, FP64 at 4 / 5: 34.6 / 39.6.
+template <int PREC, int TAB> struct MinCtasAdj {
+  static constexpr int value = PREC == LBM_F64_DF ? 3
+                               : PREC == LBM_F64  ? (TAB == kAdjAny ? 5 : 4)
+                               : TAB == kSlot     ? 8
+                               : TAB == kAdjAny   ? 7
+                                                  : 6;
+};
 template <int PREC, bool DEP, int TAB, bool DRAG, bool LP1 = false>
-__global__ void __launch_bounds__(kBlock, MinCtasAdj<PREC>::value) k_adjoint(DevTables t, KParams kp, CollConst<typename St<PREC>::R> cc,
+__global__ void __launch_bounds__(kBlock, MinCtasAdj<PREC, TAB>::value) k_adjoint(DevTables t, KParams kp, CollConst<typename St<PREC>::R> cc,
                                                     AdjConst<typename St<PREC>::R> c,
                                                     const typename St<PREC>::T* __restrict__ G,
                                                     const typename Lam<PREC>::T* __restrict__ lam_next,

