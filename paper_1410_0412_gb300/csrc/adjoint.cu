@@ -165,9 +165,10 @@ __device__ __forceinline__ void adj_moments(const R (&mu)[kQ], const AdjConst<R>
 // / 18.98 (100 steps on the 128^3 box).  Adjacency list (60 steps on the box):
 // FP32 at 6 / 7 / 8: 17.0 / 15.8 / 17.0, FP64 at 4 / 5 / 6: 37.5 / 36.1 / 40.5.
 // Run entries (60 steps on a 128^3 foam): FP32 at 5 / 6 / 7 / 8: 12.0 / 11.6 /
-// 13.4 / 13.6, FP64 at 4 / 5: 34.6 / 39.6.
+// 13.4 / 13.6, FP64 at 4 / 5: 34.6 / 39.6.  Double-float at 4 / 5 / 6: 1713 / 1589
+// / 1527 (2000 steps on the box, adjacency list).
 template <int PREC, int TAB> struct MinCtasAdj {
-  static constexpr int value = PREC == LBM_F64_DF ? 3
+  static constexpr int value = PREC == LBM_F64_DF ? 6
                                : PREC == LBM_F64  ? (TAB == kAdjAny ? 5 : 4)
                                : TAB == kSlot     ? 8
                                : TAB == kAdjAny   ? 7
