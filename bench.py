@@ -36,17 +36,12 @@ import geometry  # noqa: E402
 
 MEASURED_PEAKS = os.path.join(ROOT, "MEASURED_PEAKS.json")
 FALLBACK_HBM_GBS = 6800.0
-# FP64-pipe instructions per node of the AA steps with a uniform body force
-# along x, counted by ncu over the nodes of one launch, the same for the even
-# and odd step: sm__inst_executed_pipe_fp64.sum = 31 per node with
-# omega_plus = 1, of which 27 are arithmetic (smsp__sass_thread_inst_executed
-# _op_{dadd,dfma,dmul}_pred_on.sum: 1 DADD, 13 DFMA, 13 DMUL) and 4 the int64 ->
-# double conversions of two pairs' outputs.  The moments and the pair update
-# run on the integer pipe in fixed point; what stays on the FP64 pipe is the
-# per-node terms (density, the reciprocal's Newton steps, velocity, K0, T, O)
-# and the rest PDF, which takes one FMA more when omega_plus != 1.
-COLL_DP_INSTR_GENERAL = 32
-COLL_DP_INSTR_UNIT_OMEGA = 31
+# FP64-pipe instructions per node of the AA steps with a uniform body force: the
+# int64 -> double conversions of the 19 outputs (ncu, sm__inst_executed_pipe
+# _fp64.sum over the nodes of one launch).  Moments, class terms and pair update
+# run in fixed point on the integer and FMA pipes, for every omega_plus.
+COLL_DP_INSTR_GENERAL = 19
+COLL_DP_INSTR_UNIT_OMEGA = 19
 # DRAM bytes (dram__bytes_read.sum + dram__bytes_write.sum) of one launch of a
 # kernel on the 10,896,954-node bed, from an ncu capture of the current kernel
 # version, with the profile that holds it; kernels not listed print null.
