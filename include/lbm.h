@@ -372,6 +372,14 @@ LBM_API int lbm_fx_pairs_host(const double* d, const double* terms, int64_t n, d
 LBM_API int lbm_fx_collide_host(const double* d, const float* s, int64_t n, const lbm_params* params, double* out,
                                 int* ok);
 
+/* Host image of the read-back's density and velocity quotients of LBM_F64 grids
+ * (exact integer sums, integer quotients), run on the host.  d: host double
+ * [n][19], PDFs in params' storage; out: host double [n][4]: rho and j / rho (x,
+ * y, z), without the force and drag terms; ok: host int [n], 0 where the node is
+ * outside the integer range (out is then 0; the kernels divide in FP64 there).
+ * LBM_ERR_ARG for bad params, NULL pointers or n < 0. */
+LBM_API int lbm_fx_velocity_host(const double* d, int64_t n, const lbm_params* params, double* out, int* ok);
+
 /* Host image of the LBM_F64 adjoint step's arithmetic in fixed point.  d: host
  * double [n][19], forward PDFs F_n in params' storage; mu: host double [n][19],
  * the gathered adjoint vector; s: host float [n] or NULL.  lam: host double

@@ -629,6 +629,23 @@ def lbm_fx_collide_host(d, params, s=None):
     return out, ok.astype(bool)
 
 
+def lbm_fx_velocity_host(d, params):
+    """Host image of the read-back's FP64 density and velocity quotients (``lbm_fx_velocity_host``).
+
+    d: [n, 19] PDFs in the storage of ``params``.  Returns (out [n, 4], ok [n]):
+    rho and j / rho per node, without the force and drag terms.
+    """
+    import numpy as np
+    a = np.ascontiguousarray(np.asarray(d, dtype=np.float64))
+    if a.ndim != 2 or a.shape[1] != 19:
+        raise ValueError("d must have shape [n, 19]")
+    out = np.empty((a.shape[0], 4), dtype=np.float64)
+    ok = np.empty(a.shape[0], dtype=np.int32)
+    check(_lib.load().lbm_fx_velocity_host(a.ctypes.data, a.shape[0], ctypes.byref(params.c()), out.ctypes.data,
+                                           ok.ctypes.data), "lbm_fx_velocity_host")
+    return out, ok.astype(bool)
+
+
 def lbm_fx_adjoint_host(d, mu, params, s=None):
     """Host image of the FP64 adjoint step's arithmetic in fixed point (``lbm_fx_adjoint_host``).
 
@@ -933,7 +950,8 @@ __all__ = [
     "PartitionedSolver", "lbm_halo_exchange", "lbm_partition_run_aa", "lbm_partition_run_osnt",
     "lbm_objective_flux", "lbm_adjoint_step", "lbm_ckpt_workspace_bytes", "lbm_flux_forward", "lbm_flux_backward",
     "flux_objective", "new_adjoint", "lbm_macroscopic_noalloc", "lbm_check_finite", "lbm_bandwidth_kernel", "lbm_fp64_peak_kernel",
-    "lbm_exact_moments_host", "lbm_fx_pairs_host", "lbm_fx_collide_host", "lbm_fx_adjoint_host",
+    "lbm_exact_moments_host", "lbm_fx_pairs_host", "lbm_fx_collide_host", "lbm_fx_velocity_host",
+    "lbm_fx_adjoint_host",
     "State", "FluxObjective",
 ]
 

@@ -93,6 +93,7 @@ SIGNATURES = {
     "lbm_exact_moments_host": [_P, _I64, _P],
     "lbm_fx_pairs_host": [_P, _P, _I64, ctypes.c_double, ctypes.c_double, _I, _P, _P],
     "lbm_fx_collide_host": [_P, _P, _I64, ctypes.POINTER(lbm_params), _P, _P],
+    "lbm_fx_velocity_host": [_P, _I64, ctypes.POINTER(lbm_params), _P, _P],
     "lbm_fx_adjoint_host": [_P, _P, _P, _I64, ctypes.POINTER(lbm_params), _P, _P, _P],
     "lbm_device_table_bytes": [_P, _I, _PSZ],
     "lbm_lattice_upload": [_P, _I, _P, _SZ, _P],

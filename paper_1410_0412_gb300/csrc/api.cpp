@@ -440,6 +440,22 @@ int lbm_fx_collide_host(const double* d, const float* s, int64_t n, const lbm_pa
   return LBM_OK;
 }
 
+int lbm_fx_velocity_host(const double* d, int64_t n, const lbm_params* params, double* out, int* ok) {
+  KParams kp;
+  if (int rc = make_kparams(params, LBM_F64, &kp)) return rc;
+  if (n < 0 || (n > 0 && (!d || !out || !ok))) return set_error(LBM_ERR_ARG, "d, out or ok is NULL, or n < 0");
+  for (int64_t k = 0; k < n; ++k) {
+    double f[19], o[4] = {0.0};
+    std::memcpy(f, d + 19 * k, sizeof f);
+    int64_t S, Jx, Jy, Jz;
+    const int emax = dev::fx_moments(f, S, Jx, Jy, Jz);
+    ok[k] = dev::fx_velocity(kp.rho_s, emax, S, Jx, Jy, Jz, o[0], o[1], o[2], o[3]);
+    if (!ok[k]) std::memset(o, 0, sizeof o);
+    std::memcpy(out + 4 * k, o, sizeof o);
+  }
+  return LBM_OK;
+}
+
 int lbm_fx_adjoint_host(const double* d, const double* mu, const float* s, int64_t n, const lbm_params* params,
                         double* lam, double* grad, int* ok) {
   KParams kp;

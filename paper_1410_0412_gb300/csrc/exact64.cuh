@@ -708,14 +708,32 @@ __host__ __device__ __forceinline__ void fx_update(const FxColl& c, const FxClas
   d[0] = fx_to_double_cvt(v0, emax - kx);
 }
 
-// J 2^(emax - 1080) / rho as a double within (1/2 + 2^-4) ulp, for rho = D
-// 2^(er - 63), 2^63 <= D < 2^64, r = fx_recip(D) and 64 <= emax - er < 1900: J is
-// shifted to 63 bits, so that the product keeps 59 or more.
+// J 2^(emax - 1080) / rho as a double within (1/2 + 2^-4) ulp, for |J| < 2^62
+// (ten PDFs below 2^58), rho = D 2^(er - 63), 2^63 <= D < 2^64, r = fx_recip(D)
+// and 64 <= emax - er < 1900.  J is shifted to 62 bits, so that the product keeps
+// 58 or more.  Not to 63: mulhi_q64 takes factors below 2^63 - 2^31, and a J
+// just below a power of two (a velocity of 1/16) came out with the wrong sign.
 __host__ __device__ __forceinline__ double fx_quotient(int64_t J, int emax, Bal r, int er) {
   const uint64_t a = static_cast<uint64_t>(J ^ (J >> 63)) | 1u;
-  const int lz = clz64(a);
-  const int64_t m = mulhi_q64(bal(static_cast<int64_t>(static_cast<uint64_t>(J) << (lz - 1))), r);
-  return fx_to_double_cvt(m, emax - er - lz + 3);  // m 2^(emax - er - lz - 1077)
+  const int lz = clz64(a);  // 2..63
+  const int64_t m = mulhi_q64(bal(static_cast<int64_t>(static_cast<uint64_t>(J) << (lz - 2))), r);
+  return fx_to_double_cvt(m, emax - er - lz + 4);  // m 2^(emax - er - lz - 1076)
+}
+
+// Density rho = rho_s + S and j / rho of one node from its moments (scale emax) by
+// integer quotients; false for nodes outside their range (no positive normal
+// density, Inf or NaN PDFs), whose quotients the caller forms in FP64.
+__host__ __device__ __forceinline__ bool fx_velocity(double rho_s, int emax, int64_t S, int64_t Jx, int64_t Jy,
+                                                     int64_t Jz, double& r, double& ux, double& uy, double& uz) {
+  r = rho_s + fx_to_double_cvt(S, emax);
+  const uint64_t b = dbits(r);
+  const int er = static_cast<int>(b >> 52) - 1023;
+  if (!(emax < kFxMaxExp && er > -1000 && er < 1000 && emax - er >= 64 && emax - er < 1900)) return false;
+  const Bal q = bal(fx_recip((b << 11) | kSignBit));
+  ux = fx_quotient(Jx, emax, q, er);
+  uy = fx_quotient(Jy, emax, q, er);
+  uz = fx_quotient(Jz, emax, q, er);
+  return true;
 }
 
 // Binades of the pair scale below the moments' (see above).

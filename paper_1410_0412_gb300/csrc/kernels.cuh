@@ -1420,15 +1420,7 @@ __device__ __forceinline__ void node_rho_u(const KParams& kp, const R (&d)[kQ], 
                                            double& r, double& ux, double& uy, double& uz) {
   int64_t S, Jx, Jy, Jz;
   const int emax = fx_moments(d, S, Jx, Jy, Jz);
-  r = kp.rho_s + fx_to_double_cvt(S, emax);
-  const uint64_t b = dbits(r);
-  const int er = static_cast<int>(b >> 52) - 1023;
-  if (emax < kFxMaxExp && er > -1000 && er < 1000 && emax - er >= 64 && emax - er < 1900) {
-    const Bal q = bal(fx_recip((b << 11) | kSignBit));
-    ux = fx_quotient(Jx, emax, q, er);
-    uy = fx_quotient(Jy, emax, q, er);
-    uz = fx_quotient(Jz, emax, q, er);
-  } else {
+  if (!fx_velocity(kp.rho_s, emax, S, Jx, Jy, Jz, r, ux, uy, uz)) {
     double f[kQ], jx = 0.0, jy = 0.0, jz = 0.0;
     r = 0.0;
 #pragma unroll
