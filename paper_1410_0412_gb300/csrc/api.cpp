@@ -377,7 +377,10 @@ int lbm_fx_pairs_host(const double* d, const double* terms, int64_t n, double qm
     const int emax = !general && near ? dev::fx_moments<true, true>(f, Sk, D, S, Jx, Jy, Jz, emax_fast)
                                       : dev::fx_moments<true>(f, Sk, D, S, Jx, Jy, Jz);
     double* o = out + 19 * k;
-    ok[k] = dev::fx_class_ok(emax, t[0], t[1], t[2], t[3], t[4], t[5], t[6], t[7], t[8], t[9]) ? 1 : 0;
+    ok[k] = dev::q64_fits(qm) && dev::q64_fits(qp) &&
+                    dev::fx_class_ok(emax, t[0], t[1], t[2], t[3], t[4], t[5], t[6], t[7], t[8], t[9])
+                ? 1
+                : 0;
     if (!ok[k]) {
       for (int i = 0; i < 19; ++i) o[i] = 0.0;
       continue;

@@ -473,15 +473,11 @@ __host__ __device__ __forceinline__ void fx_pairs(const FxClass& q, const int64_
   fx_pair<LP1, GENERAL>(Eyz - q.Cyz, q.Oy - q.Oz, D[9], Sk[9], qm, qp, px, es, p[17], p[18]);
 }
 
-// Q64 image of a rate constant |x| <= 1/2: round(x * 2^64), kept below 2^63 -
-// 2^31 in magnitude for mulhi_q64 (rates within 2^-33 of 0 or 2 alone).
-inline int64_t q64_of(double x) {
-  constexpr int64_t most = INT64_MAX - INT32_MAX - int64_t(1);
-  const double v = std::ldexp(x, 64);
-  if (v >= 9.2233720368e18) return most;
-  if (v <= -9.2233720368e18) return -most;
-  return static_cast<int64_t>(std::llround(v));
-}
+// Q64 image of a rate constant |x| <= 1/2: round(x * 2^64), and whether mulhi_q64
+// may take it: |x| 2^64 < 2^63 - 2^31.  A rate beyond that (1 - l+- within 2^-32 of
+// +-1) has no image of its precision, and the caller takes the FP64 update.
+inline bool q64_fits(double x) { return std::fabs(x) < 0.5 - 0x1p-33; }
+inline int64_t q64_of(double x) { return q64_fits(x) ? static_cast<int64_t>(std::llround(std::ldexp(x, 64))) : 0; }
 
 // ---- the class values in fixed point ---------------------------------------------------
 //
@@ -516,6 +512,7 @@ struct FxColl {
   double rho_s;              // density of the storage shift, 0 for full storage
   bool shift;                // rho_s != 0 (a flag: the comparison is an FP64-pipe instruction)
   int emin;                  // least moment scale (deviation storage: that of the force)
+  int emax;                  // moment scales from here on are out of range: kFxMaxExp, or 0 when a rate is (q64_fits)
   bool gx;                   // the force points along x
 };
 
@@ -531,6 +528,7 @@ inline FxColl make_fx_coll(double lp, double lm, const double (&g)[3], double rh
   c.foh = q64_of(am / 6.0 / 2.0);
   c.qm = q64_of((1.0 - lm) / 2);
   c.qp = q64_of((1.0 - lp) / 2);
+  c.emax = q64_fits((1.0 - lm) / 2) && q64_fits((1.0 - lp) / 2) ? kFxMaxExp : 0;
   for (int a = 0; a < 3; ++a) {
     int e = 0;
     const double m = std::frexp(g[a], &e);  // g = m 2^e, 1/2 <= |m| < 1
@@ -612,7 +610,7 @@ __host__ __device__ __forceinline__ bool fx_class_int(const FxColl& c, int emax,
   const int pre = sh > 1 ? sh - 1 : 0, down = 1 - sh + pre;  // >= 0
   const int post = down > 63 ? 63 : down;
   const int nj = (pre > 1 ? 30 - pre : 29) - kx;
-  ok = ok && emax < kFxMaxExp && nj >= 0 && (mag(Jx) | mag(Jy) | mag(Jz)) >> (nj & 31) == 0;
+  ok = ok && emax < c.emax && nj >= 0 && (mag(Jx) | mag(Jy) | mag(Jz)) >> (nj & 31) == 0;
   const Bal r = bal(fx_recip(D));
   const uint32_t px = 1u << kx;
   int64_t qx = static_cast<int64_t>(static_cast<uint64_t>(Jx) * px);
@@ -766,7 +764,7 @@ struct FxAdj {
   int64_t c3, c3s;       // l-/12, a-/12 (c3 - c3s s)
   int64_t ap4;           // a+/4
   int64_t g[3];
-  bool ok;               // the force is in range
+  bool ok;               // the force and the rates are in range
 };
 
 inline FxAdj make_fx_adj(double lp, double lm, const double (&g)[3]) {
@@ -778,7 +776,7 @@ inline FxAdj make_fx_adj(double lp, double lm, const double (&g)[3]) {
   c.c3 = q64_of(lm / 12.0);
   c.c3s = q64_of(am / 12.0);
   c.ap4 = q64_of(ap / 4.0);
-  c.ok = true;
+  c.ok = q64_fits(lp / 4.0) && q64_fits(ap / 2.0);
   for (int a = 0; a < 3; ++a) {
     c.ok = c.ok && std::fabs(g[a]) < 0.015625;
     c.g[a] = c.ok ? q64_of(g[a]) : 0;
@@ -806,7 +804,7 @@ __host__ __device__ __forceinline__ bool fx_adjoint(const FxColl& c, const FxAdj
   // rho = D 2^(er - 63)
   uint64_t D;
   int er;
-  bool ok = a.ok && ef < kFxMaxExp && em < kFxMaxExp;
+  bool ok = a.ok && ef < c.emax && em < c.emax;
   if (c.shift) {  // uniform
     const uint64_t b = dbits(c.rho_s + fx_to_double_cvt(S, ef));
     D = (b << 11) | kSignBit;
