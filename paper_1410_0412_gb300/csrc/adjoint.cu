@@ -465,7 +465,7 @@ int launch_adjoint_t(const lbm_lattice* L, const KParams& kp, const void* G, con
   const int N = int(L->N);
   // dependent launches as the OS-NT steps around it; without a run slot table,
   // and with pressure faces, it reads the adjacency entries
-  by_dep<PREC, kFormOsnt>(L, [&](auto dep) {
+  by_dep<PREC, kFormOsnt>(L, ria, [&](auto dep) {
     auto go = [&](auto tab) {
       by_bool(s != nullptr, [&](auto drag) {
         by_lp1<PREC>(use_lp1<PREC>(kp), [&](auto lp1) {
@@ -477,7 +477,7 @@ int launch_adjoint_t(const lbm_lattice* L, const KParams& kp, const void* G, con
     };
     if (!ria)
       go(TableC<dev::kAdjAny>{});
-    else if (table_kind(L, ria) == dev::kSlot)
+    else if (table_kind<PREC, kFormOsnt>(L, ria) == dev::kSlot)
       go(TableC<dev::kSlot>{});
     else
       go(TableC<dev::kRunAny>{});

@@ -1521,14 +1521,6 @@ inline unsigned grid_of(int64_t N) { return unsigned((N + dev::kBlock - 1) / dev
 // read-back).  Never more than the workspace holds (reduce_parts).
 inline unsigned reduce_grid(int64_t nparts) { return unsigned(std::min<int64_t>(std::max<int64_t>(nparts, 1), 16 * 152)); }
 
-// The table a step of this lattice reads (dev::Table).  Grids of 2^32 slots or
-// more (above 226 M nodes) have no 32-bit slot index.
-inline int table_kind(const lbm_lattice* L, int ria) {
-  if (ria) return !L->dev.run_slot ? dev::kRunAny : L->dev.pressure ? dev::kSlotFace : dev::kSlot;
-  const bool wide = int64_t(kQ) * L->Npad >= (int64_t(1) << 32);
-  return wide || L->dev.pressure ? dev::kAdjAny : dev::kAdj;
-}
-
 inline bool has_force(const KParams& kp) { return kp.g[0] != 0.0 || kp.g[1] != 0.0 || kp.g[2] != 0.0; }
 
 // The l+ = 1 collision (see collide) is instantiated for the FP64-storage
@@ -1537,28 +1529,78 @@ inline bool has_force(const KParams& kp) { return kp.g[0] != 0.0 || kp.g[1] != 0
 template <int PREC> constexpr bool kLp1Path = PREC == LBM_F64 || PREC == LBM_F64_DF;
 template <int PREC> inline bool use_lp1(const KParams& kp) { return kLp1Path<PREC> && kp.lp == 1.0; }
 
+// The step forms, and what the choices below go by: the bytes of PDFs that a step
+// moves, and how far its nodes' neighbours are apart (runs per node: 0.02 to 0.15
+// in rows, 0.3 in blocked rows, 0.4 among small spheres, 1 on a Hilbert curve).
+enum Form { kFormOsnt, kFormAa, kFormEt };
+template <int PREC> inline int64_t step_bytes(const lbm_lattice* L) {
+  return 2 * kQ * int64_t(sizeof(typename dev::St<PREC>::T)) * L->N;
+}
+constexpr int64_t kSmallStep = int64_t(256) << 20;
+inline bool scattered(const lbm_lattice* L) { return 2 * L->R > L->N && L->N > (1 << 18); }
+
+// The table a step of this lattice reads (dev::Table).  Grids of 2^32 slots or
+// more (above 226 M nodes) have no 32-bit slot index.  Beyond that, slots resolved
+// before the loads (kSlot, kAdj) are the faster form wherever neighbours are near;
+// with one run per node the single-precision AA odd steps are faster on the
+// adjacency entries, which they decode at each access (us a step, slots ->
+// entries; Hilbert bed of 112^3 / 160^3 / 224^3: FP16S RIA 32.2 -> 27.0 / 95.2 ->
+// 76.8 / 243 -> 200; FP32 RIA 41.9 -> 39.2 at 112^3, equal above kSmallStep, where
+// it is not a dependent launch; FP16S list 31.6 -> 28.5 / 91.9 -> 81.2 / 223 -> 208;
+// FP32 list 39.8 -> 38.2 / 116 -> 109 / 309 -> 286), below 2^18 nodes slots again
+// (48^3: FP16S RIA 4.0 against 4.3).  Large FP32 AA and FP16S OS-NT steps with the
+// list take the entries in every order (FP32 144^3 blocked rows 72.9 -> 71.3, 256^3
+// rows 365 -> 367; FP16S OS-NT 256^3 rows 354 -> 342).
+template <int PREC, int FORM> inline int table_kind(const lbm_lattice* L, int ria) {
+  const bool small = step_bytes<PREC>(L) <= kSmallStep, f32 = PREC == LBM_F32, f16 = PREC == LBM_F16S;
+  const bool aa = FORM == kFormAa;
+  if (ria) {
+    if (!L->dev.run_slot) return dev::kRunAny;
+    if (L->dev.pressure) return dev::kSlotFace;
+    return aa && scattered(L) && (f16 || (f32 && small)) ? dev::kRunAny : dev::kSlot;
+  }
+  const bool wide = int64_t(kQ) * L->Npad >= (int64_t(1) << 32);
+  if (wide || L->dev.pressure) return dev::kAdjAny;
+  const bool entries = aa ? (f16 && scattered(L)) || (f32 && (scattered(L) || !small))
+                          : FORM == kFormOsnt && f16 && !small;
+  return entries ? dev::kAdjAny : dev::kAdj;
+}
+
 // Which steps are launched as dependent kernels.  FP64 and the two-grid and
 // Esoteric Twist steps of FP32, and OS-NT of FP16S: always, faster at every size
 // measured (10 steps, plain -> dependent, us, on beds of 96^3 / 200^3: FP64 AA-R
 // 383 -> 359 / 3040 -> 3025, OS-NT-R 412 -> 371 / 3207 -> 3106; FP32 OS-NT-R
 // 188 -> 157 / 1638 -> 1569, ET-R 204 -> 178 / 2146 -> 2104; FP16S OS-NT-R 127 ->
-// 118 / 1089 -> 1064).  The others lose the non-coherent loads, 1-3 % of a large
-// step, and are dependent when a step moves at most 256 MB of PDFs: FP32 AA-R
+// 118 / 1089 -> 1064), but for FP32 ET-R with pressure faces in rows (foam of 192^3
+// 199.0 -> 200.8 a step; on a Hilbert curve 238.8 -> 236.9).  The others lose the
+// non-coherent loads, 1-3 % of a large step, and are dependent when a step moves at
+// most 256 MB of PDFs: FP32 AA-R
 // 151 -> 132 at 83 MB, 424 -> 412 at 198, 805 -> 804 at 386, 1570 -> 1591 at 754;
 // FP16S AA-R 123 -> 98 at 42, 507 -> 498 at 193, 960 -> 969 at 377; FP16S ET-R
-// 398 -> 371 at 99, 1657 -> 1685 at 377.  The double-float steps are plain.
-enum Form { kFormOsnt, kFormAa, kFormEt };
+// 398 -> 371 at 99, 1657 -> 1685 at 377.  Where the order has a run per four nodes
+// or more, FP16S AA-R by slots turns at about 96 MB (blocked rows, a step: 19.9 ->
+// 18.4 at 74, 27.3 -> 27.6 at 112, 43.6 -> 44.5 at 161), and so does the AA step by
+// the list's entries (Hilbert beds and foams: 29.5 -> 28.5 at 74, 35.7 -> 36.4 at 99,
+// 58.8 -> 59.2 at 161).  The double-float steps are plain.
 template <int PREC, int FORM>
 constexpr int kDependent = PREC == LBM_F64_DF                                                                  ? 0
                            : PREC == LBM_F64 || (PREC == LBM_F32 && FORM != kFormAa) || FORM == kFormOsnt ? 2
                                                                                                             : 1;
+template <int PREC, int FORM> inline bool dependent(const lbm_lattice* L, int ria) {
+  const bool faces = PREC == LBM_F32 && FORM == kFormEt && ria && L->dev.pressure && !scattered(L);
+  if (kDependent<PREC, FORM> != 1 && !faces) return kDependent<PREC, FORM> == 2;
+  const bool apart = PREC == LBM_F16S && FORM == kFormAa && 4 * L->R > L->N && scattered(L) == !ria;
+  return step_bytes<PREC>(L) <= (apart ? int64_t(96) << 20 : kSmallStep);
+}
 // f gets DEP as the rule says.
-template <int PREC, int FORM, class F> inline void by_dep(const lbm_lattice* L, F f) {
-  if constexpr (kDependent<PREC, FORM> == 0)
+template <int PREC, int FORM, class F> inline void by_dep(const lbm_lattice* L, int ria, F f) {
+  constexpr bool kNever = kDependent<PREC, FORM> == 0;
+  constexpr bool kAlways = kDependent<PREC, FORM> == 2 && !(PREC == LBM_F32 && FORM == kFormEt);
+  if constexpr (kNever)
     f(std::false_type{});
-  else if constexpr (kDependent<PREC, FORM> == 2)
+  else if constexpr (kAlways)
     f(std::true_type{});
-  else if (2 * kQ * int64_t(sizeof(typename dev::St<PREC>::T)) * L->N <= (int64_t(256) << 20))
+  else if (dependent<PREC, FORM>(L, ria))
     f(std::true_type{});
   else
     f(std::false_type{});
@@ -1629,8 +1671,8 @@ int launch_osnt_t(const lbm_lattice* L, const KParams& kp, const void* src, void
   T* b = static_cast<T*>(dst);
   const int N = int(L->N);
   const auto c = dev::make_coll_step<PREC>(kp);
-  by_dep<PREC, kFormOsnt>(L, [&](auto dep) {
-    by_table(table_kind(L, ria), [&](auto tab) {
+  by_dep<PREC, kFormOsnt>(L, ria, [&](auto dep) {
+    by_table(table_kind<PREC, kFormOsnt>(L, ria), [&](auto tab) {
       by_terms(s != nullptr, has_force(kp), [&](auto force, auto drag) {
         by_lp1<PREC>(use_lp1<PREC>(kp), [&](auto lp1) {
           constexpr bool kDep = decltype(dep)::value, kF = decltype(force)::value, kD = decltype(drag)::value;
@@ -1653,7 +1695,7 @@ int launch_aa_t(const lbm_lattice* L, const KParams& kp, void* pdf, int parity, 
   const unsigned blk = dev::kBlock, g = grid_of(L->N), g2 = unsigned((L->N + 2 * blk - 1) / (2 * blk));
   const auto c = dev::make_coll_step<PREC>(kp);
   if (parity == 0) {
-    by_dep<PREC, kFormAa>(L, [&](auto dep) {
+    by_dep<PREC, kFormAa>(L, ria, [&](auto dep) {
       by_terms(s != nullptr, has_force(kp), [&](auto force, auto drag) {
         constexpr bool kDep = decltype(dep)::value, kF = decltype(force)::value, kD = decltype(drag)::value;
         if constexpr (PREC == LBM_F16S)
@@ -1667,8 +1709,8 @@ int launch_aa_t(const lbm_lattice* L, const KParams& kp, void* pdf, int parity, 
     });
     return cuda_check("AA even step launch");
   }
-  by_dep<PREC, kFormAa>(L, [&](auto dep) {
-    by_table(table_kind(L, ria), [&](auto tab) {
+  by_dep<PREC, kFormAa>(L, ria, [&](auto dep) {
+    by_table(table_kind<PREC, kFormAa>(L, ria), [&](auto tab) {
       by_terms(s != nullptr, has_force(kp), [&](auto force, auto drag) {
         constexpr bool kDep = decltype(dep)::value, kF = decltype(force)::value, kD = decltype(drag)::value;
         constexpr int kTab = decltype(tab)::value;
@@ -1694,7 +1736,7 @@ int launch_et_t(const lbm_lattice* L, const KParams& kp, void* pdf, int parity, 
   T* A = static_cast<T*>(pdf);
   const int N = int(L->N);
   const auto c = dev::make_coll_step<PREC>(kp);
-  by_dep<PREC, kFormEt>(L, [&](auto dep) {
+  by_dep<PREC, kFormEt>(L, ria, [&](auto dep) {
     by_bool(ria != 0, [&](auto run) {
       by_bool(parity != 0, [&](auto odd) {
         by_terms(s != nullptr, has_force(kp), [&](auto force, auto drag) {
