@@ -407,12 +407,13 @@ template <bool FORCE, bool DRAG, bool LP1>
 int fx_collide_node(const dev::FxColl& c, double (&f)[19], double s) {
   int64_t Sk[10], D[10], S, Jx, Jy, Jz, f0;
   int emax_fast;
-  const bool near = dev::fx_pos_near(f, emax_fast);
+  const bool near = dev::fx_pos_near(f, emax_fast) && emax_fast >= c.emin;
   const int emax = near ? dev::fx_moments<true, true>(f, Sk, D, S, Jx, Jy, Jz, emax_fast, &f0)
                         : dev::fx_moments<true>(f, Sk, D, S, Jx, Jy, Jz, 0, &f0, c.emin);
-  const int kx = dev::fx_kx<LP1>(c, near);
+  const int kx = dev::fx_kx<LP1>(c);
   dev::FxClass q;
   if (!dev::fx_class_int<FORCE, DRAG, LP1>(c, emax, kx, S, Jx, Jy, Jz, s, q)) return 0;
+  if (LP1 && !c.shift && !dev::fx_room4(D)) return 0;
   dev::fx_update<LP1>(c, q, emax, kx, D, Sk, f0, f);
   return 1;
 }

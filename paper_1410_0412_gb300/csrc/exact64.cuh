@@ -353,8 +353,8 @@ __host__ __device__ __forceinline__ void exact_moments(const double (&d)[19], do
 // the low words, at most a quarter of a unit, is left out: three multiply-adds
 // and about four ALU instructions, where the exact high word of a signed
 // 64 x 64 product takes about 14.  Both factors must stay below 2^63 - 2^31
-// in magnitude (the high halves round up) and one of them below 2^62 (the
-// middle sum).
+// in magnitude: the high halves, which round up, are then below 2^31 and the
+// middle sum below 2^63.
 struct Bal {
   int32_t h, l;
 };
@@ -391,8 +391,8 @@ __host__ __device__ __forceinline__ int dexp(double x) { return static_cast<int>
 // (for PDFs near w_i rho, below a quarter of an ulp of the smallest, the
 // diagonal ones, when kx = 4).
 //
-// For class values given as doubles the host image takes kx = 4 when l+ = 1,
-// else 2; valid when |u_a| < 1/4 (biased exponent <= 1020), |K0| < B/2
+// For class values given as doubles the host image takes kx = 4 when l+ = 1 and
+// fx_room4, else 2; valid when |u_a| < 1/4 (biased exponent <= 1020), |K0| < B/2
 // (exponent <= emax - 2) and |T_a|, |O_a| < B/4 (exponent <= emax - 3), which
 // with every |d_i| < 2B keeps every intermediate below 2^63.  fx_class_ok
 // checks it.
@@ -425,6 +425,23 @@ __host__ __device__ __forceinline__ bool fx_class_ok(int emax, double ux, double
 #pragma unroll
   for (int i = 0; i < 5; ++i) eto = dexp(v[i]) > eto ? dexp(v[i]) : eto;
   return emax < kFxMaxExp && eu <= 1020 && dexp(K0) <= emax - 2 && eto <= emax - 3;
+}
+
+// The bits of a value's high word that differ from its sign: fx_mag(v) < 2^k
+// exactly when -2^(32 + k) <= v < 2^(32 + k).
+__host__ __device__ __forceinline__ uint32_t fx_mag(int64_t v) {
+  const int32_t h = static_cast<int32_t>(v >> 32);
+  return static_cast<uint32_t>(h ^ (h >> 31));
+}
+
+// Whether the pair differences leave room for kx = 4: |D_k| 2^4 < 2^63 - 2^36 for
+// mulhi_q64.  Only two PDFs of opposite signs, both within 2^-27 of 2^(emax - 1022),
+// do not.
+__host__ __device__ __forceinline__ bool fx_room4(const int64_t (&D)[10]) {
+  uint32_t m = 0;
+#pragma unroll
+  for (int k = 1; k <= 9; ++k) m = fx_mag(D[k]) > m ? fx_mag(D[k]) : m;
+  return m < (1u << 27) - 1;
 }
 
 // The class values at the pair scale es from doubles (see above).
@@ -493,9 +510,9 @@ inline int64_t q64_of(double x) { return q64_fits(x) ? static_cast<int64_t>(std:
 // 50 instructions a node, 16 SM cycles a warp each) were what bound the FP64
 // steps.
 //
-// The pair scale is 2^(es - 1080) with es = emax - kx: kx = 4 for positive
-// PDFs near each other when l+ = 1 (full storage), 2 for other full-storage
-// nodes, and 0 for deviations, whose momentum reaches 12 times their largest
+// The pair scale is 2^(es - 1080) with es = emax - kx: kx = 4 for full storage
+// with l+ = 1, 2 for full storage otherwise, and 0 for deviations, whose momentum
+// reaches 12 times their largest
 // member.  Bounds (each checked, in units of the pair scale unless noted):
 // |J_a| < 2^61, |G_a| < 2^59, |u_a| < 1/4, 0 <= s <= 1, and at the moment
 // scale |S| < 2^60 (kx >= 2) or 2^62 (kx = 0).  With l+-, a+- in their ranges
@@ -577,6 +594,11 @@ __host__ __device__ __forceinline__ int64_t fx_recip(uint64_t D) {
   return static_cast<int64_t>((r1 + static_cast<uint64_t>((static_cast<int64_t>(r1 >> 33) * e2) >> 29)) >> 1);
 }
 
+// Binades of the pair scale below the moments' (see above).  Uniform: a node's bits
+// must not depend on the nodes that share its warp, and a scale chosen node by node
+// costs the steps 1-2 %.
+template <bool LP1> __host__ __device__ __forceinline__ int fx_kx(const FxColl& c) { return c.shift ? 0 : LP1 ? 4 : 2; }
+
 // Class values at the pair scale of one node, from its moments at scale emax;
 // false where a bound fails (the caller then takes the FP64 update).  s: the
 // node's Brinkman solid fraction (DRAG only).
@@ -584,11 +606,6 @@ template <bool FORCE, bool DRAG, bool LP1>
 __host__ __device__ __forceinline__ bool fx_class_int(const FxColl& c, int emax, int kx, int64_t S, int64_t Jx,
                                                       int64_t Jy, int64_t Jz, double s, FxClass& q) {
   const int es = emax - kx;
-  // the bits of a value's high word that differ from its sign
-  auto mag = [](int64_t v) {
-    const int32_t h = static_cast<int32_t>(v >> 32);
-    return static_cast<uint32_t>(h ^ (h >> 31));
-  };
   // rho = D 2^(er - 63), 2^63 <= D < 2^64
   uint64_t D;
   int er;
@@ -597,10 +614,10 @@ __host__ __device__ __forceinline__ bool fx_class_int(const FxColl& c, int emax,
     const uint64_t b = dbits(c.rho_s + fx_to_double_cvt(S, emax));
     D = (b << 11) | kSignBit;
     er = static_cast<int>(b >> 52) - 1023;  // a negative density, Inf or NaN: er >= 1024
-    ok = er > -1000 && er < 1000 && mag(S) < 1u << 30;
+    ok = er > -1000 && er < 1000 && fx_mag(S) < 1u << 30;
   } else {
     const int lz = clz64(static_cast<uint64_t>(S));
-    ok = S > 0 && mag(S) < 1u << 28;
+    ok = S > 0 && fx_mag(S) < 1u << 28;
     D = (static_cast<uint64_t>(S) << (lz & 63)) | kSignBit;
     er = emax - 1017 - lz;
   }
@@ -610,7 +627,7 @@ __host__ __device__ __forceinline__ bool fx_class_int(const FxColl& c, int emax,
   const int pre = sh > 1 ? sh - 1 : 0, down = 1 - sh + pre;  // >= 0
   const int post = down > 63 ? 63 : down;
   const int nj = (pre > 1 ? 30 - pre : 29) - kx;
-  ok = ok && emax < c.emax && nj >= 0 && (mag(Jx) | mag(Jy) | mag(Jz)) >> (nj & 31) == 0;
+  ok = ok && emax < c.emax && nj >= 0 && (fx_mag(Jx) | fx_mag(Jy) | fx_mag(Jz)) >> (nj & 31) == 0;
   const Bal r = bal(fx_recip(D));
   const uint32_t px = 1u << kx;
   int64_t qx = static_cast<int64_t>(static_cast<uint64_t>(Jx) * px);
@@ -655,7 +672,7 @@ __host__ __device__ __forceinline__ bool fx_class_int(const FxColl& c, int emax,
     return static_cast<int64_t>(static_cast<uint64_t>(m) << 3) >> post;
   };
   const int64_t ux = velocity(qx), uy = velocity(qy), uz = velocity(qz);
-  ok = ok && (mag(ux) | mag(uy) | mag(uz)) < 1u << 30;
+  ok = ok && (fx_mag(ux) | fx_mag(uy) | fx_mag(uz)) < 1u << 30;
   int64_t Tx, Ty, Tz;  // halved, as are Ox, Oy, Oz
   if (LP1) {  // l+/4 and a+/2 are both 1/4
     Tx = (qx + Fx) >> 3;
@@ -732,11 +749,6 @@ __host__ __device__ __forceinline__ bool fx_velocity(double rho_s, int emax, int
   uy = fx_quotient(Jy, emax, q, er);
   uz = fx_quotient(Jz, emax, q, er);
   return true;
-}
-
-// Binades of the pair scale below the moments' (see above).
-template <bool LP1> __host__ __device__ __forceinline__ int fx_kx(const FxColl& c, bool near) {
-  return c.shift ? 0 : (LP1 && near) ? 4 : 2;
 }
 
 // ---- the adjoint step in fixed point ----------------------------------------------------

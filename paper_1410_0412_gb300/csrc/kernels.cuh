@@ -671,21 +671,24 @@ __device__ __forceinline__ void collide_m(R (&d)[kQ], const CollConst<R>& c, con
 // update in fixed point on the integer and FMA pipes (exact64.cuh) when every
 // node of the warp is in its range (fx_class_int; a warp-uniform branch),
 // otherwise in FP64 from the moments rounded to double.  NaN or Inf PDFs take
-// the FP64 branch and come out NaN.
+// the FP64 branch and come out NaN.  Among nodes in range a node's bits follow from
+// its own PDFs (both conversions give the same integers), whatever its warp holds.
 template <bool FORCE, bool DRAG, bool LP1>
 __device__ __forceinline__ void collide_f64(double (&d)[kQ], const CollConst<double>& c, const double s) {
   int64_t Sk[10], D[10], S, Jx, Jy, Jz, f0;
   // the shorter conversions when every node of the warp has positive PDFs
   // within 5 binades of its largest (full-f storage near equilibrium)
   int emax_fast, emax;
-  const bool near = __all_sync(__activemask(), fx_pos_near(d, emax_fast));
-  if (near)
+  bool room = true;
+  if (__all_sync(__activemask(), fx_pos_near(d, emax_fast) && emax_fast >= c.fx.emin)) {
     emax = fx_moments<!LP1, true>(d, Sk, D, S, Jx, Jy, Jz, emax_fast, &f0);
-  else
+  } else {
     emax = fx_moments<!LP1>(d, Sk, D, S, Jx, Jy, Jz, 0, &f0, c.fx.emin);
-  const int kx = fx_kx<LP1>(c.fx, near);
+    if (LP1) room = c.fx.shift || fx_room4(D);
+  }
+  const int kx = fx_kx<LP1>(c.fx);
   FxClass q;
-  const bool ok = fx_class_int<FORCE, DRAG, LP1>(c.fx, emax, kx, S, Jx, Jy, Jz, s, q);
+  const bool ok = fx_class_int<FORCE, DRAG, LP1>(c.fx, emax, kx, S, Jx, Jy, Jz, s, q) && room;
   if (__all_sync(__activemask(), ok)) {
     fx_update<LP1>(c.fx, q, emax, kx, D, Sk, f0, d);
   } else {
