@@ -385,7 +385,7 @@ int lbm_fx_pairs_host(const double* d, const double* terms, int64_t n, double qm
       for (int i = 0; i < 19; ++i) o[i] = 0.0;
       continue;
     }
-    const int kx = lp1 ? 4 : 2;
+    const int kx = lp1 && dev::fx_room4(D) ? 4 : 2;
     const dev::FxClass q = dev::fx_class(emax - kx, t[0], t[1], t[2], t[3], t[4], t[5], t[6], t[7], t[8], t[9]);
     if (lp1)
       general ? dev::fx_pairs<true, true>(q, D, Sk, qm_fx, qp_fx, emax - kx, kx, p)
