@@ -515,8 +515,9 @@ inline int64_t q64_of(double x) { return q64_fits(x) ? static_cast<int64_t>(std:
 // reaches 12 times their largest
 // member.  Bounds (each checked, in units of the pair scale unless noted):
 // |J_a| < 2^61, |G_a| < 2^59, |u_a| < 1/4, 0 <= s <= 1, and at the moment
-// scale |S| < 2^60 (kx >= 2) or 2^62 (kx = 0).  With l+-, a+- in their ranges
-// (k1 = l+/4 and a+/2 < 1/2, l-/6 < 1/3, a-/6 < 1/6) this gives |q| < 1.13
+// scale |S| < 2^60 (kx >= 2) or 2^62 (kx = 0, where also |S| >= 2^56 or some
+// |J_a| >= 2^57).  With l+-, a+- in their ranges (k1 = l+/4 and a+/2 < 1/2,
+// l-/6 < 1/3, a-/6 < 1/6) this gives |q| < 1.13
 // 2^61, |F| < 1.38 2^61, |T| < 1.26 2^61, |c.T| < 2.51 2^61, |O| < 0.61 2^61,
 // |K0| < 0.25 2^61 (0.45 2^61 at kx = 4) and every output below 2^63.
 struct FxColl {
@@ -614,7 +615,11 @@ __host__ __device__ __forceinline__ bool fx_class_int(const FxColl& c, int emax,
     const uint64_t b = dbits(c.rho_s + fx_to_double_cvt(S, emax));
     D = (b << 11) | kSignBit;
     er = static_cast<int>(b >> 52) - 1023;  // a negative density, Inf or NaN: er >= 1024
-    ok = er > -1000 && er < 1000 && fx_mag(S) < 1u << 30;
+    // |S| >= 2^56 or some |J_a| >= 2^57, unless the force sets the scale: where the
+    // large deviations cancel in both, so do the results, and a scale tied to the
+    // deviations would leave them few bits
+    const uint32_t top = (fx_mag(S) << 1) | fx_mag(Jx) | fx_mag(Jy) | fx_mag(Jz);
+    ok = er > -1000 && er < 1000 && fx_mag(S) < 1u << 30 && (top >= 1u << 25 || emax == c.emin);
   } else {
     const int lz = clz64(static_cast<uint64_t>(S));
     ok = S > 0 && fx_mag(S) < 1u << 28;
