@@ -246,7 +246,7 @@ __global__ void __launch_bounds__(kBlock, MinCtasAdj<PREC, TAB>::value) k_adjoin
     if (__all_sync(__activemask(), ok)) {
       if (grad_s) {
         const double rho = c.rho_s + fx_to_double_cvt(S, ef);
-        grad_s[n] = ::fma(rho, fx_to_double_cvt(o.gs, o.eg), grad_s[n]);
+        grad_s[n] = ::fma(rho, o.gs, grad_s[n]);
       }
       // lambda_a,b = e +- o, e = A + qp P_k, o = qm D_k + c_a.B; rest: A + (1 - l+) mu_0
       const Bal qm = bal(cc.fx.qm), qp = bal(cc.fx.qp);

@@ -487,7 +487,7 @@ int lbm_fx_adjoint_host(const double* d, const double* mu, const float* s, int64
               : dev::fx_adjoint<false>(c, a, ef, S, Jx, Jy, Jz, 0.0, em, m0, Pi, Di, o);
     grad[k] = 0.0;
     if (ok[k]) {
-      grad[k] = (kp.rho_s + dev::fx_to_double_cvt(S, ef)) * dev::fx_to_double_cvt(o.gs, o.eg);
+      grad[k] = (kp.rho_s + dev::fx_to_double_cvt(S, ef)) * o.gs;
       out[0] = dev::fx_to_double_cvt(o.A + dev::mulhi_q64(c.qp, 2 * m0), em);
       for (int q = 1; q <= 9; ++q) {
         const int64_t B[3] = {o.Bx, o.By, o.Bz};

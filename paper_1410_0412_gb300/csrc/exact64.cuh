@@ -764,23 +764,29 @@ __host__ __device__ __forceinline__ bool fx_velocity(double rho_s, int emax, int
 //   A = l+ M0 - (l+/2 - a+ s) u.X + 3 a- M1.g + kd P.g / 2,   B = kd P,
 //   dJ/ds / rho = -a+ u.X - 3 a- M1.u - kd P.u / 2,
 // all linear in mu: products of the integer moments (w = 1/36 and 1/18 make them
-// integers over 36) with u, g and per-launch constants as Q64 fractions.  u is
-// kept normalised, u = u' 2^-p with 1/32 < |u'| < 0.28 for its largest
-// component, and what enters dJ/ds only
-// through u (K u, M1.u, Y.u) is carried p bits finer than mu, so that the
-// gradient of a slow flow keeps its relative accuracy.
+// integers over 36) with u, g and per-launch constants as Q64 fractions.  lambda is
+// formed at mu's scale.  dJ/ds is a sum of products of M1, K, u and g, any of which
+// may be small beside max|mu| or 1 (a smooth adjoint field, a slow flow), so each
+// of the four is normalised first: K to K 2^zk and M1 to M1 2^zn (members below 2^62,
+// the largest at 2^61 or more; K exactly, with the remainder of M0's third), u to u'
+// 2^-p and g to g' 2^-zg with their largest components at 1/8 or more.  The three sums
+// M1.u, u.X and Y.u keep 56 bits or more of their terms and are added in FP64.  At
+// mu's scale throughout, dJ/ds lost 1e-12 of itself to rounding on a smooth field at
+// |u| = 1e-6, where the FP64 form kept 1e-16.
 //
 // Bounds: |mu_i| < 2^58 at mu's scale, so |36 M0| / 2 < 18, |36 M1| < 12,
-// |36 M2_aa| < 12, |36 M2_ab| < 4 and |4 K_aa| < 24 (times 2^58 each); |J 2^z| <
-// 2^62, |G| < 2^59 and p >= 0 give |u'| < 0.28 2^64 and |4 X| < 9 2^58; |g_a| < 2^-6
-// (checked on the host) makes Y small; then |P| < 7 2^58, |A| < 5 2^58 and every
-// output is below 2^62.  Each product is within 3/4 of a unit.
+// |36 M2_aa| < 12, |36 M2_ab| < 4 and |4 K_aa| < 24 (times 2^58 each; normalised
+// values below 16, or these at zk = zn = 0); |J 2^z| < 2^62, |G| < 2^59 and p >= 0
+// give |u'| < 0.28 2^64 and |4 X| < 13.5 2^58; |g_a| < 2^-6 (checked on the host)
+// makes Y small at mu's scale, and |g'| < 1/4 bounds it there; then |P| < 7 2^58,
+// |A| < 5 2^58 and every output is below 2^62.  Each product is within 3/4 of a unit.
 struct FxAdj {
   int64_t l18;           // l+/18 as a Q64 fraction, and so the next
   int64_t c1, c1s;       // l+/4, a+/2  (c1 - c1s s)
   int64_t c3, c3s;       // l-/12, a-/12 (c3 - c3s s)
   int64_t ap4;           // a+/4
-  int64_t g[3];
+  int64_t g[3], gn[3];   // g, and g 2^zg
+  int zg;
   bool ok;               // the force and the rates are in range
 };
 
@@ -794,12 +800,32 @@ inline FxAdj make_fx_adj(double lp, double lm, const double (&g)[3]) {
   c.c3s = q64_of(am / 12.0);
   c.ap4 = q64_of(ap / 4.0);
   c.ok = q64_fits(lp / 4.0) && q64_fits(ap / 2.0);
+  double top = 0.0;
   for (int a = 0; a < 3; ++a) {
     c.ok = c.ok && std::fabs(g[a]) < 0.015625;
+    top = std::fmax(top, std::fabs(g[a]));
+  }
+  int e = 0;
+  std::frexp(top, &e);  // top in [2^(e - 1), 2^e)
+  c.zg = c.ok && top > 0.0 ? -2 - e : 0;
+  for (int a = 0; a < 3; ++a) {
     c.g[a] = c.ok ? q64_of(g[a]) : 0;
+    c.gn[a] = c.ok ? q64_of(std::ldexp(g[a], c.zg)) : 0;
   }
   return c;
 }
+
+// Magnitude bits of a value, the shift that takes the largest of several (their bits
+// or-ed) to [2^61, 2^62), at most 59 and 0 for larger ones, and shifts by such counts.
+__host__ __device__ __forceinline__ uint64_t fx_bits(int64_t v) { return static_cast<uint64_t>(v ^ (v >> 63)); }
+__host__ __device__ __forceinline__ int fx_norm(uint64_t bits) {
+  const int n = clz64(bits) - 2;
+  return n < 0 ? 0 : n > 59 ? 59 : n;
+}
+__host__ __device__ __forceinline__ int64_t fx_shl(int64_t v, int n) {
+  return static_cast<int64_t>(static_cast<uint64_t>(v) << (n & 63));
+}
+__host__ __device__ __forceinline__ int64_t fx_shr(int64_t v, int n) { return v >> ((n > 63 ? 63 : n) & 63); }
 
 // Least moment scale of the adjoint vector: leaves room below it for the finer
 // scale of the gradient (adjoint values below 2^-880 flush to zero).
@@ -807,8 +833,7 @@ constexpr int kFxMinExpAdj = 200;
 
 struct FxAdjOut {
   int64_t A, Bx, By, Bz;  // at mu's scale
-  int64_t gs;             // dJ/ds / rho at the scale em - p
-  int eg;                 // em - p
+  double gs;              // dJ/ds / rho
 };
 
 // A, B and the gradient term of one node: from the forward moments (S, J at
@@ -870,49 +895,61 @@ __host__ __device__ __forceinline__ bool fx_adjoint(const FxColl& c, const FxAdj
     c1 -= 4 * mulhi_q64(bal(a.c1s), s4);
     c3 -= 4 * mulhi_q64(bal(a.c3s), s4);
   }
-  // u' = mulhi(q, r) 4, u = u' 2^-p (Q64)
-  const Bal ux = bal(4 * mulhi_q64(bal(qx), r)), uy = bal(4 * mulhi_q64(bal(qy), r)), uz = bal(4 * mulhi_q64(bal(qz), r));
-  int p = z + 1016 + er - ef;
-  p = (ux.h | ux.l | uy.h | uy.l | uz.h | uz.l) ? p : 0;
-  ok = ok && p >= 0 && em - p >= 64;
-  const int ps = p < 63 ? (p & 63) : 63;
-  auto fine = [&](Bal v) { return bal(((static_cast<int64_t>(v.h) << 32) + v.l) >> ps); };  // Q64 u
-  // moments over 36 (M0 halved) and 4 K
-  const int64_t A1 = Pi[1] + Pi[2] + Pi[3];
-  const int64_t m0h = 6 * m0 + A1 + ((Pi[4] + Pi[5] + Pi[6] + Pi[7] + Pi[8] + Pi[9]) >> 1);
-  const int64_t t0 = 2 * mulhi_q64(int64_t(0x5555555555555555ll), m0h);  // 36 M0 / 3
-  const Bal kxx = bal(2 * Pi[1] + Pi[4] + Pi[5] + Pi[6] + Pi[7] - t0);
-  const Bal kyy = bal(2 * Pi[2] + Pi[4] + Pi[5] + Pi[8] + Pi[9] - t0);
-  const Bal kzz = bal(2 * Pi[3] + Pi[6] + Pi[7] + Pi[8] + Pi[9] - t0);
-  const Bal kxy = bal(Pi[4] - Pi[5]), kxz = bal(Pi[6] - Pi[7]), kyz = bal(Pi[8] - Pi[9]);
-  const Bal nx = bal(2 * Di[1] + Di[4] + Di[5] + Di[6] + Di[7]);
-  const Bal ny = bal(2 * Di[2] + Di[4] - Di[5] + Di[8] + Di[9]);
-  const Bal nz = bal(2 * Di[3] + Di[6] - Di[7] + Di[8] - Di[9]);
-  // 4 X and M1.u (36), p bits finer
+  // u' = mulhi(q, r) 2^(2 + ku), u = u' 2^-p (Q64), its largest component in [2^61, 2^62)
+  const int64_t vx = 4 * mulhi_q64(bal(qx), r), vy = 4 * mulhi_q64(bal(qy), r), vz = 4 * mulhi_q64(bal(qz), r);
+  const uint64_t mu = fx_bits(vx) | fx_bits(vy) | fx_bits(vz);
+  const int ku = fx_norm(mu);
+  const Bal ux = bal(fx_shl(vx, ku)), uy = bal(fx_shl(vy, ku)), uz = bal(fx_shl(vz, ku));
+  const int p = (vx | vy | vz) != 0 ? z + ku + 1016 + er - ef : 0;
+  ok = ok && p >= 0;
+  // moments over 36 (M0 halved); 36 M0 = 3 t0 + rem, |rem| <= 6
+  const int64_t A1 = Pi[1] + Pi[2] + Pi[3], Ad = Pi[4] + Pi[5] + Pi[6] + Pi[7] + Pi[8] + Pi[9];
+  const int64_t m0h = 6 * m0 + A1 + (Ad >> 1);
+  constexpr int64_t third = 0x5555555555555555ll;
+  const int64_t t0 = 2 * mulhi_q64(third, m0h);
+  const int64_t rem = static_cast<int64_t>(12 * static_cast<uint64_t>(m0) + 2 * static_cast<uint64_t>(A1) +
+                                           static_cast<uint64_t>(Ad) - 3 * static_cast<uint64_t>(t0));
+  // 4 K 2^zk and 36 M1 2^zn
+  const int64_t lxx = 2 * Pi[1] + Pi[4] + Pi[5] + Pi[6] + Pi[7] - t0;
+  const int64_t lyy = 2 * Pi[2] + Pi[4] + Pi[5] + Pi[8] + Pi[9] - t0;
+  const int64_t lzz = 2 * Pi[3] + Pi[6] + Pi[7] + Pi[8] + Pi[9] - t0;
+  const int64_t lxy = Pi[4] - Pi[5], lxz = Pi[6] - Pi[7], lyz = Pi[8] - Pi[9];
+  const int zk = fx_norm(fx_bits(lxx) | fx_bits(lyy) | fx_bits(lzz) | fx_bits(lxy) | fx_bits(lxz) | fx_bits(lyz));
+  const int64_t r3 = mulhi_q64(third, fx_shl(rem, zk));
+  const Bal kxx = bal(fx_shl(lxx, zk) - r3), kyy = bal(fx_shl(lyy, zk) - r3), kzz = bal(fx_shl(lzz, zk) - r3);
+  const Bal kxy = bal(fx_shl(lxy, zk)), kxz = bal(fx_shl(lxz, zk)), kyz = bal(fx_shl(lyz, zk));
+  const int64_t hx = 2 * Di[1] + Di[4] + Di[5] + Di[6] + Di[7];
+  const int64_t hy0 = 2 * Di[2] + Di[4] - Di[5] + Di[8] + Di[9];
+  const int64_t hz = 2 * Di[3] + Di[6] - Di[7] + Di[8] - Di[9];
+  const int zn = fx_norm(fx_bits(hx) | fx_bits(hy0) | fx_bits(hz));
+  const Bal nx = bal(fx_shl(hx, zn)), ny = bal(fx_shl(hy0, zn)), nz = bal(fx_shl(hz, zn));
+  // 4 X (scale em - p - zk), M1.u (36; em - p - zn) and 4 u.X (em - 2p - zk)
   const int64_t Xx = mulhi_q64(kxx, ux) + mulhi_q64(kxy, uy) + mulhi_q64(kxz, uz);
   const int64_t Xy = mulhi_q64(kxy, ux) + mulhi_q64(kyy, uy) + mulhi_q64(kyz, uz);
   const int64_t Xz = mulhi_q64(kxz, ux) + mulhi_q64(kyz, uy) + mulhi_q64(kzz, uz);
   const int64_t nu = mulhi_q64(nx, ux) + mulhi_q64(ny, uy) + mulhi_q64(nz, uz);
-  const int64_t uX = mulhi_q64(fine(ux), bal(Xx)) + mulhi_q64(fine(uy), bal(Xy)) + mulhi_q64(fine(uz), bal(Xz));
-  // 4 Y, Y.u (p bits finer) and M1.g (36)
-  const Bal gx = bal(a.g[0]);
+  const int64_t uX = mulhi_q64(ux, bal(Xx)) + mulhi_q64(uy, bal(Xy)) + mulhi_q64(uz, bal(Xz));
+  // 4 Y (em - zk - zg), 4 Y.u (em - p - zk - zg) and M1.g (36; em - zn - zg)
+  const Bal gx = bal(a.gn[0]);
   int64_t Yx = mulhi_q64(kxx, gx), Yy = mulhi_q64(kxy, gx), Yz = mulhi_q64(kxz, gx), ng = mulhi_q64(nx, gx);
   if (!c.gx) {  // uniform
-    const Bal gy = bal(a.g[1]), gz = bal(a.g[2]);
+    const Bal gy = bal(a.gn[1]), gz = bal(a.gn[2]);
     Yx += mulhi_q64(kxy, gy) + mulhi_q64(kxz, gz);
     Yy += mulhi_q64(kyy, gy) + mulhi_q64(kyz, gz);
     Yz += mulhi_q64(kyz, gy) + mulhi_q64(kzz, gz);
     ng += mulhi_q64(ny, gy) + mulhi_q64(nz, gz);
   }
-  const Bal yx = bal(Yx), yy = bal(Yy), yz = bal(Yz);
-  const int64_t uY = mulhi_q64(ux, yx) + mulhi_q64(uy, yy) + mulhi_q64(uz, yz);
+  const int64_t uY = mulhi_q64(ux, bal(Yx)) + mulhi_q64(uy, bal(Yy)) + mulhi_q64(uz, bal(Yz));
+  // back at mu's scale: P, M1.g and u.X
+  const int sx = p + zk, sy = zk + a.zg;
   const Bal b1 = bal(c1), b3 = bal(c3), ap4 = bal(a.ap4);
-  const int64_t Px = mulhi_q64(b1, bal(Xx >> ps)) + mulhi_q64(ap4, yx) + mulhi_q64(b3, nx);
-  const int64_t Py = mulhi_q64(b1, bal(Xy >> ps)) + mulhi_q64(ap4, yy) + mulhi_q64(b3, ny);
-  const int64_t Pz = mulhi_q64(b1, bal(Xz >> ps)) + mulhi_q64(ap4, yz) + mulhi_q64(b3, nz);
-  int64_t Pg = mulhi_q64(gx, bal(Px));
+  const int64_t Px = mulhi_q64(b1, bal(fx_shr(Xx, sx))) + mulhi_q64(ap4, bal(fx_shr(Yx, sy))) + fx_shr(mulhi_q64(b3, nx), zn);
+  const int64_t Py = mulhi_q64(b1, bal(fx_shr(Xy, sx))) + mulhi_q64(ap4, bal(fx_shr(Yy, sy))) + fx_shr(mulhi_q64(b3, ny), zn);
+  const int64_t Pz = mulhi_q64(b1, bal(fx_shr(Xz, sx))) + mulhi_q64(ap4, bal(fx_shr(Yz, sy))) + fx_shr(mulhi_q64(b3, nz), zn);
+  int64_t Pg = mulhi_q64(bal(a.g[0]), bal(Px));
   if (!c.gx) Pg += mulhi_q64(bal(a.g[1]), bal(Py)) + mulhi_q64(bal(a.g[2]), bal(Pz));
-  o.A = mulhi_q64(bal(a.l18), bal(m0h)) - (mulhi_q64(b1, bal(uX >> ps)) >> 1) + mulhi_q64(bal(a.c3s), bal(ng));
+  o.A = mulhi_q64(bal(a.l18), bal(m0h)) - (mulhi_q64(b1, bal(fx_shr(uX, sx + p))) >> 1) +
+        mulhi_q64(bal(a.c3s), bal(fx_shr(ng, zn + a.zg)));
   if (DRAG) {
     o.A += 2 * mulhi_q64(kd, bal(Pg));
     o.Bx = 2 * mulhi_q64(kd, bal(2 * Px));
@@ -927,8 +964,12 @@ __host__ __device__ __forceinline__ bool fx_adjoint(const FxColl& c, const FxAdj
   // -(a-/12 + kd/2 c3) M1.u - (a+/4 + kd/2 c1) u.X - kd/2 a+/4 u.Y
   const int64_t h3 = DRAG ? 2 * mulhi_q64(kd, b3) : c3 >> 1, h1 = DRAG ? 2 * mulhi_q64(kd, b1) : c1 >> 1;
   const int64_t hy = DRAG ? 2 * mulhi_q64(kd, ap4) : a.ap4 >> 1;
-  o.gs = -(mulhi_q64(bal(a.c3s + h3), bal(nu)) + mulhi_q64(bal(a.ap4 + h1), bal(uX)) + mulhi_q64(bal(hy), bal(uY)));
-  o.eg = em - p;
+  // (the first factor below 1/12, the last below 1/8: times 4 and 2)
+  const int en = em - p - zn, ex = em - p - sx, ey = em - p - sy;
+  ok = ok && en >= 70 && ex >= 70 && ey >= 70;
+  o.gs = -(fx_to_double_cvt(mulhi_q64(bal(4 * (a.c3s + h3)), bal(nu)), en - 2) +
+           fx_to_double_cvt(mulhi_q64(bal(a.ap4 + h1), bal(uX)), ex) +
+           fx_to_double_cvt(mulhi_q64(bal(2 * hy), bal(uY)), ey - 1));
   return ok;
 }
 
