@@ -40,12 +40,7 @@ FALLBACK_HBM_GBS = 6800.0
 # int64 -> double conversions of the 19 outputs (ncu, sm__inst_executed_pipe
 # _fp64.sum over the nodes of one launch).  Moments, class terms and pair update
 # run in fixed point on the integer and FMA pipes, for every omega_plus.
-COLL_DP_INSTR_GENERAL = 19
-COLL_DP_INSTR_UNIT_OMEGA = 19
-# DRAM bytes (dram__bytes_read.sum + dram__bytes_write.sum) of one launch of a
-# kernel on the 10,896,954-node bed, from an ncu capture of the current kernel
-# version, with the profile that holds it; kernels not listed print null.
-TRAFFIC_PROFILED = {}
+COLL_DP_INSTR = 19
 
 WORKLOAD = dict(name="packed_bed_256_rsa_r12", X=256, Y=256, Z=256, radius=12.0, seed=1, rejections=20000,
                 periodic=(1, 0, 0), g=(1e-6, 0.0, 0.0), omega_plus=1.0, magic=3.0 / 16.0)
@@ -780,9 +775,8 @@ def suite_bed40(args, lbm, torch):
             out["variants"][f"{name}_{prec}"] = {"GFLUPs": g, "B_l": bl, "frac_hbm": g * bl / hbm}
             del sv
             torch.cuda.empty_cache()
-    dp = COLL_DP_INSTR_UNIT_OMEGA if w["omega_plus"] == 1.0 else COLL_DP_INSTR_GENERAL
     fp = fp64_pipe_peak(lbm, torch, torch.device("cuda", 0), torch.cuda.current_stream())
-    out["aa_r_f64_fp64_pipe_frac"] = out["variants"]["aa_r_f64"]["GFLUPs"] * dp / fp["G_dfma_per_s"]
+    out["aa_r_f64_fp64_pipe_frac"] = out["variants"]["aa_r_f64"]["GFLUPs"] * COLL_DP_INSTR / fp["G_dfma_per_s"]
     out["hbm_peak_GBs"] = hbm
     return out
 
@@ -972,10 +966,8 @@ def main():
     dom_name = f"aa_{'odd_ria' if odd_dom else 'even'}_{hp}"
     dom_bl = loop_balance("aa_odd_r" if odd_dom else "aa_even", p, r)
     achieved_gbs = dom_bl * N / (dom_ms / 1e3) / 1e9
-    prof = TRAFFIC_PROFILED.get((dom_name, N)) if args.box is None else None
     roofline = {"kernel": dom_name, "bound": "hbm", "achieved": achieved_gbs, "peak": hbm, "unit": "GB/s",
-                "frac": achieved_gbs / hbm, "traffic": prof[0] if prof else None,
-                "traffic_source": prof[1] if prof else None,
+                "frac": achieved_gbs / hbm, "traffic": None, "traffic_source": None,
                 "peak_kind": f"{hbm_kind} copy bandwidth (STREAM-style), burst",
                 "bytes_per_node": dom_bl, "units_per_launch": N,
                 "kernel_ms": {"even": even_ms, "odd": odd_ms},
@@ -984,11 +976,10 @@ def main():
         # the native FP64 step's second roof: its FP64-pipe work against the
         # pipe's measured throughput (DFMA chains, CUDA events, clock sampled)
         fp = fp64_pipe_peak(lbm, torch, dev, stream)
-        dp_instr = COLL_DP_INSTR_UNIT_OMEGA if w["omega_plus"] == 1.0 else COLL_DP_INSTR_GENERAL
-        dp_rate = dp_instr * N / (dom_ms / 1e3) / 1e9
+        dp_rate = COLL_DP_INSTR * N / (dom_ms / 1e3) / 1e9
         roofline["fp64_pipe"] = {"bound": "alu", "achieved": dp_rate, "peak": fp["G_dfma_per_s"],
                                  "unit": "G FP64-instr/s", "frac": dp_rate / fp["G_dfma_per_s"],
-                                 "dp_instr_per_node": dp_instr, "peak_measured": fp}
+                                 "dp_instr_per_node": COLL_DP_INSTR, "peak_measured": fp}
 
     # ---- the same pair with the double-float collision (FP64 grids, same FP64 parity bar) -------------
     companion = None

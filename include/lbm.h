@@ -310,11 +310,14 @@ LBM_API int lbm_export_tables(const lbm_lattice* lat, int32_t* node_xyz, int32_t
  * comparison on the host.  With r a run, h its first node and a = run_adj[i][r]:
  *  kind 0 (AA odd step):  slot(i, r) = inv(i) Npad + a  (a >= 0),  i Npad + h (wall)
  *  kind 1 (OS-NT step):   slot(i, r) = i Npad + a       (a >= 0),  inv(i) Npad + h (wall)
- * out: host int32 [R][18] (run-major, as the device holds them without the
- * padding words), entry i - 1 of row r for i = 1..18.  *available is set to 1
- * when the lattice has the tables, else 0 (pressure markers, or a grid of
- * 2^31 slots or more: the steps then decode run_adj) and out is left alone.
- * out may be NULL to ask for availability only. */
+ * out: host int32 [R][18] (run-major, as the device holds them without its two
+ * trailing words), entry i - 1 of row r for i = 1..18.  *available is set to 1 when
+ * the lattice has the tables and no pressure markers, else 0 and out is left alone.
+ * A grid of 2^31 slots or more has no tables.  A lattice with pressure markers has
+ * them when its runs number at most half its nodes; the trailing words then hold the
+ * directions that meet an inlet and an outlet, and the tables are not exported.
+ * Without tables the steps decode run_adj.  out may be NULL to ask for availability
+ * only. */
 LBM_API int lbm_export_run_slots(lbm_lattice* lat, int kind, int32_t* out, int* available);
 
 /* Adjacency entries of chosen nodes only (lattices too large to export in
@@ -330,9 +333,9 @@ LBM_API int lbm_check_finite(const double* values, int64_t count, void* stream);
  * without a GPU.  The LBM_F64 step kernels form a node's moments -- the
  * density deviation sum_i d_i, the momentum sum_i c_i d_i, and the pair sums
  * and differences d_a +- d_inv(a) that the TRT collision (Sect. 2) splits
- * into even and odd parts -- as exact fixed-point sums on the integer pipe,
- * each rounded once to the nearest double; this runs the same routine on the
- * host.  d: host double [n][19] (node-major, direction order as above);
+ * into even and odd parts -- as exact fixed-point sums on the integer pipe;
+ * this runs the same routine on the host and rounds each sum once to the nearest
+ * double.  d: host double [n][19] (node-major, direction order as above);
  * out: host double [n][22]: drho, jx, jy, jz, sa_1..sa_9, da_1..da_9, pair k
  * holding directions 2k-1 and 2k.  A PDF more than 5 binades below the node's
  * largest loses the bits below 2^-57 of that largest (truncated).  A node
@@ -348,14 +351,15 @@ LBM_API int lbm_exact_moments_host(const double* d, int64_t n, double* out);
  * o = qm (d_a - d_b) + c_a.O, qm = (1 - l-)/2, qp = (1 - l+)/2.  The LBM_F64
  * step kernels evaluate this in 64-bit fixed point at a scale 2^(es - 1080)
  * tied to the node's largest PDF, with one rounding to double per output,
- * whenever the node's values lie in that scale's range; this runs the same
- * routine on the host.  d: host double [n][19] (node-major); terms: host
+ * whenever the node's values lie in that scale's range; this runs the same pair
+ * routine on the host, from terms given as doubles (the kernels form them in fixed
+ * point as well: lbm_fx_collide_host is the image of the whole).  d: host double [n][19] (node-major); terms: host
  * double [n][10]: ux, uy, uz, K0, Tx, Ty, Tz, Ox, Oy, Oz; flags: bit 0 for
  * the l+ = 1 form (qp must be 0), bit 1 to take the general conversions
  * everywhere (the kernels take shorter ones for positive values in a common
  * range; the results are the same bits).  out: host double [n][19]: out[0] = es, out[1..18]
  * the post-collision pair values; ok: host int [n], 0 where the node is
- * outside the range (out is then 0; the kernels take the FP64 update there).
+ * outside the range (out is then 0).
  * Each value is within 8 units of 2^(es - 1080) of the exact rational result,
  * before its rounding to nearest.  LBM_ERR_ARG for NULL pointers, n < 0, or
  * |qm| or |qp| >= 1/2. */

@@ -267,7 +267,7 @@ __global__ void __launch_bounds__(kBlock, MinCtasAdj<PREC, TAB>::value) k_adjoin
     jy = fx_to_double(Jy, ef);
     jz = fx_to_double(Jz, ef);
   } else {
-    moments<R, false>(d, sa, da, drho, jx, jy, jz);
+    moments(d, sa, da, drho, jx, jy, jz);
   }
   const R rho = c.rho_s + drho;
   const R irho = recip(rho);

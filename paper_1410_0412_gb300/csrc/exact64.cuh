@@ -20,9 +20,9 @@
 //    to 0.5 * x for every x whose half is a normal number, Inf or NaN.
 //
 // On the 256^3 bed (10.9 M nodes) the FP64 AA-R step pair went from 1.61 ms,
-// with the class terms in FP64 (31 FP64 instructions a node), to 1.23 ms; the
-// even step moves its bytes at 0.96 of the measured copy rate (ncu: DRAM 78 %,
-// integer pipe 66 %, FP64 pipe 71 %).
+// with the class terms in FP64 (31 FP64 instructions a node), to 1.23 ms.  The even
+// step of a 160^3 bed (3.03 M nodes, ncu): DRAM 78 %, integer pipe 66 %, FP64 pipe
+// 68 %.
 //
 // All functions are __host__ __device__ so that a host test can check the
 // moments bit for bit against exact rational arithmetic.
@@ -118,26 +118,12 @@ __host__ __device__ __forceinline__ double fx_to_double(int64_t v, int emax) {
   return dfrom(((static_cast<uint64_t>(emax + 5 - lz) << 52) + m) | s);
 }
 
-// 32-bit funnel shifts (the PTX shf instructions) with a portable host image.
+// 32-bit funnel shift (the PTX shf instruction) with a portable host image.
 __host__ __device__ __forceinline__ uint32_t shf_l(uint32_t lo, uint32_t hi, unsigned n) {  // n in [0, 31]
 #ifdef __CUDA_ARCH__
   return __funnelshift_l(lo, hi, n);
 #else
   return n ? (hi << n) | (lo >> (32 - n)) : hi;
-#endif
-}
-__host__ __device__ __forceinline__ uint32_t shf_r(uint32_t lo, uint32_t hi, unsigned n) {  // n in [0, 31]
-#ifdef __CUDA_ARCH__
-  return __funnelshift_r(lo, hi, n);
-#else
-  return n ? (lo >> n) | (hi << (32 - n)) : lo;
-#endif
-}
-__host__ __device__ __forceinline__ int clz32(uint32_t a) {
-#ifdef __CUDA_ARCH__
-  return __clz(static_cast<int>(a));
-#else
-  return a ? __builtin_clz(a) : 32;
 #endif
 }
 
@@ -325,7 +311,8 @@ __host__ __device__ __forceinline__ bool fx_pos_near(const double (&d)[19], int&
   return (mn >> 20) >= kFxMinExp && emax < kFxMaxExp && emax - (mn >> 20) <= 5;
 }
 
-// The moments as doubles: pair sums sa_k (only when NEED_SA) and differences
+// The moments as doubles (lbm_exact_moments_host; the kernels keep the integers):
+// pair sums sa_k (only when NEED_SA) and differences
 // da_k, the density deviation drho = sum d_i and the momentum j = sum c_i d_i,
 // each the double nearest to the exact fixed-point sum.  A node whose scale
 // reaches kFxMaxExp (an Inf, a NaN or |d_i| >= 2^1017) gets drho = NaN.

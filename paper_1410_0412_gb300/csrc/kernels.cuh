@@ -529,25 +529,21 @@ __device__ __forceinline__ void coll_pair(R (&d)[kQ], const R sa, const R da, co
 }
 
 // Pair sums sa_k = d_a + d_b and differences da_k = d_a - d_b, the density
-// deviation and the momentum.  FP64 takes them exactly on the integer pipe
-// (exact64.cuh), with sa converted only when the caller needs it (l+ != 1).
-template <class R, bool NEED_SA, bool IEEE = false>
+// deviation and the momentum.  (The FP64 collision forms them in fixed point,
+// collide_f64.)
+template <class R>
 __device__ __forceinline__ void moments(const R (&d)[kQ], R (&sa)[10], R (&da)[10], R& drho, R& jx, R& jy, R& jz) {
-  if constexpr (std::is_same<R, double>::value && !IEEE) {
-    exact_moments<NEED_SA>(d, sa, da, drho, jx, jy, jz);
-  } else {
 #pragma unroll
-    for (int k = 1; k <= 9; ++k) {
-      sa[k] = d[2 * k - 1] + d[2 * k];
-      da[k] = d[2 * k - 1] - d[2 * k];
-    }
-    drho = d[0];
-#pragma unroll
-    for (int k = 1; k <= 9; ++k) drho += sa[k];
-    jx = da[1] + da[4] + da[5] + da[6] + da[7];
-    jy = da[2] + da[4] - da[5] + da[8] + da[9];
-    jz = da[3] + da[6] - da[7] + da[8] - da[9];
+  for (int k = 1; k <= 9; ++k) {
+    sa[k] = d[2 * k - 1] + d[2 * k];
+    da[k] = d[2 * k - 1] - d[2 * k];
   }
+  drho = d[0];
+#pragma unroll
+  for (int k = 1; k <= 9; ++k) drho += sa[k];
+  jx = da[1] + da[4] + da[5] + da[6] + da[7];
+  jy = da[2] + da[4] - da[5] + da[8] + da[9];
+  jz = da[3] + da[6] - da[7] + da[8] - da[9];
 }
 
 // Halving: an exponent decrement for FP64 (exact64.cuh), a multiply otherwise.
@@ -714,7 +710,7 @@ __device__ __forceinline__ void collide(R (&d)[kQ], const CollConst<R>& c, const
     return;
   }
   R sa[10], da[10], drho, jx, jy, jz;
-  moments<R, !LP1>(d, sa, da, drho, jx, jy, jz);
+  moments(d, sa, da, drho, jx, jy, jz);
   if (SC) {  // storage units -> physical units for the moments
     drho = drho * c.inv_s;
     jx = jx * c.inv_s;
@@ -918,7 +914,7 @@ __global__ void __launch_bounds__(kBlock) k_aa_even_h2(DevTables t, KParams kp, 
 template <bool FORCE, bool DRAG, bool LP1>
 __device__ __forceinline__ void collide_odd_df(const double (&g64)[kQ], const CollConst<df>& c, df sn, df (&d)[kQ]) {
   double sa64[10], da64[10], drho64, jx64, jy64, jz64;
-  moments<double, !LP1, true>(g64, sa64, da64, drho64, jx64, jy64, jz64);
+  moments(g64, sa64, da64, drho64, jx64, jy64, jz64);
   df sa[10], da[10];
 #pragma unroll
   for (int k = 1; k <= 9; ++k) {

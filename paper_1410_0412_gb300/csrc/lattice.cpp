@@ -460,29 +460,26 @@ int partition_ghosts(const lbm_lattice* L, int P, int64_t* ghosts) {
 // lexicographic order of the (wrapped) coordinates, x fastest.
 int derive_et_tables(lbm_lattice* L);
 
-// The AA odd step's slots per run.  With RIA, node n = head + off of run r
-// reads f_i from slot (inv i, run_adj[i][r] + off) when the head pulls from a
-// fluid node, and from its own slot (i, head + off) through a bounce-back
-// marker; as a flat index of the [19][Npad] grid this is
-// run_slot(i, r) + off in both cases, with
+// Run slot tables: the slots of each run's first node, resolved once.  With RIA,
+// node n = head + off of run r reads f_i from slot (inv i, run_adj[i][r] + off) when
+// the head pulls from a fluid node, and from its own slot (i, head + off) through a
+// marker; as a flat index of the [19][Npad] grid this is run_slot(i, r) + off in both
+// cases, with
 //   run_slot[i][r] = inv(i) Npad + run_adj[i][r]   (fluid source)
-//                  = i Npad + run_start[r]          (bounce-back).
-// The step also writes P_i to the slot f_inv(i) came from, so the same entries
-// give its stores.  The OS-NT step pulls post-collision P_i from slot
+//                  = i Npad + run_start[r]          (marker).
+// The AA odd step also writes P_i to the slot f_inv(i) came from, so the same
+// entries give its stores.  The OS-NT step pulls post-collision P_i from slot
 // (i, run_adj[i][r] + off) of the source grid, or P_inv(i) from the node's own
 // slot (inv i, head + off) through a marker: run_slot_osnt[i][r] =
-// i Npad + run_adj[i][r] or inv(i) Npad + run_start[r].  This pre-resolves the
-// table (the same 4 bytes per run and direction as run_adj) so the kernel
-// spends one add per access.  Lattices
-// with pressure markers (whose anti-bounce-back needs the marker kind) or a
-// grid of 2^31 or more slots do not qualify: run_slot_state = 0.
-// Run slot tables, for grids below 2^31 slots.  Row r holds the AA odd step's
-// (run_slot) and the OS-NT step's (run_slot_osnt) slots of run r's first node;
-// words 18 and 19 hold the directions whose pull meets an inlet or an outlet
-// (bit i - 1).  A lattice with pressure faces has them when its runs number at
-// most half its nodes: 160 bytes a run are then no more than the adjacency list,
-// while at one run per node (a Hilbert order) the rows read as many bytes as the
-// runs' adjacency entries and would double the tables of a large lattice.
+// i Npad + run_adj[i][r] or inv(i) Npad + run_start[r].  The kernel spends one add
+// per access.
+//
+// Rows are run-major (80 bytes a run and table, against 72 of run_adj); words 18 and
+// 19 hold the directions whose pull meets an inlet or an outlet (bit i - 1).  A grid
+// of 2^31 slots or more has no tables.  A lattice with pressure faces has them when
+// its runs number at most half its nodes: 160 bytes a run are then no more than the
+// adjacency list, while at one run per node (a Hilbert order) the rows read as many
+// bytes as the runs' adjacency entries and would double the tables of a large lattice.
 int derive_run_slots(lbm_lattice* L) {
   if (L->run_slot_state >= 0) return LBM_OK;
   if (int64_t(19) * L->Npad >= (int64_t(1) << 31)) {
