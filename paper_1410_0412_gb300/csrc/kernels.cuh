@@ -668,9 +668,10 @@ __device__ __forceinline__ void collide_m(R (&d)[kQ], const CollConst<R>& c, con
 // range (fx_class_int), otherwise in FP64 from the moments rounded to double.  NaN
 // or Inf PDFs take the FP64 branch and come out NaN.  With l+ = 1 each node decides
 // for itself, and its bits follow from its own PDFs alone (both conversions give the
-// same integers).  At general rates a warp with any node out of range takes FP64
-// whole: the nine pair sums leave no registers for two live branches (a per-node
-// choice cost 2.6 % there).
+// same integers).  The warp-uniform branch before that decision is for warps that are
+// in range whole, nearly all: as one divergent branch the 46 k-node box took 5.9 us a
+// step instead of 5.7.  At general rates a warp with any node out of range takes
+// FP64 whole: the nine pair sums leave no registers for the second branch (2.6 %).
 template <bool FORCE, bool DRAG, bool LP1>
 __device__ __forceinline__ void collide_f64(double (&d)[kQ], const CollConst<double>& c, const double s) {
   int64_t Sk[10], D[10], S, Jx, Jy, Jz, f0;
@@ -687,7 +688,9 @@ __device__ __forceinline__ void collide_f64(double (&d)[kQ], const CollConst<dou
   const int kx = fx_kx<LP1>(c.fx);
   FxClass q;
   const bool ok = fx_class_int<FORCE, DRAG, LP1>(c.fx, emax, kx, S, Jx, Jy, Jz, s, q) && room;
-  if (LP1 ? ok : __all_sync(__activemask(), ok)) {
+  if (__all_sync(__activemask(), ok)) {
+    fx_update<LP1>(c.fx, q, emax, kx, D, Sk, f0, d);
+  } else if (LP1 && ok) {
     fx_update<LP1>(c.fx, q, emax, kx, D, Sk, f0, d);
   } else {
     const double drho = emax < kFxMaxExp ? fx_to_double(S, emax) : dfrom(0x7ff8000000000000ull);
