@@ -857,11 +857,15 @@ class Solver:
 
     def step(self, n=1, stream=None):
         if self.form == "osnt":
-            n = len(range(n))
-            lbm_run_osnt(self.lat, self.prec, self.params, self.grids[0], self.grids[1], n, self.s, self.ria, stream)
-            if n % 2:
-                self.grids.reverse()
-            self.t += n
+            left = range(n)
+            while len(left):
+                k = min(len(left), 1 << 30)  # the library counts steps in 32 bits
+                lbm_run_osnt(self.lat, self.prec, self.params, self.grids[0], self.grids[1], k, self.s, self.ria,
+                             stream)
+                if k % 2:
+                    self.grids.reverse()
+                self.t += k
+                left = left[k:]
         elif self.form == "et":
             lbm_run_et(self.lat, self.prec, self.params, self.grids[0], self.t % 2, n, self.s, self.ria, stream)
             self.t += n
