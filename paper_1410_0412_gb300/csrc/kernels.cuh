@@ -1585,7 +1585,11 @@ template <int PREC, int FORM> inline int table_kind(const lbm_lattice* L, int ri
 // or more, FP16S AA-R by slots turns at about 96 MB (blocked rows, a step: 19.9 ->
 // 18.4 at 74, 27.3 -> 27.6 at 112, 43.6 -> 44.5 at 161), and so does the AA step by
 // the list's entries (Hilbert beds and foams: 29.5 -> 28.5 at 74, 35.7 -> 36.4 at 99,
-// 58.8 -> 59.2 at 161).  The double-float steps are plain.
+// 58.8 -> 59.2 at 161).  A partition's chunks, which step side by side between an
+// exchange and a join, have no step before them to overlap and take the plain
+// launches here (bed in 16 chunks, FP32 AA-R, GFLUP/s dependent -> plain: rows 32.7 ->
+// 33.3, Hilbert 27.1 -> 27.9, renumbered 31.9 -> 33.2).  The double-float steps are
+// plain.
 template <int PREC, int FORM>
 constexpr int kDependent = PREC == LBM_F64_DF                                                                  ? 0
                            : PREC == LBM_F64 || (PREC == LBM_F32 && FORM != kFormAa) || FORM == kFormOsnt ? 2
@@ -1593,6 +1597,7 @@ constexpr int kDependent = PREC == LBM_F64_DF                                   
 template <int PREC, int FORM> inline bool dependent(const lbm_lattice* L, int ria) {
   const bool faces = PREC == LBM_F32 && FORM == kFormEt && ria && L->dev.pressure && !scattered(L);
   if (kDependent<PREC, FORM> != 1 && !faces) return kDependent<PREC, FORM> == 2;
+  if (L->partition_local) return false;
   const bool apart = PREC == LBM_F16S && FORM == kFormAa && 4 * L->R > L->N && scattered(L) == !ria;
   return step_bytes<PREC>(L) <= (apart ? int64_t(96) << 20 : kSmallStep);
 }
