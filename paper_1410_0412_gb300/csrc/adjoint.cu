@@ -226,7 +226,7 @@ __global__ void __launch_bounds__(kBlock, MinCtasAdj<PREC, TAB>::value) k_adjoin
     // FP64: the whole step in fixed point (fx_adjoint) where every node of the
     // warp is in range.  It was bound by the FP64 pipe (about 160 instructions
     // a node, 80 % busy, DRAM 28 %): 0.175 ms for 0.77 M nodes with drag; now
-    // 0.102 ms.
+    // 0.104 ms.
     int64_t S, Jx, Jy, Jz, Sk[10], Dk[10];
     const int ef = fx_moments<false>(d, Sk, Dk, S, Jx, Jy, Jz, 0, nullptr, cc.fx.emin);
     uint64_t b[kQ];

@@ -21,8 +21,8 @@
 //
 // On the 256^3 bed (10.9 M nodes) the FP64 AA-R step pair went from 1.61 ms,
 // with the class terms in FP64 (31 FP64 instructions a node), to 1.23 ms.  The even
-// step of a 160^3 bed (3.03 M nodes, ncu): DRAM 78 %, integer pipe 66 %, FP64 pipe
-// 68 %.
+// step of a 160^3 bed (3.03 M nodes, ncu): DRAM 77 %, integer pipe 66 %, FP64 pipe
+// 67 %.
 //
 // All functions are __host__ __device__ so that a host test can check the
 // moments bit for bit against exact rational arithmetic.
