@@ -71,3 +71,17 @@ def test_constant_field_has_no_gradient():
     mu = np.full((6, 19), 1.0) * np.array([[1.0], [-3.5], [1e-9], [7e5], [1 / 3], [0.0]])
     _, grad, ok = lbm.lbm_fx_adjoint_host(_forward(6, 4, True, 0.01), mu, p, np.full(6, 0.5, np.float32))
     assert ok.all() and (grad == 0).all()
+
+
+@pytest.mark.parametrize("u", [1e-30, 1e-90, 1e-140, 1e-200, 1e-280])
+def test_the_slowest_flows_stay_in_the_range(u):
+    # a front that runs into a fluid at rest: terms quadratic in u underflow, the linear one still counts
+    p = lbm.Params(omega_plus=1.0, magic=3 / 16, g=(0.0, 0.0, 0.0), shifted=True)
+    d = np.zeros((3, 19))
+    d[:, 1], d[:, 4], d[:, 7] = u, -0.7 * u, 0.2 * u
+    mu = np.random.default_rng(3).standard_normal((3, 19))
+    _, grad, ok = lbm.lbm_fx_adjoint_host(d, mu, p, np.full(3, 0.5, np.float32))
+    assert ok.all()
+    for k in range(3):
+        _, ex, rho, um = _exact(d[k], mu[k], p, 0.5)
+        assert abs(Fraction(float(grad[k])) - ex) <= rho * _scale(mu[k], um, p.g) + abs(ex) / 2 ** 51
