@@ -160,13 +160,13 @@ __device__ __forceinline__ void adj_moments(const R (&mu)[kQ], const AdjConst<R>
 // lam_next / lam: adjoint of the canonical states F_{n+1} / F_n, layout [19][Npad].
 // LP1: l+ = 1 (FP64-storage paths), where (1 - l+)/2 = 1 - l+ = 0.
 // Resident CTAs per SM, by table, from sweeps of checkpointed gradients (ms).
-// Run slots, FP64 at 3 / 4 / 5 / 6: 13.43 / 12.80 / 13.11 / 14.08 (60 steps on
-// 0.77 M nodes; above 4 it spills); FP32 at 6 / 7 / 8 / 9: 19.67 / 19.61 / 18.99
-// / 18.98 (100 steps on the 128^3 box).  Adjacency list (60 steps on the box):
-// FP32 at 6 / 7 / 8: 17.0 / 15.8 / 17.0, FP64 at 4 / 5 / 6: 37.5 / 36.1 / 40.5.
-// Run entries (60 steps on a 128^3 foam): FP32 at 5 / 6 / 7 / 8: 12.0 / 11.6 /
-// 13.4 / 13.6, FP64 at 4 / 5: 34.6 / 39.6.  Double-float at 4 / 5 / 6: 1713 / 1589
-// / 1527 (2000 steps on the box, adjacency list).
+// Run slots, FP64 at 3 / 4 / 5: 13.67 / 12.68 / 13.34 (60 steps on 0.77 M nodes;
+// spills above 4); FP32 at 6 / 7 / 8 / 9: 19.67 / 19.61 / 18.99 / 18.98 (100 steps on
+// the 128^3 box).  Adjacency list: FP32 at 6 / 7 / 8: 17.0 / 15.8 / 17.0 (60 steps on
+// the box), FP64 at 4 / 5 / 6: 11.60 / 11.20 / 12.65 (40 steps on a 96^3 box).  Run
+// entries (60 steps on a 128^3 foam): FP32 at 5 / 6 / 7 / 8: 12.0 / 11.6 / 13.4 / 13.6,
+// FP64 at 4 / 5: 34.6 / 39.6.  Double-float at 4 / 5 / 6: 1713 / 1589 / 1527 (2000
+// steps on the box, adjacency list).
 template <int PREC, int TAB> struct MinCtasAdj {
   static constexpr int value = PREC == LBM_F64_DF ? 6
                                : PREC == LBM_F64  ? (TAB == kAdjAny ? 5 : 4)
