@@ -353,13 +353,13 @@ LBM_API int lbm_exact_moments_host(const double* d, int64_t n, double* out);
  * tied to the node's largest PDF, with one rounding to double per output,
  * whenever the node's values lie in that scale's range; this runs the same pair
  * routine on the host, from terms given as doubles (the kernels form them in fixed
- * point as well: lbm_fx_collide_host is the image of the whole).  d: host double [n][19] (node-major); terms: host
- * double [n][10]: ux, uy, uz, K0, Tx, Ty, Tz, Ox, Oy, Oz; flags: bit 0 for
- * the l+ = 1 form (qp must be 0), bit 1 to take the general conversions
- * everywhere (the kernels take shorter ones for positive values in a common
- * range; the results are the same bits).  out: host double [n][19]: out[0] = es, out[1..18]
- * the post-collision pair values; ok: host int [n], 0 where the node is
- * outside the range (out is then 0).
+ * point as well: lbm_fx_collide_host is the image of the whole).  d: host double
+ * [n][19] (node-major); terms: host double [n][10]: ux, uy, uz, K0, Tx, Ty, Tz, Ox,
+ * Oy, Oz; flags: bit 0 for the l+ = 1 form (qp must be 0), bit 1 to take the general
+ * conversions everywhere (the kernels take shorter ones for positive values in a
+ * common range; the results are the same bits).  out: host double [n][19]: out[0] =
+ * es, out[1..18] the post-collision pair values; ok: host int [n], 0 where the node
+ * is outside the range or |qm| or |qp| within 2^-33 of 1/2 (out is then 0).
  * Each value is within 8 units of 2^(es - 1080) of the exact rational result,
  * before its rounding to nearest.  LBM_ERR_ARG for NULL pointers, n < 0, or
  * |qm| or |qp| >= 1/2. */
